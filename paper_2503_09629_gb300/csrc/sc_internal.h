@@ -228,14 +228,12 @@ cudaError_t launch_z4c_derivs(const double* Y, double* scratch, long fs, int sy,
 // before any graph capture).
 cudaError_t z4c_init_launch_config();
 // order: finite-difference order of the derivatives, 4 or 8 (Kreiss-Oliger stays r = 4).
-// op_class: the PlainK build of the kernel (same results; see PlainK).
 cudaError_t launch_z4c_dxy(const double* Y, double* scratch, long fs, int sy, const RowSeg* segs, int nsegs,
-                           cudaStream_t s, int order = 4, bool op_class = false);
+                           cudaStream_t s, int order = 4);
 // max_cols: the largest nx * ny of the tiles (work is dealt out per tile in
 // chunks sized by it); cudaErrorInvalidValue if below 1.
 cudaError_t launch_z4c_derivs_split(const double* Y, double* scratch, long fs, int sy, int sz,
-                                    const Tile* tiles, int ntiles, cudaStream_t s, int order, int max_cols,
-                                    bool op_class = false);
+                                    const Tile* tiles, int ntiles, cudaStream_t s, int order, int max_cols);
 // bps: warps per scheduler of the stage kernel's build (the register budget of
 // bps 128-thread blocks per SM), 2 or 3 (a tuning choice); threads: block
 // size, 128 (tiles of at most 128 cells) or 64 (tiles of at most 64 cells, 2 bps

@@ -19,7 +19,7 @@
 // shared pair sums/differences in the stencils, fused multiply-adds, one
 // division for 1/det(gt) and one for 1/W, and the quadratic Christoffel
 // terms of the Ricci tensor contracted through one raised-index array.
-#include "sc_internal.h"
+#include "sc_fixed.cuh"
 
 namespace sc {
 namespace {
@@ -114,42 +114,33 @@ __global__ void __launch_bounds__(kThreads) z4c_derivs_kernel(const double* __re
 // field of Hessian slot s (W, gt x6, alpha, beta x3): slots 0..6 -> fields 0..6, 7..10 -> 18..21
 __device__ __forceinline__ int d2_field(int s) { return s <= 6 ? s : s + 11; }
 
-// The stencil sums are arranged for the FP64 issue rates of this GPU: a
-// fused multiply-add whose multiplier is not +-1 and whose addend is not zero
-// issues about 1.2x as fast as an addition (or a unit-multiplier FMA, or a
-// multiplication).  So every weighted value enters through a general FMA, and
-// only values of unit weight are added; pair sums v_m + v_-m are formed only
-// where two sums share them.  lo[m] = v_-(m+1), hi[m] = v_(m+1).
-
-// Centred first derivative as the integer-weight sum: 4th order
-// 8 (v_1 - v_-1) - (v_2 - v_-2) (= 12 h u'), one addition and two FMAs;
-// 8th order 672 d1 - 168 d2 + 32 d3 - 3 d4 (= 840 h u'), dm = v_m - v_-m.
-template <int ORD, class KT>
-__device__ __forceinline__ double dfirst(const double* lo, const double* hi, const KT& K) {
-  if (ORD == 4) return fma(8.0, hi[0], fma(-8.0, lo[0], fsub(lo[1], hi[1], K)));
-  return fma(672.0, hi[0],
-             fma(-672.0, lo[0],
-                 fma(-168.0, hi[1],
-                     fma(168.0, lo[1], fma(32.0, hi[2], fma(-32.0, lo[2], fmul(3.0, fsub(lo[3], hi[3], K), K)))))));
-}
-// The same first derivative from the differences dm = v_m - v_-m, m = 1..R.
-template <int ORD, class KT>
-__device__ __forceinline__ double dfirst_d(const double* d, const KT& K) {
-  if (ORD == 4) return fma(8.0, d[0], -d[1]);
-  return fma(672.0, d[0], fma(-168.0, d[1], fma(32.0, d[2], fmul(-3.0, d[3], K))));
-}
-// Centred second derivative from the pair sums pm = v_m + v_-m, as the
-// integer-weight sum: 4th order 16 p1 - p2 - 30 u0 (= 12 h^2 u''), 8th order
-// 8064 p1 - 1008 p2 + 128 p3 - 9 p4 - 14350 u0 (= 5040 h^2 u'').
-template <int ORD, class KT>
-__device__ __forceinline__ double dsecond(const double* p, double u0, const KT& K) {
-  if (ORD == 4) return fma(16.0, p[0], fma(-30.0, u0, -p[1]));
-  return fma(-14350.0, u0, fma(8064.0, p[0], fma(-1008.0, p[1], fma(128.0, p[2], fmul(-9.0, p[3], K)))));
+// Centred first derivative as the integer-weight sum, lo[m - 1] = v_-m, hi[m - 1] = v_m:
+// 4th order 8 (v_1 - v_-1) - (v_2 - v_-2) (= 12 h u'), 8th order
+// 672 d1 - 168 d2 + 32 d3 - 3 d4 (= 840 h u'), dm = v_m - v_-m; in aligned
+// integers (sc_fixed.cuh), or in FP64 where the values do not allow that.
+template <int ORD>
+__device__ __forceinline__ double dfirst(const double* lo, const double* hi) {
+  using F = FxSums<ORD>;
+  constexpr int R = ORD / 2;
+  int E = 0;
+#pragma unroll
+  for (int m = 0; m < R; ++m) E = max(E, max(fx_exp(lo[m]), fx_exp(hi[m])));
+  if (aligned_ok(E)) {
+    typename F::Val l[R], h[R];
+#pragma unroll
+    for (int m = 0; m < R; ++m) {
+      l[m] = F::val(lo[m], E);
+      h[m] = F::val(hi[m], E);
+    }
+    return F::first(l, h, E);
+  }
+  if (ORD == 4) return fma(8.0, hi[0], fma(-8.0, lo[0], lo[1] - hi[1]));
+  return fma(672.0, hi[0] - lo[0], fma(-168.0, hi[1] - lo[1], fma(32.0, hi[2] - lo[2], -3.0 * (hi[3] - lo[3]))));
 }
 
-template <int ORD, class KT = FmaK>
+template <int ORD>
 __global__ void __launch_bounds__(128) z4c_dxy_kernel(const double* __restrict__ Y, double* __restrict__ S, long fs,
-                                                     int sy_, const RowSeg* __restrict__ segs, int nsegs, KT K) {
+                                                     int sy_, const RowSeg* __restrict__ segs, int nsegs) {
   constexpr int R = ORD / 2;
   const long sy = sy_;
   for (int sgi = blockIdx.x; sgi < nsegs; sgi += gridDim.x) {
@@ -166,7 +157,7 @@ __global__ void __launch_bounds__(128) z4c_dxy_kernel(const double* __restrict__
           lo[m - 1] = u[-m];
           hi[m - 1] = u[m];
         }
-        S[(long)(Q_D1 + 3 * f + 0) * fs + o] = dfirst<ORD>(lo, hi, K);
+        S[(long)(Q_D1 + 3 * f + 0) * fs + o] = dfirst<ORD>(lo, hi);
       }
       if (sg.which & 2) {
 #pragma unroll
@@ -174,17 +165,45 @@ __global__ void __launch_bounds__(128) z4c_dxy_kernel(const double* __restrict__
           lo[m - 1] = u[-m * sy];
           hi[m - 1] = u[m * sy];
         }
-        S[(long)(Q_D1 + 3 * f + 1) * fs + o] = dfirst<ORD>(lo, hi, K);
+        S[(long)(Q_D1 + 3 * f + 1) * fs + o] = dfirst<ORD>(lo, hi);
       }
     }
   }
 }
 
-template <int ORD, class KT = FmaK>
+// The sums of one cell that need u at the cell and its neighbours along the
+// three axes (lo[d][m - 1] = u at -m along d), in FP64: D_d of the axes in
+// dmask, the Kreiss-Oliger sum and, for d2 != null, the pure second
+// derivatives.  The form of the cells that aligned_ok refuses.
+template <int ORD>
+__device__ __forceinline__ void cell_sums_fp64(double u0, const double (*lo)[ORD == 4 ? 3 : 4],
+                                               const double (*hi)[ORD == 4 ? 3 : 4], double* d1, double* ko,
+                                               double* d2) {
+  double P[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    double p[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int m = 0; m < (ORD == 4 ? 3 : 4); ++m) p[m] = lo[d][m] + hi[d][m];
+    if (ORD == 4) {
+      d1[d] = fma(8.0, hi[d][0], fma(-8.0, lo[d][0], lo[d][1] - hi[d][1]));
+      d2[d] = fma(16.0, p[0], fma(-30.0, u0, -p[1]));
+    } else {
+      d1[d] = fma(672.0, hi[d][0] - lo[d][0],
+                  fma(-168.0, hi[d][1] - lo[d][1], fma(32.0, hi[d][2] - lo[d][2], -3.0 * (hi[d][ORD == 4 ? 0 : 3] - lo[d][ORD == 4 ? 0 : 3]))));
+      d2[d] = fma(-14350.0, u0, fma(8064.0, p[0], fma(-1008.0, p[1], fma(128.0, p[2], -9.0 * p[3]))));
+    }
+#pragma unroll
+    for (int m = 0; m < 3; ++m) P[m] += p[m];
+  }
+  *ko = fma(15.0, P[0], fma(-6.0, P[1], fma(-60.0, u0, P[2])));
+}
+
+template <int ORD>
 __global__ void __launch_bounds__(kThreads, 2) z4c_derivs_split_kernel(const double* __restrict__ Y,
                                                                       double* __restrict__ S, long fs, int sy_,
                                                                       int sz_, const Tile* __restrict__ tiles, int ntiles,
-                                                                      int max_cols, KT K) {
+                                                                      int max_cols) {
   // One thread per (x, y, field) column of a tile, walking z with sliding
   // windows: u at z-W..z+W (W = max(R, 3), R = ORD/2 the derivative radius,
   // 3 the Kreiss-Oliger radius) and, for the Hessian fields, the stored
@@ -192,6 +211,7 @@ __global__ void __launch_bounds__(kThreads, 2) z4c_derivs_split_kernel(const dou
   // Work is dealt out in units of (tile, chunk of blockDim (field, column)
   // pairs), U chunks per tile (max_cols = the largest tile's columns), so
   // the persistent blocks end together whatever the tile count.
+  using F = FxSums<ORD>;
   constexpr int R = ORD / 2;
   constexpr int WR = R > 3 ? R : 3;
   constexpr int NW = 2 * WR + 1;
@@ -224,124 +244,84 @@ __global__ void __launch_bounds__(kThreads, 2) z4c_derivs_split_kernel(const dou
           wy[m] = Dy[(m - R) * sz];
         }
       }
-      // 4th order: two z steps in flight (2.4% faster than one, measured); the
-      // 8th-order windows leave no registers for that
-#pragma unroll(ORD == 4 ? 2 : 1)
+#pragma unroll(1)
       for (int k = 0; k < T.nz; ++k) {
         const long o = o0 + k * sz;
         const double* v = u + k * sz;
-        if (ORD == 4) {
-          // 4th order: every weighted value through a general FMA (see dfirst)
-          const double u0 = w[WR];
-          // u along x and y from memory, along z from the window
-          double lo[3][WR], hi[3][WR];
+        const double u0 = w[WR];
+        // u along x and y from memory, along z from the window
+        double lo[3][WR], hi[3][WR];
+        int E = fx_exp(u0);
 #pragma unroll
-          for (int m = 1; m <= WR; ++m) {
-            lo[0][m - 1] = v[-m];
-            hi[0][m - 1] = v[m];
-            lo[1][m - 1] = v[-m * sy];
-            hi[1][m - 1] = v[m * sy];
-            lo[2][m - 1] = w[WR - m];
-            hi[2][m - 1] = w[WR + m];
+        for (int m = 1; m <= WR; ++m) {
+          lo[0][m - 1] = v[-m];
+          hi[0][m - 1] = v[m];
+          lo[1][m - 1] = v[-m * sy];
+          hi[1][m - 1] = v[m * sy];
+          lo[2][m - 1] = w[WR - m];
+          hi[2][m - 1] = w[WR + m];
+        }
+#pragma unroll
+        for (int dim = 0; dim < 3; ++dim)
+#pragma unroll
+          for (int m = 0; m < WR; ++m) E = max(E, max(fx_exp(lo[dim][m]), fx_exp(hi[dim][m])));
+        double* d1 = S + (long)(Q_D1 + 3 * f) * fs + o;
+        double* d2 = S + (long)(Q_D2 + 6 * sl) * fs + o;
+        double* ko = S + (long)(Q_KO + f) * fs + o;
+        if (aligned_ok(E)) {
+          // One alignment for every sum of the cell.
+          typename F::Val P[3];
+          const typename F::Val x0 = F::val(u0, E);
+#pragma unroll
+          for (int dim = 0; dim < 3; ++dim) {
+            typename F::Val l[WR], h[WR];
+#pragma unroll
+            for (int m = 0; m < WR; ++m) {
+              l[m] = F::val(lo[dim][m], E);
+              h[m] = F::val(hi[dim][m], E);
+            }
+            // D_x, D_y of the Hessian fields are there already (z4c_dxy_kernel)
+            if (sl < 0 || dim == 2) d1[dim * fs] = F::first(l, h, E);
+            typename F::Val p[WR];
+#pragma unroll
+            for (int m = 0; m < WR; ++m) p[m] = l[m] + h[m];
+            if (sl >= 0) d2[(dim == 0 ? 0 : dim == 1 ? 3 : 5) * fs] = F::second(p, x0, E);
+#pragma unroll
+            for (int m = 0; m < 3; ++m) P[m] = dim == 0 ? p[m] : P[m] + p[m];
           }
-          // Kreiss-Oliger (r = 4): sum_d (u_-3 - 6 u_-2 + 15 u_-1 - 20 u_0 + 15 u_1 - 6 u_2 + u_3)
-          double ko;
-          if (sl < 0) {
-#pragma unroll
-            for (int dim = 0; dim < 3; ++dim) S[(long)(Q_D1 + 3 * f + dim) * fs + o] = dfirst<ORD>(lo[dim], hi[dim], K);
-            ko = fma(-60.0, u0, lo[0][2]);
-            ko = fadd(ko, hi[0][2], K);
-#pragma unroll
-            for (int dim = 1; dim < 3; ++dim) ko = fadd(fadd(ko, lo[dim][2], K), hi[dim][2], K);
-#pragma unroll
-            for (int dim = 0; dim < 3; ++dim)
-              ko = fma(15.0, hi[dim][0], fma(15.0, lo[dim][0], fma(-6.0, hi[dim][1], fma(-6.0, lo[dim][1], ko))));
-          } else {
-            // Hessian fields: the pair sums of the second derivatives, shared with the KO sum
-            double p[3][2];
-#pragma unroll
-            for (int dim = 0; dim < 3; ++dim)
-#pragma unroll
-              for (int m = 0; m < 2; ++m) p[dim][m] = fadd(lo[dim][m], hi[dim][m], K);
-            double* d2 = S + (long)(Q_D2 + 6 * sl) * fs + o;
-            d2[0 * fs] = dsecond<ORD>(p[0], u0, K);
-            d2[3 * fs] = dsecond<ORD>(p[1], u0, K);
-            d2[5 * fs] = dsecond<ORD>(p[2], u0, K);
-            ko = fma(-60.0, u0, lo[0][2]);
-            ko = fadd(ko, hi[0][2], K);
-#pragma unroll
-            for (int dim = 1; dim < 3; ++dim) ko = fadd(fadd(ko, lo[dim][2], K), hi[dim][2], K);
-            // D_z from the pair sums: 16 v_1 - 8 p1 - 2 v_2 + p2 = 8 (v_1 - v_-1) - (v_2 - v_-2)
-            S[(long)(Q_D1 + 3 * f + 2) * fs + o] =
-                fma(16.0, hi[2][0], fma(-8.0, p[2][0], fma(-2.0, hi[2][1], p[2][1])));
-#pragma unroll
-            for (int dim = 0; dim < 3; ++dim) ko = fma(15.0, p[dim][0], fma(-6.0, p[dim][1], ko));
-            // mixed: the first-derivative stencil applied to the stored D_x (along y and z) and D_y (along z)
-            double ml[R], mh[R];
-            const double* dxk = Dx + k * sz;
-#pragma unroll
-            for (int m = 1; m <= R; ++m) {
-              ml[m - 1] = dxk[-m * sy];
-              mh[m - 1] = dxk[m * sy];
-            }
-            d2[1 * fs] = dfirst<ORD>(ml, mh, K);  // D_y D_x
-#pragma unroll
-            for (int m = 1; m <= R; ++m) {
-              ml[m - 1] = wx[R - m];
-              mh[m - 1] = wx[R + m];
-            }
-            d2[2 * fs] = dfirst<ORD>(ml, mh, K);  // D_z D_x
-#pragma unroll
-            for (int m = 1; m <= R; ++m) {
-              ml[m - 1] = wy[R - m];
-              mh[m - 1] = wy[R + m];
-            }
-            d2[4 * fs] = dfirst<ORD>(ml, mh, K);  // D_z D_y
-          }
-          S[(long)(Q_KO + f) * fs + o] = ko;
+          *ko = F::ko(P[0], P[1], P[2], x0, E);
         } else {
-          // 8th order: differences and pair sums formed first (the 4th-order
-          // arrangement ran 6% slower at radius 4, with or without spills)
-          const double u0 = w[WR];
-          double p[3][4], d[4];
-          // x and y from memory, z from the window
+          double e1[3], e2[3], eko;
+          cell_sums_fp64<ORD>(u0, lo, hi, e1, &eko, e2);
+          *ko = eko;
 #pragma unroll
-          for (int dim = 0; dim < 2; ++dim) {
-            const long s = dim == 0 ? 1 : sy;
-#pragma unroll
-            for (int m = 1; m <= WR; ++m) p[dim][m - 1] = fadd(v[-m * s], v[m * s], K);
-            if (sl < 0) {
-#pragma unroll
-              for (int m = 1; m <= R; ++m) d[m - 1] = fsub(v[m * s], v[-m * s], K);
-              S[(long)(Q_D1 + 3 * f + dim) * fs + o] = dfirst_d<ORD>(d, K);
-            }
+          for (int dim = 0; dim < 3; ++dim) {
+            if (sl < 0 || dim == 2) d1[dim * fs] = e1[dim];
+            if (sl >= 0) d2[(dim == 0 ? 0 : dim == 1 ? 3 : 5) * fs] = e2[dim];
           }
+        }
+        if (sl >= 0) {
+          // mixed: the first-derivative stencil applied to the stored D_x (along y and z) and D_y (along z)
+          double ml[R], mh[R];
+          const double* dxk = Dx + k * sz;
 #pragma unroll
-          for (int m = 1; m <= WR; ++m) p[2][m - 1] = fadd(w[WR - m], w[WR + m], K);
-#pragma unroll
-          for (int m = 1; m <= R; ++m) d[m - 1] = fsub(w[WR + m], w[WR - m], K);
-          S[(long)(Q_D1 + 3 * f + 2) * fs + o] = dfirst_d<ORD>(d, K);
-          // Kreiss-Oliger (r = 4): sum_d (u_-3 - 6 u_-2 + 15 u_-1 - 20 u_0 + 15 u_1 - 6 u_2 + u_3)
-          const double P1 = fadd(fadd(p[0][0], p[1][0], K), p[2][0], K);
-          const double P2 = fadd(fadd(p[0][1], p[1][1], K), p[2][1], K);
-          const double P3 = fadd(fadd(p[0][2], p[1][2], K), p[2][2], K);
-          S[(long)(Q_KO + f) * fs + o] = fma(15.0, P1, fma(-6.0, P2, fma(-60.0, u0, P3)));
-          if (sl >= 0) {
-            double* d2 = S + (long)(Q_D2 + 6 * sl) * fs + o;
-            d2[0 * fs] = dsecond<ORD>(p[0], u0, K);
-            d2[3 * fs] = dsecond<ORD>(p[1], u0, K);
-            d2[5 * fs] = dsecond<ORD>(p[2], u0, K);
-            const double* dxk = Dx + k * sz;
-#pragma unroll
-            for (int m = 1; m <= R; ++m) d[m - 1] = fsub(dxk[m * sy], dxk[-m * sy], K);
-            d2[1 * fs] = dfirst_d<ORD>(d, K);  // D_y D_x
-#pragma unroll
-            for (int m = 1; m <= R; ++m) d[m - 1] = fsub(wx[R + m], wx[R - m], K);
-            d2[2 * fs] = dfirst_d<ORD>(d, K);  // D_z D_x
-#pragma unroll
-            for (int m = 1; m <= R; ++m) d[m - 1] = fsub(wy[R + m], wy[R - m], K);
-            d2[4 * fs] = dfirst_d<ORD>(d, K);  // D_z D_y
+          for (int m = 1; m <= R; ++m) {
+            ml[m - 1] = dxk[-m * sy];
+            mh[m - 1] = dxk[m * sy];
           }
+          d2[1 * fs] = dfirst<ORD>(ml, mh);  // D_y D_x
+#pragma unroll
+          for (int m = 1; m <= R; ++m) {
+            ml[m - 1] = wx[R - m];
+            mh[m - 1] = wx[R + m];
+          }
+          d2[2 * fs] = dfirst<ORD>(ml, mh);  // D_z D_x
+#pragma unroll
+          for (int m = 1; m <= R; ++m) {
+            ml[m - 1] = wy[R - m];
+            mh[m - 1] = wy[R + m];
+          }
+          d2[4 * fs] = dfirst<ORD>(ml, mh);  // D_z D_y
         }
         if (k + 1 < T.nz) {  // slide the windows one cell up in z
 #pragma unroll
@@ -873,41 +853,24 @@ cudaError_t launch_z4c_derivs(const double* Y, double* scratch, long fs, int sy,
 }
 
 cudaError_t launch_z4c_dxy(const double* Y, double* scratch, long fs, int sy, const RowSeg* segs, int nsegs,
-                           cudaStream_t s, int order, bool op_class) {
+                           cudaStream_t s, int order) {
   if (nsegs == 0) return cudaSuccess;
   const int grid = nsegs < caps().dxy ? nsegs : caps().dxy;
-  const FmaK K{1.0, -1.0, -0.0};
-  if (op_class) {
-    if (order == 8) z4c_dxy_kernel<8, PlainK><<<grid, 128, 0, s>>>(Y, scratch, fs, sy, segs, nsegs, PlainK{});
-    else z4c_dxy_kernel<4, PlainK><<<grid, 128, 0, s>>>(Y, scratch, fs, sy, segs, nsegs, PlainK{});
-  } else if (order == 8) {
-    z4c_dxy_kernel<8><<<grid, 128, 0, s>>>(Y, scratch, fs, sy, segs, nsegs, K);
-  } else {
-    z4c_dxy_kernel<4><<<grid, 128, 0, s>>>(Y, scratch, fs, sy, segs, nsegs, K);
-  }
+  if (order == 8) z4c_dxy_kernel<8><<<grid, 128, 0, s>>>(Y, scratch, fs, sy, segs, nsegs);
+  else z4c_dxy_kernel<4><<<grid, 128, 0, s>>>(Y, scratch, fs, sy, segs, nsegs);
   return cudaGetLastError();
 }
 
 cudaError_t launch_z4c_derivs_split(const double* Y, double* scratch, long fs, int sy, int sz,
-                                    const Tile* tiles, int ntiles, cudaStream_t s, int order, int max_cols,
-                                    bool op_class) {
+                                    const Tile* tiles, int ntiles, cudaStream_t s, int order, int max_cols) {
   if (ntiles == 0) return cudaSuccess;
   if (max_cols < 1) return cudaErrorInvalidValue;
   const long units = (long)ntiles * ((max_cols * kNZ4c + kThreads - 1) / kThreads);
   const int grid = units < caps().derivs ? (int)units : caps().derivs;
-  const FmaK K{1.0, -1.0, -0.0};
-  if (op_class) {
-    if (order == 8)
-      z4c_derivs_split_kernel<8, PlainK><<<grid, kThreads, 0, s>>>(Y, scratch, fs, sy, sz, tiles, ntiles, max_cols,
-                                                                   PlainK{});
-    else
-      z4c_derivs_split_kernel<4, PlainK><<<grid, kThreads, 0, s>>>(Y, scratch, fs, sy, sz, tiles, ntiles, max_cols,
-                                                                   PlainK{});
-  } else if (order == 8) {
-    z4c_derivs_split_kernel<8><<<grid, kThreads, 0, s>>>(Y, scratch, fs, sy, sz, tiles, ntiles, max_cols, K);
-  } else {
-    z4c_derivs_split_kernel<4><<<grid, kThreads, 0, s>>>(Y, scratch, fs, sy, sz, tiles, ntiles, max_cols, K);
-  }
+  if (order == 8)
+    z4c_derivs_split_kernel<8><<<grid, kThreads, 0, s>>>(Y, scratch, fs, sy, sz, tiles, ntiles, max_cols);
+  else
+    z4c_derivs_split_kernel<4><<<grid, kThreads, 0, s>>>(Y, scratch, fs, sy, sz, tiles, ntiles, max_cols);
   return cudaGetLastError();
 }
 
