@@ -234,11 +234,10 @@ cudaError_t launch_z4c_dxy(const double* Y, double* scratch, long fs, int sy, co
 // chunks sized by it); cudaErrorInvalidValue if below 1.
 cudaError_t launch_z4c_derivs_split(const double* Y, double* scratch, long fs, int sy, int sz,
                                     const Tile* tiles, int ntiles, cudaStream_t s, int order, int max_cols);
-// bps: warps per scheduler of the stage kernel's build (the register budget of
-// bps 128-thread blocks per SM), 2 or 3 (a tuning choice); threads: block
-// size, 128 (tiles of at most 128 cells) or 64 (tiles of at most 64 cells, 2 bps
-// blocks per SM); cudaErrorInvalidValue otherwise.  op_class: the PlainK build
-// (stage form kStageSingle only, cudaErrorInvalidValue for the others).
+// bps: warps per scheduler that the stage kernel's build leaves registers for, 2
+// or 3 (a tuning choice); threads: the tiles' size, 128 or 64 cells;
+// cudaErrorInvalidValue otherwise.  op_class: the PlainK build (stage form
+// kStageSingle only, cudaErrorInvalidValue for the others).
 cudaError_t launch_z4c_stage(const StageArgs& a, const double* scratch, const Z4cParams& p,
                              const Tile* tiles, int ntiles, cudaStream_t s, int bps, int threads,
                              bool op_class = false);

@@ -15,21 +15,16 @@
 //      derivatives, evaluates the right-hand side, adds dissipation and
 //      performs the RK4 stage update.
 // FP64 is the scarce resource on this GPU (the FP64 pipe issues 1/64 of the
-// FP32 rate), so the arithmetic is arranged to minimise FP64 operations:
-// shared pair sums/differences in the stencils, fused multiply-adds, one
-// division for 1/det(gt) and one for 1/W, and the quadratic Christoffel
-// terms of the Ricci tensor contracted through one raised-index array.
+// FP32 rate), so both passes work in integers (sc_fixed.cuh: the stencil sums;
+// sc_z4c_fixed.cuh: the tensor contractions), and the FP64 forms beside them
+// are for the cells whose values the integer forms do not take.
 #include "sc_fixed.cuh"
+#include "sc_z4c_fixed.cuh"
 
 namespace sc {
 namespace {
 
 constexpr int kThreads = 256;
-
-// scratch slots
-constexpr int Q_D1 = 0;    // 3 * f + d: first derivative of field f along d
-constexpr int Q_D2 = 66;   // 6 * s + p: second derivative, s = slot (W, gt x6, alpha, beta x3), p = xx,xy,xz,yy,yz,zz
-constexpr int Q_KO = 132;  // f: sum_d delta_d^6 u_f (unscaled)
 
 // slot of field f among the fields with second derivatives, -1 if none
 __host__ __device__ inline int d2_slot(int f) {
@@ -340,11 +335,6 @@ __global__ void __launch_bounds__(kThreads, 2) z4c_derivs_split_kernel(const dou
       }
     }
   }
-}
-
-// symmetric index helpers: xx xy xz yy yz zz
-__device__ __forceinline__ int sidx(int i, int j) {
-  return (i == j) ? (i == 0 ? 0 : (i == 1 ? 3 : 5)) : (i + j == 1 ? 1 : (i + j == 2 ? 2 : 4));
 }
 
 // Right-hand side of the Z4c system at one cell (Sec. III.A; vacuum, so the
@@ -671,44 +661,89 @@ __device__ __forceinline__ void z4c_rhs_point(const double* __restrict__ Y, cons
 #undef D2
 }
 
+// The cells that the fixed-point form leaves to FP64, out of line: their
+// registers and spills stay out of the kernel's own budget.
+template <class KT>
+__device__ __noinline__ void z4c_rhs_fp64(const double* __restrict__ Y, const double* __restrict__ S, long fs, long o,
+                                          Z4cParams P, double eta, DerivScales ds, double* rhs, KT K) {
+  z4c_rhs_point<false>(Y, S, fs, o, P, eta, ds, rhs, nullptr, K);
+}
+
+// Dissipation and the stage update of one field at one cell.
+template <int FORM, class KT>
+struct StageUpdate {
+  const StageArgs& a;
+  const double* S;
+  long o;
+  double ko;
+  KT K;
+  struct Pre {
+    double ko, yn, k1, k2, k3;
+  };
+  __device__ __forceinline__ Pre load(int f) const {
+    const long fo = (long)f * a.fs + o;
+    Pre p;
+    p.ko = S[(long)(Q_KO + f) * a.fs + o];
+    if (FORM != kStageNone) p.yn = a.yn[fo];
+    if (FORM == kStageRk4 || FORM == kStageTwo) p.k1 = a.k1[fo];
+    if (FORM == kStageRk4) {
+      p.k2 = a.k2[fo];
+      p.k3 = a.k3[fo];
+    }
+    return p;
+  }
+  __device__ __forceinline__ void operator()(int f, double rhs, const Pre& p) const {
+    const long fo = (long)f * a.fs + o;
+    const double kv = fma(ko, p.ko, rhs);
+    a.k[fo] = kv;
+    if (FORM == kStageSingle) {
+      a.out[fo] = fma(a.cdt, kv, p.yn);
+    } else if (FORM == kStageRk4) {
+      const double s = fadd(fma(2.0, p.k3, fma(2.0, p.k2, p.k1)), kv, K);
+      a.out[fo] = fma(a.cdt, s, p.yn);
+    } else if (FORM == kStageTwo) {
+      a.out[fo] = fma(a.cdt, kv, fma(a.c1dt, p.k1, p.yn));
+    }
+  }
+};
+
 // FORM: the stage update of StageArgs (kStageSingle, kStageRk4, kStageTwo,
-// kStageNone), fixed at compile time so the update adds no registers to the
-// RHS.  BPS: warps per scheduler the build is constrained to (the register
-// budget of BPS 128-thread blocks per SM), a choice of sc_autotune: 3 (at
-// most 168 registers; the RHS then spills about 1 KB per thread, written back
-// to DRAM, which the FP64-bound kernel can afford, while 3 warps per
-// scheduler instead of 2 hide the FP64 dependency latency better) or 2 (255
-// registers, a few spills).  Blocks of 128 threads over 128-cell tiles, or
-// of 64 threads over 64-cell tiles (twice as many per SM) on large levels,
-// where the finer split balances the SMs (the host picks per level).
+// kStageNone), fixed at compile time.  Blocks of 64 threads take 64 cells at a
+// time (a tile, or half of a 128-cell one), so that 152 SMs share the 125 units
+// of a 20^3 level.  BPS (a choice of sc_autotune): 2 leaves 255 registers a
+// thread, 3 has six blocks of 168 registers per SM, as many as the tensors'
+// shared memory (35 KB a block) allows.
+// Bound by latency and issue: 14,750 instructions a cell (7,700 on the integer ALU,
+// 5,300 multiply-adds and moves, 130 FP64) at 1.3 per clock and SM.  262,144 cells:
+// 0.501 ms in FP64 (97% of that pipe's ceiling), 0.269 with BPS 2, 0.287 with 3;
+// 110,592 cells: 0.290, 0.155, 0.164; 8,000 cells: 0.041, 0.029, 0.031.
+constexpr int kStageThreads = 64;
+
 template <int FORM, int BPS, class KT = FmaK>
-__global__ void __launch_bounds__(128, BPS) z4c_stage_kernel(StageArgs a, const double* __restrict__ S, Z4cParams P,
-                                                            const Tile* __restrict__ tiles, int ntiles, KT K) {
+__global__ void __launch_bounds__(kStageThreads, 2 * BPS) z4c_stage_kernel(StageArgs a, const double* __restrict__ S,
+                                                                          Z4cParams P, const Tile* __restrict__ tiles,
+                                                                          int ntiles, int chunks,
+                                                                          const __grid_constant__ FxScales c, KT K) {
+  __shared__ long long slots[FM_SLOTS * kStageThreads];
+  const FxMem<kStageThreads> mem{slots + threadIdx.x};
   const double ko = P.ko_sigma / (64.0 * a.h);
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const Tile T = tiles[t];
-    const int n = T.nx * T.ny * T.nz;
-    for (int q = threadIdx.x; q < n; q += blockDim.x) {
-      const int i = q % T.nx;
-      const int j = (q / T.nx) % T.ny;
-      const int k = q / (T.nx * T.ny);
-      const long o = (long)(T.z0 + k) * a.sz + (long)(T.y0 + j) * a.sy + (T.x0 + i);
+  for (int u = blockIdx.x; u < ntiles * chunks; u += gridDim.x) {
+    const Tile T = tiles[u / chunks];
+    const int q = u % chunks * kStageThreads + threadIdx.x;
+    if (q >= T.nx * T.ny * T.nz) continue;
+    const int i = q % T.nx;
+    const int j = (q / T.nx) % T.ny;
+    const int k = q / (T.nx * T.ny);
+    const long o = (long)(T.z0 + k) * a.sz + (long)(T.y0 + j) * a.sy + (T.x0 + i);
+    const double eta = a.eta ? a.eta[o] : P.eta;
+    const StageUpdate<FORM, KT> update{a, S, o, ko, K};
+    // (the stage's inputs and outputs are different arrays, so a cell that turns
+    // out to need the FP64 form is simply written again)
+    if (!z4c_rhs_fixed(a.Y, S, a.fs, o, P, eta, c, mem, K, update)) {
       double rhs[kNZ4c];
-      z4c_rhs_point<false>(a.Y, S, a.fs, o, P, a.eta ? a.eta[o] : P.eta, a.ds, rhs, nullptr, K);
-#pragma unroll
-      for (int f = 0; f < kNZ4c; ++f) {
-        const long fo = (long)f * a.fs + o;
-        const double kv = fma(ko, S[(long)(Q_KO + f) * a.fs + o], rhs[f]);
-        a.k[fo] = kv;
-        if (FORM == kStageSingle) {
-          a.out[fo] = fma(a.cdt, kv, a.yn[fo]);
-        } else if (FORM == kStageRk4) {
-          const double s = fadd(fma(2.0, a.k3[fo], fma(2.0, a.k2[fo], a.k1[fo])), kv, K);
-          a.out[fo] = fma(a.cdt, s, a.yn[fo]);
-        } else if (FORM == kStageTwo) {
-          a.out[fo] = fma(a.cdt, kv, fma(a.c1dt, a.k1[fo], a.yn[fo]));
-        }
-      }
+      z4c_rhs_fp64(a.Y, S, a.fs, o, P, eta, a.ds, rhs, K);
+#pragma unroll 1
+      for (int f = 0; f < kNZ4c; ++f) update(f, rhs[f], update.load(f));
     }
   }
 }
@@ -827,11 +862,11 @@ cudaError_t z4c_init_launch_config() {
   GridCaps& c = g_caps[dev & 63];
   if (c.ready) return cudaSuccess;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, z4c_stage_kernel<kStageSingle, 2>, 128, 0)) !=
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, z4c_stage_kernel<kStageSingle, 2>, kStageThreads, 0)) !=
       cudaSuccess)
     return e;
   c.stage[2] = nsm * (occ > 0 ? occ : 1);
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, z4c_stage_kernel<kStageSingle, 3>, 128, 0)) !=
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, z4c_stage_kernel<kStageSingle, 3>, kStageThreads, 0)) !=
       cudaSuccess)
     return e;
   c.stage[3] = nsm * (occ > 0 ? occ : 1);
@@ -878,14 +913,15 @@ namespace {
 
 template <int BPS>
 void launch_stage_bps(const StageArgs& a, const double* scratch, const Z4cParams& p, const Tile* tiles, int ntiles,
-                      int grid, int threads, cudaStream_t s, const FmaK& K, bool op_class) {
+                      int grid, int chunks, cudaStream_t s, const FmaK& K, bool op_class) {
+  const FxScales c = fx_scales(a.ds);
   if (op_class)
-    z4c_stage_kernel<kStageSingle, BPS, PlainK><<<grid, threads, 0, s>>>(a, scratch, p, tiles, ntiles, PlainK{});
-  else if (a.form == kStageRk4) z4c_stage_kernel<kStageRk4, BPS><<<grid, threads, 0, s>>>(a, scratch, p, tiles, ntiles, K);
-  else if (a.form == kStageTwo) z4c_stage_kernel<kStageTwo, BPS><<<grid, threads, 0, s>>>(a, scratch, p, tiles, ntiles, K);
+    z4c_stage_kernel<kStageSingle, BPS, PlainK><<<grid, kStageThreads, 0, s>>>(a, scratch, p, tiles, ntiles, chunks, c, PlainK{});
+  else if (a.form == kStageRk4) z4c_stage_kernel<kStageRk4, BPS><<<grid, kStageThreads, 0, s>>>(a, scratch, p, tiles, ntiles, chunks, c, K);
+  else if (a.form == kStageTwo) z4c_stage_kernel<kStageTwo, BPS><<<grid, kStageThreads, 0, s>>>(a, scratch, p, tiles, ntiles, chunks, c, K);
   else if (a.form == kStageNone)
-    z4c_stage_kernel<kStageNone, BPS><<<grid, threads, 0, s>>>(a, scratch, p, tiles, ntiles, K);
-  else z4c_stage_kernel<kStageSingle, BPS><<<grid, threads, 0, s>>>(a, scratch, p, tiles, ntiles, K);
+    z4c_stage_kernel<kStageNone, BPS><<<grid, kStageThreads, 0, s>>>(a, scratch, p, tiles, ntiles, chunks, c, K);
+  else z4c_stage_kernel<kStageSingle, BPS><<<grid, kStageThreads, 0, s>>>(a, scratch, p, tiles, ntiles, chunks, c, K);
 }
 
 }  // namespace
@@ -898,11 +934,12 @@ cudaError_t launch_z4c_stage(const StageArgs& a, const double* scratch, const Z4
   if (op_class && a.form != kStageSingle) return cudaErrorInvalidValue;
   // persistent grid: the resident blocks (twice as many at 64 threads, whose
   // registers per block are half)
-  const int cap = caps().stage[bps] * (128 / threads);
-  const int grid = ntiles < cap ? ntiles : cap;
+  const int cap = caps().stage[bps], chunks = threads / kStageThreads;
+  const long units = (long)ntiles * chunks;
+  const int grid = units < cap ? (int)units : cap;
   const FmaK K{1.0, -1.0, -0.0};
-  if (bps == 2) launch_stage_bps<2>(a, scratch, p, tiles, ntiles, grid, threads, s, K, op_class);
-  else launch_stage_bps<3>(a, scratch, p, tiles, ntiles, grid, threads, s, K, op_class);
+  if (bps == 2) launch_stage_bps<2>(a, scratch, p, tiles, ntiles, grid, chunks, s, K, op_class);
+  else launch_stage_bps<3>(a, scratch, p, tiles, ntiles, grid, chunks, s, K, op_class);
   return cudaGetLastError();
 }
 
