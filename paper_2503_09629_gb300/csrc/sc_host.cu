@@ -255,10 +255,9 @@ struct Level {
   int ntiles = 0;
   int tile_cols = 0;                // largest nx * ny of the tiles
   std::vector<int> box_tile_begin;  // tiles of box b: [box_tile_begin[b], box_tile_begin[b + 1])
-  Tile* ptiles = nullptr;           // 32 x ny x 1 tiles for the pointwise Z4c kernel (one cell per thread)
-  int nptiles = 0;
-  int ptile_threads = 128;          // 32 * ny: the stage kernel's block size on this level
-  std::vector<int> box_ptile_begin;
+  CellRun* runs = nullptr;          // the pointwise Z4c kernel's units (one cell per thread)
+  int nruns = 0;
+  std::vector<int> box_run_begin;
   AmrCell* amr = nullptr;
   int namr = 0;
   AmrTile* atiles = nullptr;  // separable-prolongation tiles and their position -> AMR index map
@@ -455,7 +454,7 @@ sc_status validate(const sc_desc* d) {
 // Build geometry, classification and work lists of every level (host side).
 struct HostLists {
   std::vector<Tile> tiles;
-  std::vector<Tile> ptiles;
+  std::vector<CellRun> runs;
   std::vector<AmrCell> amr;
   std::vector<int> amr_gi, amr_gw;  // unwrapped / wrapped global fine index per AMR cell
   std::vector<AmrTile> atiles;      // slab tiles served by the separable kernel
@@ -766,33 +765,21 @@ sc_status classify_level(sc_ctx* c, int l, HostLists& hl) {
       }
   if (l > 0 && !hl.amr.empty()) build_amr_tiles(c, l, hl);
   build_stencil_tiles(L, c->tile, hl.tiles);
-  // Pointwise tiles of the Z4c stage kernel, one cell per thread: 64-cell
-  // tiles in 64-thread blocks on levels of at least 2^17 cells (a 64^3
-  // level's 4096 tiles split over the 152 SMs to within 0.2%, against 4% for
-  // 2048 tiles of 128 cells: 892 instead of 895 ms per step of the 7-level
-  // benchmark), 128-cell tiles in 128-thread blocks on smaller ones (requests
-  // of that size served concurrently on streams ran 3% slower in total with
-  // the smaller blocks: 2.73e8 against 2.82e8 zone-updates/s on the serving
-  // ensemble).
-  const int pny = L.interior_cells >= (1L << 17) ? 2 : 4;
-  L.ptile_threads = 32 * pny;
-  L.box_ptile_begin.clear();
+  // Runs of cells of the Z4c stage kernel, one cell per thread.
+  L.box_run_begin.clear();
   for (const sc_box& B : L.boxes) {
-    L.box_ptile_begin.push_back((int)hl.ptiles.size());
-    for (int z = B.lo[2]; z <= B.hi[2]; ++z)
-      for (int y = B.lo[1]; y <= B.hi[1]; y += pny)
-        for (int x = B.lo[0]; x <= B.hi[0]; x += 32) {
-          Tile t;
-          t.x0 = x - g.org[0];
-          t.y0 = y - g.org[1];
-          t.z0 = z - g.org[2];
-          t.nx = std::min(32, B.hi[0] - x + 1);
-          t.ny = std::min(pny, B.hi[1] - y + 1);
-          t.nz = 1;
-          hl.ptiles.push_back(t);
-        }
+    L.box_run_begin.push_back((int)hl.runs.size());
+    CellRun r;
+    r.off = (int32_t)g.off(B.lo[0], B.lo[1], B.lo[2]);
+    r.nx = B.hi[0] - B.lo[0] + 1;
+    r.ny = B.hi[1] - B.lo[1] + 1;
+    const int cells = r.nx * r.ny * (B.hi[2] - B.lo[2] + 1);
+    for (r.first = 0; r.first < cells; r.first += kRunCells) {
+      r.n = std::min(kRunCells, cells - r.first);
+      hl.runs.push_back(r);
+    }
   }
-  L.box_ptile_begin.push_back((int)hl.ptiles.size());
+  L.box_run_begin.push_back((int)hl.runs.size());
   // rows where the Z4c evolution stores D_x (interior cells and their 2-cell
   // extension in y or z) and D_y (extension in z) of the Hessian fields
   if (c->system == SC_Z4C) {
@@ -924,13 +911,13 @@ sc_status setup_level_device(sc_ctx* c, int l, HostLists& hl) {
       (st = level_upload(c, L, hl.periodic, &L.periodic)) || (st = level_upload(c, L, hl.phys, &L.phys)) ||
       (st = level_upload(c, L, hl.restr, &L.restr)) || (st = level_upload(c, L, hl.rblocks, &L.rblocks)) ||
       (st = level_upload(c, L, hl.atiles, &L.atiles)) || (st = level_upload(c, L, hl.aslots, &L.aslots)) ||
-      (st = level_upload(c, L, hl.dxy, &L.dxy)) || (st = level_upload(c, L, hl.ptiles, &L.ptiles)))
+      (st = level_upload(c, L, hl.dxy, &L.dxy)) || (st = level_upload(c, L, hl.runs, &L.runs)))
     return st;
   L.ntiles = (int)hl.tiles.size();
   L.namr = (int)hl.amr.size();
   L.natiles = (int)hl.atiles.size();
   L.tile_fmas = hl.tile_fmas;
-  L.nptiles = (int)hl.ptiles.size();
+  L.nruns = (int)hl.runs.size();
   L.ndxy = (int)hl.dxy.size();
   L.namr_blocked = hl.namr_blocked;
   L.nperiodic = (int)hl.periodic.size();
@@ -1190,13 +1177,13 @@ sc_status run_op(sc_ctx* c, const Op& o, cudaStream_t s) {
         if (c->system == SC_WAVE) {
           CU(launch_wave_stage(a, L.tiles + t0, nt, s, c->order, foldp));
         } else {
-          const int p0 = nparts == 1 ? 0 : L.box_ptile_begin[b];
-          const int np = nparts == 1 ? L.nptiles : L.box_ptile_begin[b + 1] - p0;
+          const int p0 = nparts == 1 ? 0 : L.box_run_begin[b];
+          const int np = nparts == 1 ? L.nruns : L.box_run_begin[b + 1] - p0;
           if (one_pass) CU(launch_z4c_derivs(a.Y, c->scratch, g.fs, a.sy, a.sz, L.tiles + t0, nt, s));
           else
             CU(launch_z4c_derivs_split(a.Y, c->scratch, g.fs, a.sy, a.sz, L.tiles + t0, nt, s, c->order,
                                        L.tile_cols));
-          CU(launch_z4c_stage(a, c->scratch, c->zp, L.ptiles + p0, np, s, c->stage_bps, L.ptile_threads));
+          CU(launch_z4c_stage(a, c->scratch, c->zp, L.runs + p0, np, s, c->stage_bps));
         }
       }
       if (L.nphys) CU(launch_radiative_stage(a, L.phys, L.nphys, c->F, g, c->system, s));
@@ -1617,7 +1604,7 @@ sc_status time_candidate(sc_ctx* c, Level& L, int kind, const Tile* tiles, int n
   for (int r = -1; r < reps; ++r) {
     if (r == 0) CU(cudaEventRecord(e0, c->stream));
     if (kind == 1) {
-      CU(launch_z4c_stage(a, c->scratch, c->zp, L.ptiles, L.nptiles, c->stream, bps, L.ptile_threads));
+      CU(launch_z4c_stage(a, c->scratch, c->zp, L.runs, L.nruns, c->stream, bps));
     } else if (c->system == SC_WAVE) {
       CU(launch_wave_stage(a, tiles, ntiles, c->stream, c->order));
     } else if (deriv_form == 1) {
@@ -2426,7 +2413,7 @@ sc_status sc_time_stage_kernels(sc_ctx* c, int level, int nrep, double* ms) {
   CU(cudaEventRecord(e[1], c->stream));
   if (c->system == SC_Z4C)
     for (int r = 0; r < nrep; ++r)
-      CU(launch_z4c_stage(a, c->scratch, c->zp, L.ptiles, L.nptiles, c->stream, c->stage_bps, L.ptile_threads));
+      CU(launch_z4c_stage(a, c->scratch, c->zp, L.runs, L.nruns, c->stream, c->stage_bps));
   CU(cudaEventRecord(e[2], c->stream));
   CU(cudaEventSynchronize(e[2]));
   CU(cudaEventElapsedTime(&t0, e[0], e[1]));
@@ -2446,7 +2433,7 @@ sc_status sc_run_op_class_pass(sc_ctx* c, int level) {
   const StageArgs a = tuning_stage_args(L, c->order);
   CU(launch_z4c_dxy(a.Y, c->scratch, g.fs, a.sy, L.dxy, L.ndxy, c->stream, c->order));
   CU(launch_z4c_derivs_split(a.Y, c->scratch, g.fs, a.sy, a.sz, L.tiles, L.ntiles, c->stream, c->order, L.tile_cols));
-  CU(launch_z4c_stage(a, c->scratch, c->zp, L.ptiles, L.nptiles, c->stream, c->stage_bps, L.ptile_threads, true));
+  CU(launch_z4c_stage(a, c->scratch, c->zp, L.runs, L.nruns, c->stream, c->stage_bps, true));
   CU(cudaStreamSynchronize(c->stream));
   return SC_OK;
 }

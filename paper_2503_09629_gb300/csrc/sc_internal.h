@@ -41,6 +41,16 @@ struct Tile {
   int x0, y0, z0, nx, ny, nz;
 };
 
+// Up to 64 consecutive cells of a box, numbered x-fastest over the whole box:
+// array offset of the box's first cell, its extents in x and y, and the numbers
+// of the run's first cell and of its cells.
+struct CellRun {
+  int32_t off;
+  int32_t nx, ny;
+  int32_t first, n;
+};
+constexpr int kRunCells = 64;
+
 // Refinement-boundary ghost cell: destination offset in the fine array,
 // offset of the first parent stencil cell in the parent array, parity of
 // the fine index per dimension (bit d set: fine centre at +1/4 parent cell).
@@ -235,12 +245,10 @@ cudaError_t launch_z4c_dxy(const double* Y, double* scratch, long fs, int sy, co
 cudaError_t launch_z4c_derivs_split(const double* Y, double* scratch, long fs, int sy, int sz,
                                     const Tile* tiles, int ntiles, cudaStream_t s, int order, int max_cols);
 // bps: warps per scheduler that the stage kernel's build leaves registers for, 2
-// or 3 (a tuning choice); threads: the tiles' size, 128 or 64 cells;
-// cudaErrorInvalidValue otherwise.  op_class: the PlainK build (stage form
-// kStageSingle only, cudaErrorInvalidValue for the others).
-cudaError_t launch_z4c_stage(const StageArgs& a, const double* scratch, const Z4cParams& p,
-                             const Tile* tiles, int ntiles, cudaStream_t s, int bps, int threads,
-                             bool op_class = false);
+// or 3 (a tuning choice); cudaErrorInvalidValue otherwise.  op_class: the PlainK
+// build (stage form kStageSingle only, cudaErrorInvalidValue for the others).
+cudaError_t launch_z4c_stage(const StageArgs& a, const double* scratch, const Z4cParams& p, const CellRun* runs,
+                             int nruns, cudaStream_t s, int bps, bool op_class = false);
 cudaError_t launch_radiative_stage(const StageArgs& a, const int32_t* cells, int ncells, int F,
                                    const Geom& g, int system, cudaStream_t s);
 cudaError_t launch_z4c_constraints(const double* Y, const double* scratch, double* out, long fs, int sy,

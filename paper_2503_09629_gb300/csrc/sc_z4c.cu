@@ -708,33 +708,30 @@ struct StageUpdate {
 };
 
 // FORM: the stage update of StageArgs (kStageSingle, kStageRk4, kStageTwo,
-// kStageNone), fixed at compile time.  Blocks of 64 threads take 64 cells at a
-// time (a tile, or half of a 128-cell one), so that 152 SMs share the 125 units
-// of a 20^3 level.  BPS (a choice of sc_autotune): 2 leaves 255 registers a
+// kStageNone), fixed at compile time.  A block takes the up to 64 cells of a
+// run, consecutive over the rows of a box, so that every lane has a cell whatever
+// the extents (tiles of 32 x 2 cells left 38% of the lanes idle at 20 or 40 cells
+// a row, 25% at 48), and the 152 SMs share the 125 runs of a 20^3 level.  BPS (a choice of sc_autotune): 2 leaves 255 registers a
 // thread, 3 has six blocks of 168 registers per SM, as many as the tensors'
 // shared memory (35 KB a block) allows.
 // Bound by latency and issue: 14,750 instructions a cell (7,700 on the integer ALU,
 // 5,300 multiply-adds and moves, 130 FP64) at 1.3 per clock and SM.  262,144 cells:
 // 0.501 ms in FP64 (97% of that pipe's ceiling), 0.269 with BPS 2, 0.287 with 3;
 // 110,592 cells: 0.290, 0.155, 0.164; 8,000 cells: 0.041, 0.029, 0.031.
-constexpr int kStageThreads = 64;
 
 template <int FORM, int BPS, class KT = FmaK>
-__global__ void __launch_bounds__(kStageThreads, 2 * BPS) z4c_stage_kernel(StageArgs a, const double* __restrict__ S,
-                                                                          Z4cParams P, const Tile* __restrict__ tiles,
-                                                                          int ntiles, int chunks,
-                                                                          const __grid_constant__ FxScales c, KT K) {
-  __shared__ long long slots[FM_SLOTS * kStageThreads];
-  const FxMem<kStageThreads> mem{slots + threadIdx.x};
+__global__ void __launch_bounds__(kRunCells, 2 * BPS) z4c_stage_kernel(StageArgs a, const double* __restrict__ S,
+                                                                      Z4cParams P, const CellRun* __restrict__ runs,
+                                                                      int nruns, const __grid_constant__ FxScales c,
+                                                                      KT K) {
+  __shared__ long long slots[FM_SLOTS * kRunCells];
+  const FxMem<kRunCells> mem{slots + threadIdx.x};
   const double ko = P.ko_sigma / (64.0 * a.h);
-  for (int u = blockIdx.x; u < ntiles * chunks; u += gridDim.x) {
-    const Tile T = tiles[u / chunks];
-    const int q = u % chunks * kStageThreads + threadIdx.x;
-    if (q >= T.nx * T.ny * T.nz) continue;
-    const int i = q % T.nx;
-    const int j = (q / T.nx) % T.ny;
-    const int k = q / (T.nx * T.ny);
-    const long o = (long)(T.z0 + k) * a.sz + (long)(T.y0 + j) * a.sy + (T.x0 + i);
+  for (int u = blockIdx.x; u < nruns; u += gridDim.x) {
+    const CellRun R = runs[u];
+    if ((int)threadIdx.x >= R.n) continue;
+    const int q = R.first + threadIdx.x, row = q / R.nx, z = row / R.ny;
+    const long o = R.off + (long)z * a.sz + (long)(row - z * R.ny) * a.sy + (q - row * R.nx);
     const double eta = a.eta ? a.eta[o] : P.eta;
     const StageUpdate<FORM, KT> update{a, S, o, ko, K};
     // (the stage's inputs and outputs are different arrays, so a cell that turns
@@ -842,7 +839,7 @@ __global__ void __launch_bounds__(128) z4c_constraints_kernel(const double* __re
 // evenly over the whole GPU instead of leaving a partial last wave.
 struct GridCaps {
   int ready = 0;
-  int stage[4] = {304, 304, 304, 456};  // 128-thread blocks, by warps per scheduler of the build (2 or 3)
+  int stage[4] = {608, 608, 608, 912};  // by warps per scheduler of the build (2 or 3)
   int derivs = 1216, dxy = 2432;
 };
 GridCaps g_caps[64];
@@ -862,11 +859,11 @@ cudaError_t z4c_init_launch_config() {
   GridCaps& c = g_caps[dev & 63];
   if (c.ready) return cudaSuccess;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, z4c_stage_kernel<kStageSingle, 2>, kStageThreads, 0)) !=
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, z4c_stage_kernel<kStageSingle, 2>, kRunCells, 0)) !=
       cudaSuccess)
     return e;
   c.stage[2] = nsm * (occ > 0 ? occ : 1);
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, z4c_stage_kernel<kStageSingle, 3>, kStageThreads, 0)) !=
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, z4c_stage_kernel<kStageSingle, 3>, kRunCells, 0)) !=
       cudaSuccess)
     return e;
   c.stage[3] = nsm * (occ > 0 ? occ : 1);
@@ -912,34 +909,30 @@ cudaError_t launch_z4c_derivs_split(const double* Y, double* scratch, long fs, i
 namespace {
 
 template <int BPS>
-void launch_stage_bps(const StageArgs& a, const double* scratch, const Z4cParams& p, const Tile* tiles, int ntiles,
-                      int grid, int chunks, cudaStream_t s, const FmaK& K, bool op_class) {
+void launch_stage_bps(const StageArgs& a, const double* scratch, const Z4cParams& p, const CellRun* runs, int nruns,
+                      int grid, cudaStream_t s, const FmaK& K, bool op_class) {
   const FxScales c = fx_scales(a.ds);
   if (op_class)
-    z4c_stage_kernel<kStageSingle, BPS, PlainK><<<grid, kStageThreads, 0, s>>>(a, scratch, p, tiles, ntiles, chunks, c, PlainK{});
-  else if (a.form == kStageRk4) z4c_stage_kernel<kStageRk4, BPS><<<grid, kStageThreads, 0, s>>>(a, scratch, p, tiles, ntiles, chunks, c, K);
-  else if (a.form == kStageTwo) z4c_stage_kernel<kStageTwo, BPS><<<grid, kStageThreads, 0, s>>>(a, scratch, p, tiles, ntiles, chunks, c, K);
+    z4c_stage_kernel<kStageSingle, BPS, PlainK><<<grid, kRunCells, 0, s>>>(a, scratch, p, runs, nruns, c, PlainK{});
+  else if (a.form == kStageRk4) z4c_stage_kernel<kStageRk4, BPS><<<grid, kRunCells, 0, s>>>(a, scratch, p, runs, nruns, c, K);
+  else if (a.form == kStageTwo) z4c_stage_kernel<kStageTwo, BPS><<<grid, kRunCells, 0, s>>>(a, scratch, p, runs, nruns, c, K);
   else if (a.form == kStageNone)
-    z4c_stage_kernel<kStageNone, BPS><<<grid, kStageThreads, 0, s>>>(a, scratch, p, tiles, ntiles, chunks, c, K);
-  else z4c_stage_kernel<kStageSingle, BPS><<<grid, kStageThreads, 0, s>>>(a, scratch, p, tiles, ntiles, chunks, c, K);
+    z4c_stage_kernel<kStageNone, BPS><<<grid, kRunCells, 0, s>>>(a, scratch, p, runs, nruns, c, K);
+  else z4c_stage_kernel<kStageSingle, BPS><<<grid, kRunCells, 0, s>>>(a, scratch, p, runs, nruns, c, K);
 }
 
 }  // namespace
 
-cudaError_t launch_z4c_stage(const StageArgs& a, const double* scratch, const Z4cParams& p, const Tile* tiles,
-                             int ntiles, cudaStream_t s, int bps, int threads, bool op_class) {
-  if (ntiles == 0) return cudaSuccess;
+cudaError_t launch_z4c_stage(const StageArgs& a, const double* scratch, const Z4cParams& p, const CellRun* runs,
+                             int nruns, cudaStream_t s, int bps, bool op_class) {
+  if (nruns == 0) return cudaSuccess;
   if (bps != 2 && bps != 3) return cudaErrorInvalidValue;
-  if (threads != 64 && threads != 128) return cudaErrorInvalidValue;
   if (op_class && a.form != kStageSingle) return cudaErrorInvalidValue;
-  // persistent grid: the resident blocks (twice as many at 64 threads, whose
-  // registers per block are half)
-  const int cap = caps().stage[bps], chunks = threads / kStageThreads;
-  const long units = (long)ntiles * chunks;
-  const int grid = units < cap ? (int)units : cap;
+  // persistent grid: the resident blocks
+  const int grid = nruns < caps().stage[bps] ? nruns : caps().stage[bps];
   const FmaK K{1.0, -1.0, -0.0};
-  if (bps == 2) launch_stage_bps<2>(a, scratch, p, tiles, ntiles, grid, chunks, s, K, op_class);
-  else launch_stage_bps<3>(a, scratch, p, tiles, ntiles, grid, chunks, s, K, op_class);
+  if (bps == 2) launch_stage_bps<2>(a, scratch, p, runs, nruns, grid, s, K, op_class);
+  else launch_stage_bps<3>(a, scratch, p, runs, nruns, grid, s, K, op_class);
   return cudaGetLastError();
 }
 
