@@ -8,7 +8,7 @@
 // own block range, so both forms execute identical arithmetic per value.
 #pragma once
 
-#include "sc_internal.h"
+#include "sc_fixed.cuh"
 
 namespace sc {
 
@@ -301,24 +301,44 @@ __device__ __forceinline__ void wave_stage_body(const StageArgs& a, const Tile* 
       const int j = (q / T.nx) % T.ny;
       const int k = q / (T.nx * T.ny);
       const long o = (T.z0 + k) * sz + (T.y0 + j) * sy + (T.x0 + i);
-      const double* u = a.Y;
-      const double u0 = u[o];
-      // 4th order: -1, 16, -30, 16, -1 over offsets -2..2 in each dimension, / (12 h^2);
-      // 8th order: -9, 128, -1008, 8064, -14350, ... over -4..4, / (5040 h^2)
-      // sm = sum over the 6 neighbours at distance m, in FMA form (bitwise the plain sums)
-      auto ring = [&](int m) {
-        return fadd(fadd(fadd(u[o - m], u[o + m], K), fadd(u[o - m * sy], u[o + m * sy], K), K),
-                    fadd(u[o - m * sz], u[o + m * sz], K), K);
-      };
-      const double s1 = ring(1), s2 = ring(2);
-      double lap;
-      if (ORD == 4) {
-        lap = fmul(fma(-90.0, u0, fma(16.0, s1, -s2)), inv12h2, K);
-      } else {
-        const double s3 = ring(3), s4 = ring(4);
-        lap = fmul(fma(-43050.0, u0, fma(8064.0, s1, fma(-1008.0, s2, fma(128.0, s3, fmul(-9.0, s4, K))))), inv12h2,
-                   K);
+      const double* u = a.Y + o;
+      const double u0 = u[0];
+      // sm = sum over the 6 neighbours at distance m; 4th order: 16 s1 - s2 - 90 u0 over
+      // 12 h^2, 8th order: 8064 s1 - 1008 s2 + 128 s3 - 9 s4 - 43050 u0 over 5040 h^2; in
+      // aligned integers (sc_fixed.cuh), or in FP64 where the values do not allow that
+      constexpr int R = ORD / 2;
+      double v[R][6];
+      int E = fx_exp(u0);
+#pragma unroll
+      for (int m = 0; m < R; ++m) {
+        v[m][0] = u[-(m + 1)];
+        v[m][1] = u[m + 1];
+        v[m][2] = u[-(m + 1) * sy];
+        v[m][3] = u[(m + 1) * sy];
+        v[m][4] = u[-(m + 1) * sz];
+        v[m][5] = u[(m + 1) * sz];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) E = max(E, fx_exp(v[m][q]));
       }
+      double lap;
+      if (aligned_ok(E)) {
+        using F = FxSums<ORD>;
+        typename F::Val s[R];
+#pragma unroll
+        for (int m = 0; m < R; ++m) {
+          s[m] = F::val(v[m][0], E);
+#pragma unroll
+          for (int q = 1; q < 6; ++q) s[m] += F::val(v[m][q], E);
+        }
+        lap = F::laplacian(s, F::val(u0, E), E);
+      } else {
+        double s[4];
+#pragma unroll
+        for (int m = 0; m < R; ++m) s[m] = ((v[m][0] + v[m][1]) + (v[m][2] + v[m][3])) + (v[m][4] + v[m][5]);
+        if (ORD == 4) lap = fma(-90.0, u0, fma(16.0, s[0], -s[1]));
+        else lap = fma(-43050.0, u0, fma(8064.0, s[0], fma(-1008.0, s[1], fma(128.0, s[2], -9.0 * s[3]))));
+      }
+      lap = fmul(lap, inv12h2, K);
       const double ku = a.Y[a.fs + o];  // d_t u = Pi
       const double kp = lap;            // d_t Pi = Laplacian u
       a.k[o] = ku;

@@ -5,13 +5,14 @@
 // clock, on two pipes that run side by side, beside FP64 instructions too).  A
 // finite-difference stencil has small integer weights, so its sum needs no
 // floating point until the end: the stencil's values are aligned to the
-// exponent of the largest of them, as signed integers with 2 (4th order) or 9
+// exponent of the largest of them, as signed integers with 2 (4th order) or 6
 // (8th order) bits below that value's last place, summed exactly, and the sum
 // is rounded once on its way back to FP64.  The alignment drops what lies
-// below 2^-54 (2^-61) of the stencil's own largest value, always downwards, so
-// that its mean cancels in sums whose weights add up to zero; everything else
-// is exact.  A chain of FP64 additions instead rounds every partial sum at
-// 2^-53 of its size, which the weights make several times the largest value.
+// below 2^-54 (2^-58) of the stencil's own largest value, always downwards, so
+// that its mean cancels in sums whose weights add up to zero; the halves of an
+// 8th-order sum are joined at 2^-47 of its largest term or less.  A chain of FP64
+// additions instead rounds every partial sum at 2^-53 of its size, which the
+// weights make several (8th order: thousands of) times the largest value.
 // The result depends on the stencil's values alone, not on tiles or boxes.
 //
 // Stencils that hold an infinity or a NaN, or whose largest value lies near
@@ -69,33 +70,25 @@ __device__ __forceinline__ double fx_back(long long X, int E) {
   return __hiloint2double(h ? h + (E - ((1075 + GUARD - SHIFT) << 20)) : 0, __double2loint(d));
 }
 
-// 8th order: weights up to 14350 (sum of magnitudes 2^15) do not fit beside a
-// 53-bit value in 64 bits, so the aligned value is cut into four 16-bit limbs
-// (the highest signed) and every limb is summed in 32 bits by itself:
-// 65535 * 2^14 (the weights of either sign) stays below 2^30.
-struct Limbs {
-  int l[4];
+// 8th order: weighted sums (sums of weight magnitudes up to 98304) do not fit
+// beside a 59-bit value in 64 bits, so the terms are cut into a low half, taken as
+// signed, and a high half, and each half is summed by 32 x 32 + 64 bit
+// multiply-adds: two instructions a term.  (Four 16-bit limbs summed in 32 bits
+// took eight: the pass over 262,144 cells ran in 0.385 ms.)
+struct FxWide {
+  long long hh = 0, ll = 0;
+  __device__ __forceinline__ void add(int w, long long x) {
+    int l, h;
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(l), "=r"(h) : "l"(x));
+    hh += (long long)w * (h + (int)((unsigned)l >> 31));
+    ll += (long long)w * l;
+  }
+  // in units of 2^SHIFT, rounded down
+  template <int SHIFT>
+  __device__ __forceinline__ long long get() const {
+    return (hh << (32 - SHIFT)) + (ll >> SHIFT);
+  }
 };
-__device__ __forceinline__ Limbs fx_limbs(long long x) {
-  const unsigned lo = (unsigned)x;
-  const int hi = (int)(x >> 32);
-  return Limbs{{(int)(lo & 0xffffu), (int)(lo >> 16), (int)((unsigned)hi & 0xffffu), hi >> 16}};
-}
-__device__ __forceinline__ Limbs operator+(const Limbs& a, const Limbs& b) {
-  return Limbs{{a.l[0] + b.l[0], a.l[1] + b.l[1], a.l[2] + b.l[2], a.l[3] + b.l[3]}};
-}
-__device__ __forceinline__ Limbs operator-(const Limbs& a, const Limbs& b) {
-  return Limbs{{a.l[0] - b.l[0], a.l[1] - b.l[1], a.l[2] - b.l[2], a.l[3] - b.l[3]}};
-}
-// The limb sums as one integer in units of 2^SHIFT (rounded down), SHIFT <= 15:
-// 16 bits of each limb below the next one's place, then the carries added.
-template <int SHIFT>
-__device__ __forceinline__ long long fx_join(const Limbs& s) {
-  long long X = (long long)s.l[1] * (1 << (16 - SHIFT)) + (s.l[0] >> SHIFT);
-  X += ((long long)s.l[2] << (32 - SHIFT));
-  X += ((long long)s.l[3] << (48 - SHIFT));
-  return X;
-}
 
 // The stencil sums of one order.  lo[m - 1], hi[m - 1] are the values at -m, m.
 template <int ORD>
@@ -114,6 +107,10 @@ struct FxSums<4> {
   __device__ static __forceinline__ double second(const Val* p, Val u0, int E) {
     return fx_back<kGuard, 0>((p[0] << 4) - p[1] - ((u0 << 5) - (u0 << 1)), E);
   }
+  // the three second derivatives' sum, Pm the sum over the six neighbours at distance m (weights: 192)
+  __device__ static __forceinline__ double laplacian(const Val* P, Val u0, int E) {
+    return fx_back<kGuard, 0>((P[0] << 4) - P[1] - 90 * u0, E);
+  }
   // P3 - 6 P2 + 15 P1 - 60 u0, Pm the sum over the six neighbours at distance m
   __device__ static __forceinline__ double ko(Val P1, Val P2, Val P3, Val u0, int E) {
     const Val u60 = (u0 << 6) - (u0 << 2);
@@ -123,30 +120,46 @@ struct FxSums<4> {
 
 template <>
 struct FxSums<8> {
-  static constexpr int kGuard = 9;
-  using Val = Limbs;
-  __device__ static __forceinline__ Val val(double v, int E) { return fx_limbs(fx_align(fx_unpack<kGuard>(v), E)); }
+  static constexpr int kGuard = 6;  // 59 bits: sums of six values and their halves stay in range
+  using Val = long long;
+  __device__ static __forceinline__ Val val(double v, int E) { return fx_align(fx_unpack<kGuard>(v), E); }
   // 672 d1 - 168 d2 + 32 d3 - 3 d4 = 840 h u', dm = v_m - v_-m (weights: 1750 < 2^11)
   __device__ static __forceinline__ double first(const Val* lo, const Val* hi, int E) {
-    Val s;
-    const Val d1 = hi[0] - lo[0], d2 = hi[1] - lo[1], d3 = hi[2] - lo[2], d4 = hi[3] - lo[3];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) s.l[i] = 672 * d1.l[i] - 168 * d2.l[i] + 32 * d3.l[i] - 3 * d4.l[i];
-    return fx_back<kGuard, 11>(fx_join<11>(s), E);
+    FxWide s;
+    s.add(672, hi[0] - lo[0]);
+    s.add(-168, hi[1] - lo[1]);
+    s.add(32, hi[2] - lo[2]);
+    s.add(-3, hi[3] - lo[3]);
+    return fx_back<kGuard, 8>(s.get<8>(), E);
   }
   // 8064 p1 - 1008 p2 + 128 p3 - 9 p4 - 14350 u0 = 5040 h^2 u'' (weights: 2^15)
-  __device__ static __forceinline__ double second(const Val* p, const Val& u0, int E) {
-    Val s;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      s.l[i] = 8064 * p[0].l[i] - 1008 * p[1].l[i] + 128 * p[2].l[i] - 9 * p[3].l[i] - 14350 * u0.l[i];
-    return fx_back<kGuard, 15>(fx_join<15>(s), E);
+  __device__ static __forceinline__ double second(const Val* p, Val u0, int E) {
+    FxWide s;
+    s.add(8064, p[0]);
+    s.add(-1008, p[1]);
+    s.add(128, p[2]);
+    s.add(-9, p[3]);
+    s.add(-14350, u0);
+    return fx_back<kGuard, 12>(s.get<12>(), E);
   }
-  __device__ static __forceinline__ double ko(const Val& P1, const Val& P2, const Val& P3, const Val& u0, int E) {
-    Val s;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) s.l[i] = 15 * P1.l[i] - 6 * P2.l[i] + P3.l[i] - 60 * u0.l[i];
-    return fx_back<kGuard, 8>(fx_join<8>(s), E);
+  // the three second derivatives' sum, Pm the sum over the six neighbours at distance m (weights: 98304)
+  __device__ static __forceinline__ double laplacian(const Val* P, Val u0, int E) {
+    FxWide s;
+    s.add(8064, P[0]);
+    s.add(-1008, P[1]);
+    s.add(128, P[2]);
+    s.add(-9, P[3]);
+    s.add(-43050, u0);
+    return fx_back<kGuard, 14>(s.get<14>(), E);
+  }
+  // (weights: 192)
+  __device__ static __forceinline__ double ko(Val P1, Val P2, Val P3, Val u0, int E) {
+    FxWide s;
+    s.add(15, P1);
+    s.add(-6, P2);
+    s.add(1, P3);
+    s.add(-60, u0);
+    return fx_back<kGuard, 5>(s.get<5>(), E);
   }
 };
 
