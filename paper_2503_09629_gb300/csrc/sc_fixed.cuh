@@ -62,6 +62,29 @@ __device__ __forceinline__ long long fx_align(const Fx& f, int E) {
 // exponent stays inside the normal range whatever the sum.
 __device__ __forceinline__ bool aligned_ok(int E) { return (unsigned)(E - (120 << 20)) <= (unsigned)(1880 << 20); }
 
+// A value that several stencils will read, unpacked once: the signed mantissa in
+// the high 54 bits, and in the low 10 the exponent less 512 (0 for what is
+// smaller, 1023 for what is larger, an infinity or a NaN).
+__device__ __forceinline__ long long fx_pack(double v) {
+  const int h = __double2hiint(v);
+  const unsigned l = (unsigned)__double2loint(v);
+  const int t = min(max(((h >> 20) & 0x7ff) - 512, 0), 1023);
+  const unsigned mh = (unsigned)((h & 0xfffff) | 0x100000);
+  const long long x = (long long)(((unsigned long long)__funnelshift_l(l, mh, 10) << 32) | (l << 10)), s = h >> 31;
+  return ((x ^ s) - s) | t;
+}
+__device__ __forceinline__ int fx_pexp(long long p) { return (int)p & 1023; }
+// The same as fx_align(fx_unpack<GUARD>) of a packed value.
+template <int GUARD>
+__device__ __forceinline__ long long fx_palign(long long p, int E) {
+  long long r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(p & ~1023ll), "r"(E + (10 - GUARD) - fx_pexp(p)));
+  return r;
+}
+// As aligned_ok, for the largest packed exponent of a stencil.
+__device__ __forceinline__ bool packed_ok(int E) { return (unsigned)(E - 120) <= 902u; }
+__device__ __forceinline__ int packed_field(int E) { return (E + 512) << 20; }
+
 // X units of 2^(exponent of E - 52 - GUARD + SHIFT), rounded to FP64.
 template <int GUARD, int SHIFT>
 __device__ __forceinline__ double fx_back(long long X, int E) {

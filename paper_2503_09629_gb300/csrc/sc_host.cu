@@ -253,11 +253,13 @@ struct Level {
   // work lists (device) and their sizes
   Tile* tiles = nullptr;
   int ntiles = 0;
-  int tile_cols = 0;                // largest nx * ny of the tiles
   std::vector<int> box_tile_begin;  // tiles of box b: [box_tile_begin[b], box_tile_begin[b + 1])
   CellRun* runs = nullptr;          // the pointwise Z4c kernel's units (one cell per thread)
   int nruns = 0;
   std::vector<int> box_run_begin;
+  Tile* dtiles = nullptr;           // tiles of the Z4c derivative pass
+  int ndtiles = 0;
+  std::vector<int> box_dtile_begin;
   AmrCell* amr = nullptr;
   int namr = 0;
   AmrTile* atiles = nullptr;  // separable-prolongation tiles and their position -> AMR index map
@@ -455,6 +457,7 @@ sc_status validate(const sc_desc* d) {
 struct HostLists {
   std::vector<Tile> tiles;
   std::vector<CellRun> runs;
+  std::vector<Tile> dtiles;
   std::vector<AmrCell> amr;
   std::vector<int> amr_gi, amr_gw;  // unwrapped / wrapped global fine index per AMR cell
   std::vector<AmrTile> atiles;      // slab tiles served by the separable kernel
@@ -656,12 +659,6 @@ void build_amr_tiles(sc_ctx* c, int l, HostLists& hl) {
 
 // Interior tiles of the stencil kernels: per box, tiles of shape tile[0..2]
 // clipped to the box (ragged tiles at the high ends).
-int max_tile_cols(const std::vector<Tile>& v) {
-  int m = 1;
-  for (const Tile& t : v) m = std::max(m, t.nx * t.ny);
-  return m;
-}
-
 void build_stencil_tiles(Level& L, const int* tile, std::vector<Tile>& out) {
   const Geom& g = L.g;
   out.clear();
@@ -682,7 +679,46 @@ void build_stencil_tiles(Level& L, const int* tile, std::vector<Tile>& out) {
         }
   }
   L.box_tile_begin.push_back((int)out.size());
-  L.tile_cols = max_tile_cols(out);
+}
+
+// Tiles of the Z4c derivative pass for the boxes of a level: the width splits
+// a box's rows evenly, the height fills a block of threads, and the depth is
+// as large as still gives every SM a few (tile, field) items, between 4 planes
+// and 16 (a block reads 6 or 8 planes more than it computes).
+void build_deriv_tiles(const Geom& g, const sc_box* boxes, size_t nboxes, std::vector<Tile>& out,
+                       std::vector<int>& begin) {
+  auto parts = [](int n, int most) { return (n + most - 1) / most; };
+  auto even = [&](int n, int most) { return parts(n, parts(n, most)); };  // the extent that splits n evenly
+  long columns = 0;                                                       // tiles if all were of full depth
+  for (size_t b = 0; b < nboxes; ++b) {
+    const sc_box& B = boxes[b];
+    const int nx = B.hi[0] - B.lo[0] + 1, ny = B.hi[1] - B.lo[1] + 1;
+    const int tx = even(nx, 32), ty = even(ny, std::min(32, kDerivCols / tx));
+    columns += (long)parts(nx, tx) * parts(ny, ty) * (B.hi[2] - B.lo[2] + 1);
+  }
+  int depth = 16;
+  while (depth > 4 && columns / depth * kNZ4c < 4L * sm_count() * 3) depth /= 2;
+  out.clear();
+  begin.clear();
+  for (size_t b = 0; b < nboxes; ++b) {
+    begin.push_back((int)out.size());
+    const sc_box& B = boxes[b];
+    const int n[3] = {B.hi[0] - B.lo[0] + 1, B.hi[1] - B.lo[1] + 1, B.hi[2] - B.lo[2] + 1};
+    const int tx = even(n[0], 32), ty = even(n[1], std::min(32, kDerivCols / tx)), tz = even(n[2], depth);
+    for (int z = 0; z < n[2]; z += tz)
+      for (int y = 0; y < n[1]; y += ty)
+        for (int x = 0; x < n[0]; x += tx) {
+          Tile t;
+          t.x0 = B.lo[0] + x - g.org[0];
+          t.y0 = B.lo[1] + y - g.org[1];
+          t.z0 = B.lo[2] + z - g.org[2];
+          t.nx = std::min(tx, n[0] - x);
+          t.ny = std::min(ty, n[1] - y);
+          t.nz = std::min(tz, n[2] - z);
+          out.push_back(t);
+        }
+  }
+  begin.push_back((int)out.size());
 }
 
 sc_status classify_level(sc_ctx* c, int l, HostLists& hl) {
@@ -765,9 +801,11 @@ sc_status classify_level(sc_ctx* c, int l, HostLists& hl) {
       }
   if (l > 0 && !hl.amr.empty()) build_amr_tiles(c, l, hl);
   build_stencil_tiles(L, c->tile, hl.tiles);
+  if (c->system == SC_Z4C) build_deriv_tiles(g, L.boxes.data(), L.boxes.size(), hl.dtiles, L.box_dtile_begin);
   // Runs of cells of the Z4c stage kernel, one cell per thread.
   L.box_run_begin.clear();
   for (const sc_box& B : L.boxes) {
+    if (c->system != SC_Z4C) break;
     L.box_run_begin.push_back((int)hl.runs.size());
     CellRun r;
     r.off = (int32_t)g.off(B.lo[0], B.lo[1], B.lo[2]);
@@ -911,13 +949,15 @@ sc_status setup_level_device(sc_ctx* c, int l, HostLists& hl) {
       (st = level_upload(c, L, hl.periodic, &L.periodic)) || (st = level_upload(c, L, hl.phys, &L.phys)) ||
       (st = level_upload(c, L, hl.restr, &L.restr)) || (st = level_upload(c, L, hl.rblocks, &L.rblocks)) ||
       (st = level_upload(c, L, hl.atiles, &L.atiles)) || (st = level_upload(c, L, hl.aslots, &L.aslots)) ||
-      (st = level_upload(c, L, hl.dxy, &L.dxy)) || (st = level_upload(c, L, hl.runs, &L.runs)))
+      (st = level_upload(c, L, hl.dxy, &L.dxy)) || (st = level_upload(c, L, hl.runs, &L.runs)) ||
+      (st = level_upload(c, L, hl.dtiles, &L.dtiles)))
     return st;
   L.ntiles = (int)hl.tiles.size();
   L.namr = (int)hl.amr.size();
   L.natiles = (int)hl.atiles.size();
   L.tile_fmas = hl.tile_fmas;
   L.nruns = (int)hl.runs.size();
+  L.ndtiles = (int)hl.dtiles.size();
   L.ndxy = (int)hl.dxy.size();
   L.namr_blocked = hl.namr_blocked;
   L.nperiodic = (int)hl.periodic.size();
@@ -1177,12 +1217,13 @@ sc_status run_op(sc_ctx* c, const Op& o, cudaStream_t s) {
         if (c->system == SC_WAVE) {
           CU(launch_wave_stage(a, L.tiles + t0, nt, s, c->order, foldp));
         } else {
+          const int d0 = nparts == 1 ? 0 : L.box_dtile_begin[b];
+          const int nd = nparts == 1 ? L.ndtiles : L.box_dtile_begin[b + 1] - d0;
           const int p0 = nparts == 1 ? 0 : L.box_run_begin[b];
           const int np = nparts == 1 ? L.nruns : L.box_run_begin[b + 1] - p0;
           if (one_pass) CU(launch_z4c_derivs(a.Y, c->scratch, g.fs, a.sy, a.sz, L.tiles + t0, nt, s));
           else
-            CU(launch_z4c_derivs_split(a.Y, c->scratch, g.fs, a.sy, a.sz, L.tiles + t0, nt, s, c->order,
-                                       L.tile_cols));
+            CU(launch_z4c_derivs_split(a.Y, c->scratch, g.fs, a.sy, a.sz, L.dtiles + d0, nd, s, c->order));
           CU(launch_z4c_stage(a, c->scratch, c->zp, L.runs + p0, np, s, c->stage_bps));
         }
       }
@@ -1594,7 +1635,7 @@ StageArgs tuning_stage_args(const Level& L, int order) {
 // (one untimed launch first, then reps): kind 0 = the stencil kernel with the
 // given tiles (the wave's fused stage, or the Z4c derivative pass in the form
 // deriv_form), kind 1 = the Z4c stage kernel built for bps blocks per SM.
-sc_status time_candidate(sc_ctx* c, Level& L, int kind, const Tile* tiles, int ntiles, int cols, int deriv_form,
+sc_status time_candidate(sc_ctx* c, Level& L, int kind, const Tile* tiles, int ntiles, int deriv_form,
                          int bps, int reps, double* ms) {
   const Geom& g = L.g;
   const StageArgs a = tuning_stage_args(L, c->order);
@@ -1611,7 +1652,7 @@ sc_status time_candidate(sc_ctx* c, Level& L, int kind, const Tile* tiles, int n
       CU(launch_z4c_derivs(a.Y, c->scratch, g.fs, a.sy, a.sz, tiles, ntiles, c->stream));
     } else {
       CU(launch_z4c_dxy(a.Y, c->scratch, g.fs, a.sy, L.dxy, L.ndxy, c->stream, c->order));
-      CU(launch_z4c_derivs_split(a.Y, c->scratch, g.fs, a.sy, a.sz, tiles, ntiles, c->stream, c->order, cols));
+      CU(launch_z4c_derivs_split(a.Y, c->scratch, g.fs, a.sy, a.sz, L.dtiles, L.ndtiles, c->stream, c->order));
     }
   }
   CU(cudaEventRecord(e1, c->stream));
@@ -1641,7 +1682,6 @@ sc_status apply_tuning(sc_ctx* c, const int* shape, int deriv_form, int bps) {
     }
     L.tiles = d;
     L.ntiles = (int)t.size();
-    L.tile_cols = max_tile_cols(t);
   }
   CU(cudaStreamSynchronize(c->stream));
   return build_graphs(c, false);
@@ -1685,7 +1725,8 @@ extern "C" sc_status sc_autotune(sc_ctx* c, int* tile_out, double* ms_out) {
     std::vector<void*> scratch_lists;
     for (int form = 0; form < nform; ++form)
       for (const auto& cd : cand) {
-        if (form == 1 && (cd[0] != 32 || cd[1] != 4 || cd[2] != 2)) continue;  // one-kernel form: default tiles
+        // Z4c: the two-kernel form has tiles of its own, the one-kernel form takes the default ones
+        if (c->system == SC_Z4C && (cd[0] != 32 || cd[1] != 4 || cd[2] != 2)) continue;
         build_stencil_tiles(L, cd, t);
         if (t.size() > cap) {
           cap = t.size() * 2;
@@ -1695,7 +1736,7 @@ extern "C" sc_status sc_autotune(sc_ctx* c, int* tile_out, double* ms_out) {
         }
         CU(cudaMemcpyAsync(d, t.data(), t.size() * sizeof(Tile), cudaMemcpyHostToDevice, c->stream));
         double ms = 0;
-        sc_status st = time_candidate(c, L, 0, d, (int)t.size(), max_tile_cols(t), form, 0, 3, &ms);
+        sc_status st = time_candidate(c, L, 0, d, (int)t.size(), form, 0, 3, &ms);
         if (st) return st;
         if (best_ms < 0 || ms < best_ms) {
           best_ms = ms;
@@ -1704,8 +1745,8 @@ extern "C" sc_status sc_autotune(sc_ctx* c, int* tile_out, double* ms_out) {
       }
     if (c->system == SC_Z4C) {
       double ms2 = 0, ms3 = 0;
-      sc_status st = time_candidate(c, L, 1, nullptr, 0, 0, 0, 2, 3, &ms2);
-      if (!st) st = time_candidate(c, L, 1, nullptr, 0, 0, 0, 3, 3, &ms3);
+      sc_status st = time_candidate(c, L, 1, nullptr, 0, 0, 2, 3, &ms2);
+      if (!st) st = time_candidate(c, L, 1, nullptr, 0, 0, 3, 3, &ms3);
       if (st) return st;
       best[4] = ms2 < ms3 ? 2 : 3;
     }
@@ -2344,8 +2385,8 @@ sc_status sc_get_constraints(sc_ctx* c, int level, int box, double* dst) {
     CU(launch_z4c_derivs(Y, c->scratch, L.g.fs, sy, sz, dt, (int)tl.size(), c->stream));
   } else {
     CU(launch_z4c_dxy(Y, c->scratch, L.g.fs, sy, L.dxy, L.ndxy, c->stream, c->order));
-    CU(launch_z4c_derivs_split(Y, c->scratch, L.g.fs, sy, sz, dt, (int)tl.size(), c->stream, c->order,
-                               max_tile_cols(tl)));
+    CU(launch_z4c_derivs_split(Y, c->scratch, L.g.fs, sy, sz, L.dtiles + L.box_dtile_begin[box],
+                               L.box_dtile_begin[box + 1] - L.box_dtile_begin[box], c->stream, c->order));
   }
   CU(launch_z4c_constraints(Y, c->scratch, c->staging, L.g.fs, sy, sz, c->zp, deriv_scales(c->order, L.g.h), dt, (int)tl.size(), ncell, blo, n,
                             c->stream));
@@ -2406,8 +2447,7 @@ sc_status sc_time_stage_kernels(sc_ctx* c, int level, int nrep, double* ms) {
       CU(launch_z4c_derivs(a.Y, c->scratch, g.fs, a.sy, a.sz, L.tiles, L.ntiles, c->stream));
     else {
       CU(launch_z4c_dxy(a.Y, c->scratch, g.fs, a.sy, L.dxy, L.ndxy, c->stream, c->order));
-      CU(launch_z4c_derivs_split(a.Y, c->scratch, g.fs, a.sy, a.sz, L.tiles, L.ntiles, c->stream, c->order,
-                                 L.tile_cols));
+      CU(launch_z4c_derivs_split(a.Y, c->scratch, g.fs, a.sy, a.sz, L.dtiles, L.ndtiles, c->stream, c->order));
     }
   }
   CU(cudaEventRecord(e[1], c->stream));
@@ -2432,7 +2472,7 @@ sc_status sc_run_op_class_pass(sc_ctx* c, int level) {
   const Geom& g = L.g;
   const StageArgs a = tuning_stage_args(L, c->order);
   CU(launch_z4c_dxy(a.Y, c->scratch, g.fs, a.sy, L.dxy, L.ndxy, c->stream, c->order));
-  CU(launch_z4c_derivs_split(a.Y, c->scratch, g.fs, a.sy, a.sz, L.tiles, L.ntiles, c->stream, c->order, L.tile_cols));
+  CU(launch_z4c_derivs_split(a.Y, c->scratch, g.fs, a.sy, a.sz, L.dtiles, L.ndtiles, c->stream, c->order));
   CU(launch_z4c_stage(a, c->scratch, c->zp, L.runs, L.nruns, c->stream, c->stage_bps, true));
   CU(cudaStreamSynchronize(c->stream));
   return SC_OK;

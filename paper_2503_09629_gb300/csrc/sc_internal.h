@@ -50,6 +50,7 @@ struct CellRun {
   int32_t first, n;
 };
 constexpr int kRunCells = 64;
+constexpr int kDerivCols = 256;  // columns of a tile of the Z4c derivative pass
 
 // Refinement-boundary ghost cell: destination offset in the fine array,
 // offset of the first parent stencil cell in the parent array, parity of
@@ -240,10 +241,9 @@ cudaError_t z4c_init_launch_config();
 // order: finite-difference order of the derivatives, 4 or 8 (Kreiss-Oliger stays r = 4).
 cudaError_t launch_z4c_dxy(const double* Y, double* scratch, long fs, int sy, const RowSeg* segs, int nsegs,
                            cudaStream_t s, int order = 4);
-// max_cols: the largest nx * ny of the tiles (work is dealt out per tile in
-// chunks sized by it); cudaErrorInvalidValue if below 1.
+// tiles: of a deriv_tiles list (at most kDerivCols columns, 32 wide, 32 high).
 cudaError_t launch_z4c_derivs_split(const double* Y, double* scratch, long fs, int sy, int sz,
-                                    const Tile* tiles, int ntiles, cudaStream_t s, int order, int max_cols);
+                                    const Tile* tiles, int ntiles, cudaStream_t s, int order);
 // bps: warps per scheduler that the stage kernel's build leaves registers for, 2
 // or 3 (a tuning choice); cudaErrorInvalidValue otherwise.  op_class: the PlainK
 // build (stage form kStageSingle only, cudaErrorInvalidValue for the others).

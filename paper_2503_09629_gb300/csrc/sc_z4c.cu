@@ -111,8 +111,14 @@ __device__ __forceinline__ int d2_field(int s) { return s <= 6 ? s : s + 11; }
 
 // Centred first derivative as the integer-weight sum, lo[m - 1] = v_-m, hi[m - 1] = v_m:
 // 4th order 8 (v_1 - v_-1) - (v_2 - v_-2) (= 12 h u'), 8th order
-// 672 d1 - 168 d2 + 32 d3 - 3 d4 (= 840 h u'), dm = v_m - v_-m; in aligned
-// integers (sc_fixed.cuh), or in FP64 where the values do not allow that.
+// 672 d1 - 168 d2 + 32 d3 - 3 d4 (= 840 h u'), dm = v_m - v_-m, in FP64.
+template <int ORD>
+__device__ __forceinline__ double dfirst_fp64(const double* lo, const double* hi) {
+  if (ORD == 4) return fma(8.0, hi[0], fma(-8.0, lo[0], lo[1] - hi[1]));
+  return fma(672.0, hi[0] - lo[0], fma(-168.0, hi[1] - lo[1], fma(32.0, hi[2] - lo[2], -3.0 * (hi[3] - lo[3]))));
+}
+
+// The same in aligned integers (sc_fixed.cuh), or in FP64 where the values do not allow that.
 template <int ORD>
 __device__ __forceinline__ double dfirst(const double* lo, const double* hi) {
   using F = FxSums<ORD>;
@@ -129,8 +135,7 @@ __device__ __forceinline__ double dfirst(const double* lo, const double* hi) {
     }
     return F::first(l, h, E);
   }
-  if (ORD == 4) return fma(8.0, hi[0], fma(-8.0, lo[0], lo[1] - hi[1]));
-  return fma(672.0, hi[0] - lo[0], fma(-168.0, hi[1] - lo[1], fma(32.0, hi[2] - lo[2], -3.0 * (hi[3] - lo[3]))));
+  return dfirst_fp64<ORD>(lo, hi);
 }
 
 template <int ORD>
@@ -194,145 +199,190 @@ __device__ __forceinline__ void cell_sums_fp64(double u0, const double (*lo)[ORD
   *ko = fma(15.0, P[0], fma(-6.0, P[1], fma(-60.0, u0, P[2])));
 }
 
+// One block per (tile, field): a thread per (x, y) column walks z with the
+// packed values at z-W..z+W in registers (W = max(R, 3), R = ORD/2 the derivative
+// radius, 3 the Kreiss-Oliger radius) and puts its centre value, and up to two
+// of the tile's halo cells, into a shared plane, so that a value is unpacked once
+// or twice instead of 19 (25) times.  Tiles: at most kDerivCols columns, 32 wide,
+// 32 high; a plane then holds at most 38 x 14 (40 x 16) values.  At 4th order D_x
+// and D_y along z are windows in registers too; at 8th order these would spill,
+// and are read again (L1).  Integer ALU 45%, latency of 16 warps: 262,144 cells with
+// the row pass before it, 0.251 ms with a thread per column and no sharing, 0.197
+// so; 110,592 cells 0.119 and 0.104; 8th order, 262,144 cells, 0.347 and 0.332.  With
+// the mixed derivatives in FP64 instead: 0.211 and 0.444; with three or four blocks
+// per SM and reads in place of the windows: 0.219 and 0.238.
 template <int ORD>
-__global__ void __launch_bounds__(kThreads, 2) z4c_derivs_split_kernel(const double* __restrict__ Y,
-                                                                      double* __restrict__ S, long fs, int sy_,
-                                                                      int sz_, const Tile* __restrict__ tiles, int ntiles,
-                                                                      int max_cols) {
-  // One thread per (x, y, field) column of a tile, walking z with sliding
-  // windows: u at z-W..z+W (W = max(R, 3), R = ORD/2 the derivative radius,
-  // 3 the Kreiss-Oliger radius) and, for the Hessian fields, the stored
-  // D_x, D_y at z-R..z+R, so each step loads one new z value per window.
-  // Work is dealt out in units of (tile, chunk of blockDim (field, column)
-  // pairs), U chunks per tile (max_cols = the largest tile's columns), so
-  // the persistent blocks end together whatever the tile count.
+__global__ void __launch_bounds__(kDerivCols, 2)
+    z4c_derivs_split_kernel(const double* __restrict__ Y, double* __restrict__ S, long fs, int sy_, int sz_,
+                            const Tile* __restrict__ tiles, int ntiles) {
   using F = FxSums<ORD>;
   constexpr int R = ORD / 2;
   constexpr int WR = R > 3 ? R : 3;
   constexpr int NW = 2 * WR + 1;
   constexpr int ND = 2 * R + 1;
+  constexpr int G = F::kGuard;
+  constexpr bool kWindows = ORD == 4;
+  __shared__ long long planes[2][(32 + 2 * WR) * (8 + 2 * WR)];
   const long sy = sy_, sz = sz_;
-  const int U = (max_cols * kNZ4c + blockDim.x - 1) / blockDim.x;
-  for (long u = blockIdx.x; u < (long)ntiles * U; u += gridDim.x) {
-    const int t = (int)(u / U);
+  int buf = 0;
+  for (int item = blockIdx.x; item < ntiles * kNZ4c; item += gridDim.x) {
+    const int t = item / kNZ4c, f = item - t * kNZ4c;
     const Tile T = tiles[t];
-    const int ncol = T.nx * T.ny;
-    const int q = (int)(u - (long)t * U) * blockDim.x + threadIdx.x;
-    if (q < ncol * kNZ4c) {
-      const int f = q / ncol;
-      const int c = q - f * ncol;
-      const int i = c % T.nx;
-      const int j = c / T.nx;
-      const long o0 = (long)T.z0 * sz + (T.y0 + j) * sy + (T.x0 + i);
-      const double* u = Y + (long)f * fs + o0;
-      const int sl = d2_slot(f);
-      double w[NW];  // u at z-WR..z+WR
+    const int ncol = T.nx * T.ny, pitch = T.nx + 2 * WR;
+    const double* base = Y + (long)f * fs + (long)T.z0 * sz + (long)T.y0 * sy + T.x0;
+    const bool active = (int)threadIdx.x < ncol;
+    const int i = threadIdx.x % T.nx, j = threadIdx.x / T.nx;
+    const int own = (j + WR) * pitch + i + WR;
+    const double* u = base + (long)j * sy + i;
+    const long o0 = (long)T.z0 * sz + (long)(T.y0 + j) * sy + (T.x0 + i);
+    // halo cells of a plane: 2 WR per row, then 2 WR rows
+    int hs[2];
+    const double* hp[2];
 #pragma unroll
-      for (int m = 0; m < NW; ++m) w[m] = u[(m - WR) * sz];
-      const double* Dx = S + (long)(Q_D1 + 3 * f + 0) * fs + o0;
-      const double* Dy = S + (long)(Q_D1 + 3 * f + 1) * fs + o0;
-      double wx[ND], wy[ND];  // D_x, D_y at z-R..z+R (Hessian fields)
-      if (sl >= 0) {
+    for (int r = 0; r < 2; ++r) {
+      int h = threadIdx.x + r * kDerivCols, x, y;
+      hs[r] = -1;
+      hp[r] = base;
+      if (h < 2 * WR * (T.nx + T.ny)) {
+        if (h < 2 * WR * T.ny) {
+          y = h / (2 * WR);
+          x = h - y * (2 * WR);
+          x = x < WR ? x - WR : T.nx + x - WR;
+        } else {
+          h -= 2 * WR * T.ny;
+          y = h / T.nx;
+          x = h - y * T.nx;
+          y = y < WR ? y - WR : T.ny + y - WR;
+        }
+        hs[r] = (y + WR) * pitch + x + WR;
+        hp[r] += (long)y * sy + x;
+      }
+    }
+    const int sl = d2_slot(f);
+    const double* Dx = S + (long)(Q_D1 + 3 * f + 0) * fs + o0;
+    const double* Dy = S + (long)(Q_D1 + 3 * f + 1) * fs + o0;
+    long long w[NW];       // packed u at z-WR..z+WR
+    double wx[ND], wy[ND];  // kWindows: D_x, D_y at z-R..z+R (Hessian fields)
+    double hv[2] = {hs[0] >= 0 ? *hp[0] : 0.0, hs[1] >= 0 ? *hp[1] : 0.0};
+    double un = 0.0;
+    if (active) {
 #pragma unroll
-        for (int m = 0; m < ND; ++m) {
+      for (int m = 0; m < NW - 1; ++m) w[m] = fx_pack(u[(m - WR) * sz]);
+      un = u[WR * sz];
+      if (kWindows && sl >= 0) {
+#pragma unroll
+        for (int m = 0; m < ND - 1; ++m) {
           wx[m] = Dx[(m - R) * sz];
           wy[m] = Dy[(m - R) * sz];
         }
       }
-#pragma unroll(1)
-      for (int k = 0; k < T.nz; ++k) {
-        const long o = o0 + k * sz;
-        const double* v = u + k * sz;
-        const double u0 = w[WR];
-        // u along x and y from memory, along z from the window
-        double lo[3][WR], hi[3][WR];
-        int E = fx_exp(u0);
+    }
+#pragma unroll 1
+    for (int k = 0; k < T.nz; ++k, buf ^= 1) {
+      long long* pl = planes[buf];
+      if (active) pl[own] = w[WR];
+      const bool more = k + 1 < T.nz;
 #pragma unroll
-        for (int m = 1; m <= WR; ++m) {
-          lo[0][m - 1] = v[-m];
-          hi[0][m - 1] = v[m];
-          lo[1][m - 1] = v[-m * sy];
-          hi[1][m - 1] = v[m * sy];
-          lo[2][m - 1] = w[WR - m];
-          hi[2][m - 1] = w[WR + m];
+      for (int r = 0; r < 2; ++r)
+        if (hs[r] >= 0) {
+          pl[hs[r]] = fx_pack(hv[r]);
+          if (more) hv[r] = hp[r][(k + 1) * sz];
         }
+      // (the two planes alternate, also from one item to the next: a plane is
+      // written again only after every thread has passed the next barrier)
+      __syncthreads();
+      if (!active) continue;
+      w[NW - 1] = fx_pack(un);
+      if (more) un = u[(k + 1 + WR) * sz];
+      const long o = o0 + k * sz;
+      if (kWindows && sl >= 0) {
+        wx[ND - 1] = Dx[(k + R) * sz];
+        wy[ND - 1] = Dy[(k + R) * sz];
+      }
+      auto at = [&](int dim, int m) {
+        return dim == 0 ? pl[own + m] : dim == 1 ? pl[own + m * pitch] : w[WR + m];
+      };
+      int E = fx_pexp(w[WR]);
+#pragma unroll
+      for (int dim = 0; dim < 3; ++dim)
+#pragma unroll
+        for (int m = 1; m <= WR; ++m) E = max(E, max(fx_pexp(at(dim, -m)), fx_pexp(at(dim, m))));
+      double* d1 = S + (long)(Q_D1 + 3 * f) * fs + o;
+      double* d2 = S + (long)(Q_D2 + 6 * sl) * fs + o;
+      double* ko = S + (long)(Q_KO + f) * fs + o;
+      if (packed_ok(E)) {
+        // One alignment for every sum of the cell.
+        const int Ef = packed_field(E);
+        typename F::Val P[3];
+        const typename F::Val x0 = fx_palign<G>(w[WR], E);
+#pragma unroll
+        for (int dim = 0; dim < 3; ++dim) {
+          typename F::Val l[WR], h[WR], p[WR];
+#pragma unroll
+          for (int m = 0; m < WR; ++m) {
+            l[m] = fx_palign<G>(at(dim, -m - 1), E);
+            h[m] = fx_palign<G>(at(dim, m + 1), E);
+            p[m] = l[m] + h[m];
+          }
+          // D_x, D_y of the Hessian fields are there already (z4c_dxy_kernel)
+          if (sl < 0 || dim == 2) d1[dim * fs] = F::first(l, h, Ef);
+          if (sl >= 0) d2[(dim == 0 ? 0 : dim == 1 ? 3 : 5) * fs] = F::second(p, x0, Ef);
+#pragma unroll
+          for (int m = 0; m < 3; ++m) P[m] = dim == 0 ? p[m] : P[m] + p[m];
+        }
+        *ko = F::ko(P[0], P[1], P[2], x0, Ef);
+      } else {
+        const double* v = u + k * sz;
+        double fl[3][ORD == 4 ? 3 : 4], fh[3][ORD == 4 ? 3 : 4], e1[3], e2[3], eko;
+        const long st[3] = {1, sy, sz};
 #pragma unroll
         for (int dim = 0; dim < 3; ++dim)
 #pragma unroll
-          for (int m = 0; m < WR; ++m) E = max(E, max(fx_exp(lo[dim][m]), fx_exp(hi[dim][m])));
-        double* d1 = S + (long)(Q_D1 + 3 * f) * fs + o;
-        double* d2 = S + (long)(Q_D2 + 6 * sl) * fs + o;
-        double* ko = S + (long)(Q_KO + f) * fs + o;
-        if (aligned_ok(E)) {
-          // One alignment for every sum of the cell.
-          typename F::Val P[3];
-          const typename F::Val x0 = F::val(u0, E);
-#pragma unroll
-          for (int dim = 0; dim < 3; ++dim) {
-            typename F::Val l[WR], h[WR];
-#pragma unroll
-            for (int m = 0; m < WR; ++m) {
-              l[m] = F::val(lo[dim][m], E);
-              h[m] = F::val(hi[dim][m], E);
-            }
-            // D_x, D_y of the Hessian fields are there already (z4c_dxy_kernel)
-            if (sl < 0 || dim == 2) d1[dim * fs] = F::first(l, h, E);
-            typename F::Val p[WR];
-#pragma unroll
-            for (int m = 0; m < WR; ++m) p[m] = l[m] + h[m];
-            if (sl >= 0) d2[(dim == 0 ? 0 : dim == 1 ? 3 : 5) * fs] = F::second(p, x0, E);
-#pragma unroll
-            for (int m = 0; m < 3; ++m) P[m] = dim == 0 ? p[m] : P[m] + p[m];
+          for (int m = 1; m <= WR; ++m) {
+            fl[dim][m - 1] = v[-m * st[dim]];
+            fh[dim][m - 1] = v[m * st[dim]];
           }
-          *ko = F::ko(P[0], P[1], P[2], x0, E);
-        } else {
-          double e1[3], e2[3], eko;
-          cell_sums_fp64<ORD>(u0, lo, hi, e1, &eko, e2);
-          *ko = eko;
+        cell_sums_fp64<ORD>(v[0], fl, fh, e1, &eko, e2);
+        *ko = eko;
 #pragma unroll
-          for (int dim = 0; dim < 3; ++dim) {
-            if (sl < 0 || dim == 2) d1[dim * fs] = e1[dim];
-            if (sl >= 0) d2[(dim == 0 ? 0 : dim == 1 ? 3 : 5) * fs] = e2[dim];
-          }
-        }
-        if (sl >= 0) {
-          // mixed: the first-derivative stencil applied to the stored D_x (along y and z) and D_y (along z)
-          double ml[R], mh[R];
-          const double* dxk = Dx + k * sz;
-#pragma unroll
-          for (int m = 1; m <= R; ++m) {
-            ml[m - 1] = dxk[-m * sy];
-            mh[m - 1] = dxk[m * sy];
-          }
-          d2[1 * fs] = dfirst<ORD>(ml, mh);  // D_y D_x
-#pragma unroll
-          for (int m = 1; m <= R; ++m) {
-            ml[m - 1] = wx[R - m];
-            mh[m - 1] = wx[R + m];
-          }
-          d2[2 * fs] = dfirst<ORD>(ml, mh);  // D_z D_x
-#pragma unroll
-          for (int m = 1; m <= R; ++m) {
-            ml[m - 1] = wy[R - m];
-            mh[m - 1] = wy[R + m];
-          }
-          d2[4 * fs] = dfirst<ORD>(ml, mh);  // D_z D_y
-        }
-        if (k + 1 < T.nz) {  // slide the windows one cell up in z
-#pragma unroll
-          for (int m = 0; m < NW - 1; ++m) w[m] = w[m + 1];
-          w[NW - 1] = v[(WR + 1) * sz];
-          if (sl >= 0) {
-#pragma unroll
-            for (int m = 0; m < ND - 1; ++m) {
-              wx[m] = wx[m + 1];
-              wy[m] = wy[m + 1];
-            }
-            wx[ND - 1] = Dx[(k + 1 + R) * sz];
-            wy[ND - 1] = Dy[(k + 1 + R) * sz];
-          }
+        for (int dim = 0; dim < 3; ++dim) {
+          if (sl < 0 || dim == 2) d1[dim * fs] = e1[dim];
+          if (sl >= 0) d2[(dim == 0 ? 0 : dim == 1 ? 3 : 5) * fs] = e2[dim];
         }
       }
+      if (sl >= 0) {
+        // mixed: the first-derivative stencil applied to the stored D_x (along y and z) and D_y (along z)
+        auto mixed = [&](const double* d, long st) {
+          double ml[R], mh[R];
+#pragma unroll
+          for (int m = 1; m <= R; ++m) {
+            ml[m - 1] = d[-m * st];
+            mh[m - 1] = d[m * st];
+          }
+          return dfirst<ORD>(ml, mh);
+        };
+        d2[1 * fs] = mixed(Dx + k * sz, sy);
+        if (kWindows) {
+          auto window = [&](double* v) {
+            double ml[R], mh[R];
+#pragma unroll
+            for (int m = 1; m <= R; ++m) {
+              ml[m - 1] = v[R - m];
+              mh[m - 1] = v[R + m];
+            }
+#pragma unroll
+            for (int m = 0; m < ND - 1; ++m) v[m] = v[m + 1];
+            return dfirst<ORD>(ml, mh);
+          };
+          d2[2 * fs] = window(wx);
+          d2[4 * fs] = window(wy);
+        } else {
+          d2[2 * fs] = mixed(Dx + k * sz, sz);
+          d2[4 * fs] = mixed(Dy + k * sz, sz);
+        }
+      }
+#pragma unroll
+      for (int m = 0; m < NW - 1; ++m) w[m] = w[m + 1];
     }
   }
 }
@@ -840,7 +890,7 @@ __global__ void __launch_bounds__(128) z4c_constraints_kernel(const double* __re
 struct GridCaps {
   int ready = 0;
   int stage[4] = {608, 608, 608, 912};  // by warps per scheduler of the build (2 or 3)
-  int derivs = 1216, dxy = 2432;
+  int derivs[2] = {456, 304}, dxy = 2432;  // derivs: 4th, 8th order
 };
 GridCaps g_caps[64];
 
@@ -867,9 +917,12 @@ cudaError_t z4c_init_launch_config() {
       cudaSuccess)
     return e;
   c.stage[3] = nsm * (occ > 0 ? occ : 1);
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, z4c_derivs_split_kernel<8>, kThreads, 0)) != cudaSuccess)
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, z4c_derivs_split_kernel<4>, kDerivCols, 0)) != cudaSuccess)
     return e;
-  c.derivs = nsm * (occ > 0 ? occ : 1);
+  c.derivs[0] = nsm * (occ > 0 ? occ : 1);
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, z4c_derivs_split_kernel<8>, kDerivCols, 0)) != cudaSuccess)
+    return e;
+  c.derivs[1] = nsm * (occ > 0 ? occ : 1);
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, z4c_dxy_kernel<8>, 128, 0)) != cudaSuccess) return e;
   c.dxy = nsm * (occ > 0 ? occ : 1);
   c.ready = 1;
@@ -893,16 +946,14 @@ cudaError_t launch_z4c_dxy(const double* Y, double* scratch, long fs, int sy, co
   return cudaGetLastError();
 }
 
-cudaError_t launch_z4c_derivs_split(const double* Y, double* scratch, long fs, int sy, int sz,
-                                    const Tile* tiles, int ntiles, cudaStream_t s, int order, int max_cols) {
+cudaError_t launch_z4c_derivs_split(const double* Y, double* scratch, long fs, int sy, int sz, const Tile* tiles,
+                                    int ntiles, cudaStream_t s, int order) {
   if (ntiles == 0) return cudaSuccess;
-  if (max_cols < 1) return cudaErrorInvalidValue;
-  const long units = (long)ntiles * ((max_cols * kNZ4c + kThreads - 1) / kThreads);
-  const int grid = units < caps().derivs ? (int)units : caps().derivs;
-  if (order == 8)
-    z4c_derivs_split_kernel<8><<<grid, kThreads, 0, s>>>(Y, scratch, fs, sy, sz, tiles, ntiles, max_cols);
-  else
-    z4c_derivs_split_kernel<4><<<grid, kThreads, 0, s>>>(Y, scratch, fs, sy, sz, tiles, ntiles, max_cols);
+  const long items = (long)ntiles * kNZ4c;
+  const int cap = caps().derivs[order == 8];
+  const int grid = items < cap ? (int)items : cap;
+  if (order == 8) z4c_derivs_split_kernel<8><<<grid, kDerivCols, 0, s>>>(Y, scratch, fs, sy, sz, tiles, ntiles);
+  else z4c_derivs_split_kernel<4><<<grid, kDerivCols, 0, s>>>(Y, scratch, fs, sy, sz, tiles, ntiles);
   return cudaGetLastError();
 }
 
