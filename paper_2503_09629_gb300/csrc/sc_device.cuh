@@ -60,20 +60,85 @@ __device__ __forceinline__ void amr_prolong_cells_body(const double* __restrict_
 // and uses nodes c-3..c+2; parity 1: +1/4 and c-2..c+3).
 __device__ __forceinline__ int tile_node_offset(int p0, int i) { return ((p0 + i) >> 1) + ((p0 + i) & 1) - p0; }
 
-// Shared-memory doubles the tile-separable prolongation needs per group of
+// Shared memory (in doubles) the tile-separable prolongation needs per group of
 // 128 threads: the parent region (at most 10 x 10 x 8 nodes), the x sums (at
-// most 8 x 10 x 8) and the y sums (at most 8 x 8 x 8).
+// most 8 x 10 x 8) and the y sums (at most 8 x 8 x 8), and an exponent of two
+// bytes for each of them.
 constexpr int kTileRegion = 800, kTileXSums = 640, kTileYSums = 512;
-constexpr int kProlongSmemPerGroup = kTileRegion + kTileXSums + kTileYSums;
+constexpr int kTileValues = kTileRegion + kTileXSums + kTileYSums;
+constexpr int kProlongSmemPerGroup = kTileValues + kTileValues / 4;
+
+// The two fine positions of parent cell c of a line (parities 0 and 1, at -1/4
+// and +1/4) from the seven nodes their stencils cover: nodes n0..n0 + 6 of the
+// line's N (those outside it belong to a position that the tile does not have).
+// Values are v * 2^e with |v| < 2^60.2 (59 bits, grown by less than 1.3 per axis:
+// the weights' magnitudes sum to 10568 / 8192).  Each position's six nodes are
+// aligned to their own largest exponent, so that its value does not depend on
+// the tile it is in, and the weights are integers over 2^13: a sum is exact to
+// the last place of that alignment.
+__device__ __forceinline__ void prolong_pair(const long long* __restrict__ v, const short* __restrict__ ve, int n0,
+                                             int N, int stride, long long* lo, long long* hi, int* elo, int* ehi) {
+  auto align = [](long long x, int n) {
+    long long r;
+    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+    return r;
+  };
+  long long x[7];
+  int e[7], mid = 0;
+#pragma unroll
+  for (int m = 0; m < 7; ++m) {
+    const int n = min(max(n0 + m, 0), N - 1) * stride;
+    x[m] = v[n];
+    e[m] = ve[n];
+    if (m > 0 && m < 6) mid = max(mid, e[m]);
+  }
+  const int E0 = max(e[0], mid), E1 = max(mid, e[6]);
+  constexpr int w[6] = {63, -495, 2310, 6930, -693, 77};  // parity 0: -1/4 from cell c, nodes c-3..c+2; parity 1 mirrored
+  FxWide a, b;
+  a.add(w[0], align(x[0], E0 - e[0]));
+  b.add(w[0], align(x[6], E1 - e[6]));
+  long long y[5];
+#pragma unroll
+  for (int m = 1; m < 6; ++m) {
+    y[m - 1] = align(x[m], E0 - e[m]);
+    a.add(w[m], y[m - 1]);
+  }
+  if (E0 != E1) {
+#pragma unroll
+    for (int m = 1; m < 6; ++m) y[m - 1] = align(x[m], E1 - e[m]);
+  }
+#pragma unroll
+  for (int m = 1; m < 6; ++m) b.add(w[6 - m], y[m - 1]);
+  *lo = a.get<13>();
+  *hi = b.get<13>();
+  *elo = E0;
+  *ehi = E1;
+}
+// A tile's lines along one axis: lines * pairs work items, line l's nodes at
+// line_base(l) + n * stride, its fine positions written by out(l, i, v, e).
+template <class BASE, class OUT>
+__device__ __forceinline__ void prolong_axis(const long long* v, const short* ve, int t, int lines, int p0, int ext,
+                                             int N, int stride, const BASE& base, const OUT& out) {
+  const int pairs = ((p0 + ext - 1) >> 1) + 1;
+  for (int q = t; q < lines * pairs; q += 128) {
+    const int c = q / lines, l = q - c * lines, b = base(l), i = 2 * c - p0;
+    long long lo, hi;
+    int elo, ehi;
+    prolong_pair(v + b, ve + b, c - p0, N, stride, &lo, &hi, &elo, &ehi);
+    if (i >= 0) out(l, i, lo, elo);
+    if (i + 1 < ext) out(l, i + 1, hi, ehi);
+  }
+}
 
 // Separable form of the same interpolation for the slab tiles of a ghost
 // shell: one group of 128 threads per (tile, vector, field) stages the
 // tile's parent region in shared memory and interpolates along x, then y,
-// then z.  Each value is the same chain of fused multiply-adds as in the
-// per-cell form (x sums over six nodes from zero, then y sums of those, then
-// z sums), so both give identical results.  Along the thin axis of a slab
-// tile (the ghost width) the sums shrink 7-8 nodes to 3-4 values, so a ghost
-// value costs about 20-40 FMAs instead of the 216 + 42 of the per-cell form.
+// then z.  Along the thin axis of a slab tile (the ghost width) the sums shrink
+// 7-8 nodes to 3-4 values, so a ghost value costs 20-40 multiplications instead
+// of the 216 + 42 of the per-cell form.  The sums are integers (prolong_pair), two
+// fine positions of a parent cell at a time: in FP64 chains (which stay for
+// tiles that hold an infinity, a NaN or a value near the ends of the exponent
+// range) the kernel was bound by that pipe, 82% of its rate.
 // ngrp groups of 128 threads (threads beyond them idle); sm: ngrp *
 // kProlongSmemPerGroup doubles.  Every thread of the block must call this
 // function (it synchronises the block).
@@ -88,6 +153,12 @@ __device__ __forceinline__ void amr_prolong_tiles_body(const double* __restrict_
   double* sR = sm + grp * kProlongSmemPerGroup;
   double* sX = sR + kTileRegion;
   double* sY = sX + kTileXSums;
+  long long* iR = reinterpret_cast<long long*>(sR);  // the same places for the integer form
+  long long* iX = iR + kTileRegion;
+  long long* iY = iX + kTileXSums;
+  short* eR = reinterpret_cast<short*>(sR + kTileValues);
+  short* eX = eR + kTileRegion;
+  short* eY = eX + kTileXSums;
   const int combos = nvec * F;
   const int ngroups = (combos + ngrp - 1) / ngrp;
   const long items = (long)ntiles * ngroups;
@@ -101,13 +172,50 @@ __device__ __forceinline__ void amr_prolong_tiles_body(const double* __restrict_
     const int Nx = tile_node_offset(px, ex - 1) + kPN, Ny = tile_node_offset(py, ey - 1) + kPN;
     const int Nz = tile_node_offset(pz, ez - 1) + kPN;
     const int v = active ? combo / F : 0, f = active ? combo % F : 0;
-    if (active) {
-      const double* base = (v == 0 ? yn : v == 1 ? k1 : v == 2 ? k2 : v == 3 ? k3 : k4) + (long)f * pfs + T.pbase;
+    const double* base = (v == 0 ? yn : v == 1 ? k1 : v == 2 ? k2 : v == 3 ? k3 : k4) + (long)f * pfs + T.pbase;
+    int bad = 0;
+    if (active)
       for (int q = t; q < Nx * Ny * Nz; q += 128) {
         const int x = q % Nx, r = q / Nx;
-        sR[q] = __ldg(base + (long)(r / Ny) * psz + (long)(r % Ny) * psy + x);  // [z][y][x]
+        const double d = __ldg(base + (long)(r / Ny) * psz + (long)(r % Ny) * psy + x);  // [z][y][x]
+        const int h = __double2hiint(d), e = (h >> 20) & 0x7ff;
+        const long long s = h >> 31;
+        const long long bits = __double_as_longlong(d), m = (bits & 0xfffffffffffffll) | 0x10000000000000ll;
+        const bool zero = (bits << 1) == 0;
+        iR[q] = zero ? 0 : ((m << 6) ^ s) - s;
+        eR[q] = (short)e;
+        bad |= (unsigned)(e - 120) > 1880u && !zero;
       }
+    if (!__syncthreads_or(bad)) {
+      if (active)
+        prolong_axis(iR, eR, t, Ny * Nz, px, ex, Nx, 1, [&](int l) { return l * Nx; },
+                     [&](int l, int i, long long x, int e) {
+                       iX[l * ex + i] = x;  // [z][y][i]
+                       eX[l * ex + i] = (short)e;
+                     });
+      __syncthreads();
+      if (active)
+        prolong_axis(iX, eX, t, ex * Nz, py, ey, Ny, ex, [&](int l) { return (l / ex) * Ny * ex + l % ex; },
+                     [&](int l, int j, long long x, int e) {
+                       const int o = ((l / ex) * ey + j) * ex + l % ex;  // [z][j][i]
+                       iY[o] = x;
+                       eY[o] = (short)e;
+                     });
+      __syncthreads();
+      if (active)
+        prolong_axis(iY, eY, t, ex * ey, pz, ez, Nz, ex * ey, [&](int l) { return l; },
+                     [&](int l, int k, long long x, int e) {
+                       const int slot = slots[T.slot_base + k * ex * ey + l];
+                       if (slot >= 0) store[((long)v * F + f) * ncells + slot] = fx_back<6, 0>(x, e << 20);
+                     });
+      __syncthreads();
+      continue;
     }
+    if (active)
+      for (int q = t; q < Nx * Ny * Nz; q += 128) {
+        const int x = q % Nx, r = q / Nx;
+        sR[q] = __ldg(base + (long)(r / Ny) * psz + (long)(r % Ny) * psy + x);
+      }
     __syncthreads();
     if (active) {  // x: each (y, z) row of nodes to the tile's ex fine positions
       for (int q = t; q < ex * Ny * Nz; q += 128) {
