@@ -392,77 +392,153 @@ __device__ __forceinline__ void restrict_blocks_body(double* __restrict__ parent
   }
 }
 
+// The halo cells of a plane of a tile that a thread brings into shared memory,
+// W columns and rows wide on each side without the corners: the shared-memory
+// place (rows of nx + 2 W; -1: none) and the offset from the tile's first cell.
+template <int W>
+__device__ __forceinline__ void halo_cell(const Tile& T, int h, long sy, int* place, long* off) {
+  *place = -1;
+  *off = 0;
+  if (h >= 2 * W * (T.nx + T.ny)) return;
+  int x, y;
+  if (h < 2 * W * T.ny) {
+    y = h / (2 * W);
+    x = h - y * (2 * W);
+    x = x < W ? x - W : T.nx + x - W;
+  } else {
+    h -= 2 * W * T.ny;
+    y = h / T.nx;
+    x = h - y * T.nx;
+    y = y < W ? y - W : T.ny + y - W;
+  }
+  *place = (y + W) * (T.nx + 2 * W) + x + W;
+  *off = (long)y * sy + x;
+}
+// Values of a plane with its halo (tiles of at most kDerivCols columns, 32 wide, 32 high).
+__host__ __device__ constexpr int plane_values(int W) { return (32 + 2 * W) * (8 + 2 * W); }
+
 // Scalar-wave stage (Sec. IV.A): k_i = f(Y_i) with the centred Laplacian (4th
 // or 8th order), then the stage update of StageArgs (Eqs. rk2-rk5 for RK4,
-// the last-stage combinations of RK3/RK2, or k only).  One tile per worker
-// at a time, the block's threads over its cells.
+// the last-stage combinations of RK3/RK2, or k only).  One tile per worker at a
+// time, a thread per column: it walks z with the packed values of u at z-R..z+R
+// in registers and shares the plane's through shared memory (planes: 2 *
+// plane_values(R)), so a value is unpacked once or twice instead of 13 (25)
+// times; the Laplacian is summed in aligned integers (sc_fixed.cuh), or in FP64
+// where the values do not allow that.  256 threads; every thread of the block must
+// call this function (it synchronises the block).
 template <int ORD>
 __device__ __forceinline__ void wave_stage_body(const StageArgs& a, const Tile* __restrict__ tiles, int ntiles,
-                                                const FmaK& K, int bid, int nb) {
-  const double inv12h2 = ORD == 4 ? 1.0 / (12.0 * a.h * a.h) : 1.0 / (5040.0 * a.h * a.h);
+                                                const FmaK& K, int bid, int nb, long long* planes) {
+  using F = FxSums<ORD>;
+  constexpr int R = ORD / 2, NW = 2 * R + 1, G = F::kGuard;
   const long sy = a.sy, sz = a.sz;
+  int buf = 0;
   for (int t = bid; t < ntiles; t += nb) {
     const Tile T = tiles[t];
-    const int n = T.nx * T.ny * T.nz;
-    for (int q = threadIdx.x; q < n; q += blockDim.x) {
-      const int i = q % T.nx;
-      const int j = (q / T.nx) % T.ny;
-      const int k = q / (T.nx * T.ny);
-      const long o = (T.z0 + k) * sz + (T.y0 + j) * sy + (T.x0 + i);
-      const double* u = a.Y + o;
-      const double u0 = u[0];
-      // sm = sum over the 6 neighbours at distance m; 4th order: 16 s1 - s2 - 90 u0 over
-      // 12 h^2, 8th order: 8064 s1 - 1008 s2 + 128 s3 - 9 s4 - 43050 u0 over 5040 h^2; in
-      // aligned integers (sc_fixed.cuh), or in FP64 where the values do not allow that
-      constexpr int R = ORD / 2;
-      double v[R][6];
-      int E = fx_exp(u0);
+    const int pitch = T.nx + 2 * R;
+    const bool active = (int)threadIdx.x < T.nx * T.ny;
+    const int j = threadIdx.x / T.nx, i = threadIdx.x - j * T.nx, own = (j + R) * pitch + i + R;
+    const long o0 = (long)T.z0 * sz + (long)T.y0 * sy + T.x0;
+    int hs[2];
+    long ho[2];
+    double hv[2];
+    halo_cell<R>(T, threadIdx.x, sy, &hs[0], &ho[0]);
+    halo_cell<R>(T, threadIdx.x + kDerivCols, sy, &hs[1], &ho[1]);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) hv[r] = hs[r] >= 0 ? a.Y[o0 + ho[r]] : 0.0;
+    const double* u = a.Y + o0 + (long)j * sy + i;
+    long long w[NW];
+    double un = 0.0;
+    if (active) {
+#pragma unroll
+      for (int m = 0; m < NW - 1; ++m) w[m] = fx_pack(u[(m - R) * sz]);
+      un = u[R * sz];
+    }
+#pragma unroll 1
+    for (int k = 0; k < T.nz; ++k, buf ^= 1) {
+      long long* pl = planes + buf * plane_values(R);
+      const bool more = k + 1 < T.nz;
+      const long o = o0 + k * sz + (long)j * sy + i;
+      double ku = 0.0, yu = 0.0, yp = 0.0, k1u = 0.0, k1p = 0.0, k2u = 0.0, k2p = 0.0, k3u = 0.0, k3p = 0.0;
+      if (active) {
+        pl[own] = w[R];
+        ku = a.Y[a.fs + o];  // d_t u = Pi
+        if (a.form != kStageNone) {
+          yu = a.yn[o];
+          yp = a.yn[a.fs + o];
+        }
+        if (a.form == kStageRk4 || a.form == kStageTwo) {
+          k1u = a.k1[o];
+          k1p = a.k1[a.fs + o];
+        }
+        if (a.form == kStageRk4) {
+          k2u = a.k2[o];
+          k2p = a.k2[a.fs + o];
+          k3u = a.k3[o];
+          k3p = a.k3[a.fs + o];
+        }
+        w[NW - 1] = fx_pack(un);
+        if (more) un = u[(k + 1 + R) * sz];
+      }
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+        if (hs[r] >= 0) {
+          pl[hs[r]] = fx_pack(hv[r]);
+          if (more) hv[r] = a.Y[o0 + ho[r] + (k + 1) * sz];
+        }
+      // (the planes alternate, also from one tile to the next: a plane is written
+      // again only after every thread has passed the next barrier)
+      __syncthreads();
+      if (!active) continue;
+      long long v[R][6];
+      int E = fx_pexp(w[R]);
 #pragma unroll
       for (int m = 0; m < R; ++m) {
-        v[m][0] = u[-(m + 1)];
-        v[m][1] = u[m + 1];
-        v[m][2] = u[-(m + 1) * sy];
-        v[m][3] = u[(m + 1) * sy];
-        v[m][4] = u[-(m + 1) * sz];
-        v[m][5] = u[(m + 1) * sz];
+        v[m][0] = pl[own - (m + 1)];
+        v[m][1] = pl[own + (m + 1)];
+        v[m][2] = pl[own - (m + 1) * pitch];
+        v[m][3] = pl[own + (m + 1) * pitch];
+        v[m][4] = w[R - (m + 1)];
+        v[m][5] = w[R + (m + 1)];
 #pragma unroll
-        for (int q = 0; q < 6; ++q) E = max(E, fx_exp(v[m][q]));
+        for (int q = 0; q < 6; ++q) E = max(E, fx_pexp(v[m][q]));
       }
       double lap;
-      if (aligned_ok(E)) {
-        using F = FxSums<ORD>;
+      if (packed_ok(E)) {
         typename F::Val s[R];
 #pragma unroll
         for (int m = 0; m < R; ++m) {
-          s[m] = F::val(v[m][0], E);
+          s[m] = fx_palign<G>(v[m][0], E);
 #pragma unroll
-          for (int q = 1; q < 6; ++q) s[m] += F::val(v[m][q], E);
+          for (int q = 1; q < 6; ++q) s[m] += fx_palign<G>(v[m][q], E);
         }
-        lap = F::laplacian(s, F::val(u0, E), E);
+        lap = F::laplacian(s, fx_palign<G>(w[R], E), packed_field(E));
       } else {
+        const double* c = u + k * sz;
         double s[4];
 #pragma unroll
-        for (int m = 0; m < R; ++m) s[m] = ((v[m][0] + v[m][1]) + (v[m][2] + v[m][3])) + (v[m][4] + v[m][5]);
-        if (ORD == 4) lap = fma(-90.0, u0, fma(16.0, s[0], -s[1]));
-        else lap = fma(-43050.0, u0, fma(8064.0, s[0], fma(-1008.0, s[1], fma(128.0, s[2], -9.0 * s[3]))));
+        for (int m = 1; m <= R; ++m)
+          s[m - 1] = ((c[-m] + c[m]) + (c[-m * sy] + c[m * sy])) + (c[-m * sz] + c[m * sz]);
+        if (ORD == 4) lap = fma(-90.0, c[0], fma(16.0, s[0], -s[1]));
+        else lap = fma(-43050.0, c[0], fma(8064.0, s[0], fma(-1008.0, s[1], fma(128.0, s[2], -9.0 * s[3]))));
       }
-      lap = fmul(lap, inv12h2, K);
-      const double ku = a.Y[a.fs + o];  // d_t u = Pi
-      const double kp = lap;            // d_t Pi = Laplacian u
+      const double kp = fmul(lap, a.ds.s2p, K);  // d_t Pi = Laplacian u, its sum over 12 h^2 or 5040 h^2
       a.k[o] = ku;
       a.k[a.fs + o] = kp;
       if (a.form == kStageSingle) {
-        a.out[o] = fma(a.cdt, ku, a.yn[o]);
-        a.out[a.fs + o] = fma(a.cdt, kp, a.yn[a.fs + o]);
+        a.out[o] = fma(a.cdt, ku, yu);
+        a.out[a.fs + o] = fma(a.cdt, kp, yp);
       } else if (a.form == kStageRk4) {
-        const double su = fadd(fma(2.0, a.k3[o], fma(2.0, a.k2[o], a.k1[o])), ku, K);
-        const double sp = fadd(fma(2.0, a.k3[a.fs + o], fma(2.0, a.k2[a.fs + o], a.k1[a.fs + o])), kp, K);
-        a.out[o] = fma(a.cdt, su, a.yn[o]);
-        a.out[a.fs + o] = fma(a.cdt, sp, a.yn[a.fs + o]);
+        const double su = fadd(fma(2.0, k3u, fma(2.0, k2u, k1u)), ku, K);
+        const double sp = fadd(fma(2.0, k3p, fma(2.0, k2p, k1p)), kp, K);
+        a.out[o] = fma(a.cdt, su, yu);
+        a.out[a.fs + o] = fma(a.cdt, sp, yp);
       } else if (a.form == kStageTwo) {
-        a.out[o] = fma(a.cdt, ku, fma(a.c1dt, a.k1[o], a.yn[o]));
-        a.out[a.fs + o] = fma(a.cdt, kp, fma(a.c1dt, a.k1[a.fs + o], a.yn[a.fs + o]));
+        a.out[o] = fma(a.cdt, ku, fma(a.c1dt, k1u, yu));
+        a.out[a.fs + o] = fma(a.cdt, kp, fma(a.c1dt, k1p, yp));
       }
+#pragma unroll
+      for (int m = 0; m < NW - 1; ++m) w[m] = w[m + 1];
     }
   }
 }

@@ -257,7 +257,7 @@ struct Level {
   CellRun* runs = nullptr;          // the pointwise Z4c kernel's units (one cell per thread)
   int nruns = 0;
   std::vector<int> box_run_begin;
-  Tile* dtiles = nullptr;           // tiles of the Z4c derivative pass
+  Tile* dtiles = nullptr;           // tiles of the Z4c derivative pass and the wave stage
   int ndtiles = 0;
   std::vector<int> box_dtile_begin;
   AmrCell* amr = nullptr;
@@ -681,11 +681,12 @@ void build_stencil_tiles(Level& L, const int* tile, std::vector<Tile>& out) {
   L.box_tile_begin.push_back((int)out.size());
 }
 
-// Tiles of the Z4c derivative pass for the boxes of a level: the width splits
-// a box's rows evenly, the height fills a block of threads, and the depth is
-// as large as still gives every SM a few (tile, field) items, between 4 planes
-// and 16 (a block reads 6 or 8 planes more than it computes).
-void build_deriv_tiles(const Geom& g, const sc_box* boxes, size_t nboxes, std::vector<Tile>& out,
+// Tiles of the Z4c derivative pass (an item is a tile and one of 22 fields) and
+// of the wave stage (an item is a tile) for the boxes of a level: the width splits
+// a box's rows evenly, the height fills a block of threads, and the depth is as
+// large as still gives every SM a few items, 16 planes at most (a block reads 4
+// to 8 planes more than it computes) and 4 at least for Z4c, 1 for the wave.
+void build_deriv_tiles(const Geom& g, const sc_box* boxes, size_t nboxes, int system, std::vector<Tile>& out,
                        std::vector<int>& begin) {
   auto parts = [](int n, int most) { return (n + most - 1) / most; };
   auto even = [&](int n, int most) { return parts(n, parts(n, most)); };  // the extent that splits n evenly
@@ -696,8 +697,10 @@ void build_deriv_tiles(const Geom& g, const sc_box* boxes, size_t nboxes, std::v
     const int tx = even(nx, 32), ty = even(ny, std::min(32, kDerivCols / tx));
     columns += (long)parts(nx, tx) * parts(ny, ty) * (B.hi[2] - B.lo[2] + 1);
   }
+  const int least = system == SC_Z4C ? 4 : 1;
+  const long items = system == SC_Z4C ? kNZ4c * columns : 4 * columns;  // wanted: 12 and 3 per SM
   int depth = 16;
-  while (depth > 4 && columns / depth * kNZ4c < 4L * sm_count() * 3) depth /= 2;
+  while (depth > least && items / depth < 12L * sm_count()) depth /= 2;
   out.clear();
   begin.clear();
   for (size_t b = 0; b < nboxes; ++b) {
@@ -801,7 +804,7 @@ sc_status classify_level(sc_ctx* c, int l, HostLists& hl) {
       }
   if (l > 0 && !hl.amr.empty()) build_amr_tiles(c, l, hl);
   build_stencil_tiles(L, c->tile, hl.tiles);
-  if (c->system == SC_Z4C) build_deriv_tiles(g, L.boxes.data(), L.boxes.size(), hl.dtiles, L.box_dtile_begin);
+  build_deriv_tiles(g, L.boxes.data(), L.boxes.size(), c->system, hl.dtiles, L.box_dtile_begin);
   // Runs of cells of the Z4c stage kernel, one cell per thread.
   L.box_run_begin.clear();
   for (const sc_box& B : L.boxes) {
@@ -1214,11 +1217,11 @@ sc_status run_op(sc_ctx* c, const Op& o, cudaStream_t s) {
       for (int b = 0; b < nparts; ++b) {
         const int t0 = nparts == 1 ? 0 : L.box_tile_begin[b];
         const int nt = nparts == 1 ? L.ntiles : L.box_tile_begin[b + 1] - t0;
+        const int d0 = nparts == 1 ? 0 : L.box_dtile_begin[b];
+        const int nd = nparts == 1 ? L.ndtiles : L.box_dtile_begin[b + 1] - d0;
         if (c->system == SC_WAVE) {
-          CU(launch_wave_stage(a, L.tiles + t0, nt, s, c->order, foldp));
+          CU(launch_wave_stage(a, L.dtiles + d0, nd, s, c->order, foldp));
         } else {
-          const int d0 = nparts == 1 ? 0 : L.box_dtile_begin[b];
-          const int nd = nparts == 1 ? L.ndtiles : L.box_dtile_begin[b + 1] - d0;
           const int p0 = nparts == 1 ? 0 : L.box_run_begin[b];
           const int np = nparts == 1 ? L.nruns : L.box_run_begin[b + 1] - p0;
           if (one_pass) CU(launch_z4c_derivs(a.Y, c->scratch, g.fs, a.sy, a.sz, L.tiles + t0, nt, s));
@@ -1330,9 +1333,10 @@ void persistent_phases(sc_ctx* c, const std::vector<Op>& ops, std::vector<POp>& 
         p.a.sy = g.pitch;
         p.a.sz = g.pitch * g.ext[1];
         p.a.h = g.h;
+        p.a.ds = deriv_scales(c->order, g.h);
         p.a.eta = L.eta;
-        p.tiles = L.tiles;
-        p.ntiles = L.ntiles;
+        p.tiles = L.dtiles;
+        p.ntiles = L.ndtiles;
         p.order = c->order;
         p.phys = L.phys;
         p.nphys = L.nphys;
@@ -1647,7 +1651,7 @@ sc_status time_candidate(sc_ctx* c, Level& L, int kind, const Tile* tiles, int n
     if (kind == 1) {
       CU(launch_z4c_stage(a, c->scratch, c->zp, L.runs, L.nruns, c->stream, bps));
     } else if (c->system == SC_WAVE) {
-      CU(launch_wave_stage(a, tiles, ntiles, c->stream, c->order));
+      CU(launch_wave_stage(a, L.dtiles, L.ndtiles, c->stream, c->order));
     } else if (deriv_form == 1) {
       CU(launch_z4c_derivs(a.Y, c->scratch, g.fs, a.sy, a.sz, tiles, ntiles, c->stream));
     } else {
@@ -1725,8 +1729,8 @@ extern "C" sc_status sc_autotune(sc_ctx* c, int* tile_out, double* ms_out) {
     std::vector<void*> scratch_lists;
     for (int form = 0; form < nform; ++form)
       for (const auto& cd : cand) {
-        // Z4c: the two-kernel form has tiles of its own, the one-kernel form takes the default ones
-        if (c->system == SC_Z4C && (cd[0] != 32 || cd[1] != 4 || cd[2] != 2)) continue;
+        // the wave stage and the two-kernel Z4c form have tiles of their own, the one-kernel form takes these
+        if (cd[0] != 32 || cd[1] != 4 || cd[2] != 2) continue;
         build_stencil_tiles(L, cd, t);
         if (t.size() > cap) {
           cap = t.size() * 2;
@@ -2442,7 +2446,7 @@ sc_status sc_time_stage_kernels(sc_ctx* c, int level, int nrep, double* ms) {
   float t0 = 0, t1 = 0;
   CU(cudaEventRecord(e[0], c->stream));
   for (int r = 0; r < nrep; ++r) {
-    if (c->system == SC_WAVE) CU(launch_wave_stage(a, L.tiles, L.ntiles, c->stream, c->order));
+    if (c->system == SC_WAVE) CU(launch_wave_stage(a, L.dtiles, L.ndtiles, c->stream, c->order));
     else if (c->deriv_form == 1 && c->order == 4)
       CU(launch_z4c_derivs(a.Y, c->scratch, g.fs, a.sy, a.sz, L.tiles, L.ntiles, c->stream));
     else {

@@ -50,7 +50,7 @@ struct CellRun {
   int32_t first, n;
 };
 constexpr int kRunCells = 64;
-constexpr int kDerivCols = 256;  // columns of a tile of the Z4c derivative pass
+constexpr int kDerivCols = 256;  // columns of a tile of the Z4c derivative pass and the wave stage
 
 // Refinement-boundary ghost cell: destination offset in the fine array,
 // offset of the first parent stencil cell in the parent array, parity of
@@ -161,7 +161,7 @@ struct StageArgs {
   int sy, sz;        // strides of y and z in doubles
   double h;
   const double* eta; // Z4c: per-cell Gamma-driver damping eta(r), or null for the constant
-  DerivScales ds;    // Z4c: scales of the stored derivative sums
+  DerivScales ds;    // scales of the derivative sums
 };
 
 // Additions, subtractions and scalings that do not fuse are written as fused

@@ -70,8 +70,8 @@ __device__ void run_phase(const POp& op, const Weights& w, double* sm, int bid, 
   switch (op.kind) {
     case kPhaseStage:
       if (op.ntiles) {
-        if (op.order == 8) wave_stage_body<8>(op.a, op.tiles, op.ntiles, K, bid, nb);
-        else wave_stage_body<4>(op.a, op.tiles, op.ntiles, K, bid, nb);
+        if (op.order == 8) wave_stage_body<8>(op.a, op.tiles, op.ntiles, K, bid, nb, reinterpret_cast<long long*>(sm));
+        else wave_stage_body<4>(op.a, op.tiles, op.ntiles, K, bid, nb, reinterpret_cast<long long*>(sm));
       }
       if (op.nphys) radiative_stage_body(op.a, op.phys, op.nphys, op.F, op.g, op.system, bid, nb);
       // the refinement-boundary ghosts of the next stage input, when the

@@ -15,10 +15,16 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// Bound by the latency of its loads at 16 warps per SM (three blocks per SM, with
+// spills: 5% slower; 8th order with one block's registers: 0.221 ms instead of
+// 0.135); DRAM at half its rate.  256^3 level (64 bytes a cell, 0.158 ms at the
+// memory's rate): 0.552 ms in FP64, 0.411 with 13 values unpacked by every thread,
+// 0.337 so; 64^3: 0.0186, 0.0145, 0.0104; 8th order, 160^3: 0.234, 0.191, 0.135.
 template <int ORD>
-__global__ void __launch_bounds__(kThreads) wave_stage_kernel(StageArgs a, const Tile* __restrict__ tiles,
+__global__ void __launch_bounds__(kThreads, 2) wave_stage_kernel(StageArgs a, const Tile* __restrict__ tiles,
                                                              int ntiles, FmaK K, ApplyArgs fill) {
-  wave_stage_body<ORD>(a, tiles, ntiles, K, blockIdx.x, gridDim.x);
+  __shared__ long long planes[2 * plane_values(ORD / 2)];
+  wave_stage_body<ORD>(a, tiles, ntiles, K, blockIdx.x, gridDim.x, planes);
   if (fill.ncells)
     amr_apply_body(fill.vec, fill.fs, fill.F, fill.cells, fill.ncells, fill.store, fill.c[0], fill.c[1], fill.c[2],
                    fill.c[3], fill.nk, blockIdx.x, gridDim.x);

@@ -18,7 +18,7 @@
 // FP32 rate), so both passes work in integers (sc_fixed.cuh: the stencil sums;
 // sc_z4c_fixed.cuh: the tensor contractions), and the FP64 forms beside them
 // are for the cells whose values the integer forms do not take.
-#include "sc_fixed.cuh"
+#include "sc_device.cuh"
 #include "sc_z4c_fixed.cuh"
 
 namespace sc {
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kDerivCols, 2)
   constexpr int ND = 2 * R + 1;
   constexpr int G = F::kGuard;
   constexpr bool kWindows = ORD == 4;
-  __shared__ long long planes[2][(32 + 2 * WR) * (8 + 2 * WR)];
+  __shared__ long long planes[2][plane_values(WR)];
   const long sy = sy_, sz = sz_;
   int buf = 0;
   for (int item = blockIdx.x; item < ntiles * kNZ4c; item += gridDim.x) {
@@ -235,28 +235,14 @@ __global__ void __launch_bounds__(kDerivCols, 2)
     const int own = (j + WR) * pitch + i + WR;
     const double* u = base + (long)j * sy + i;
     const long o0 = (long)T.z0 * sz + (long)(T.y0 + j) * sy + (T.x0 + i);
-    // halo cells of a plane: 2 WR per row, then 2 WR rows
     int hs[2];
     const double* hp[2];
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-      int h = threadIdx.x + r * kDerivCols, x, y;
-      hs[r] = -1;
+      long off;
+      halo_cell<WR>(T, threadIdx.x + r * kDerivCols, sy, &hs[r], &off);
       hp[r] = base;
-      if (h < 2 * WR * (T.nx + T.ny)) {
-        if (h < 2 * WR * T.ny) {
-          y = h / (2 * WR);
-          x = h - y * (2 * WR);
-          x = x < WR ? x - WR : T.nx + x - WR;
-        } else {
-          h -= 2 * WR * T.ny;
-          y = h / T.nx;
-          x = h - y * T.nx;
-          y = y < WR ? y - WR : T.ny + y - WR;
-        }
-        hs[r] = (y + WR) * pitch + x + WR;
-        hp[r] += (long)y * sy + x;
-      }
+      if (hs[r] >= 0) hp[r] += off;
     }
     const int sl = d2_slot(f);
     const double* Dx = S + (long)(Q_D1 + 3 * f + 0) * fs + o0;
@@ -776,14 +762,13 @@ __global__ void __launch_bounds__(kRunCells, 2 * BPS) z4c_stage_kernel(StageArgs
                                                                       KT K) {
   __shared__ long long slots[FM_SLOTS * kRunCells];
   const FxMem<kRunCells> mem{slots + threadIdx.x};
-  const double ko = P.ko_sigma / (64.0 * a.h);
   for (int u = blockIdx.x; u < nruns; u += gridDim.x) {
     const CellRun R = runs[u];
     if ((int)threadIdx.x >= R.n) continue;
     const int q = R.first + threadIdx.x, row = q / R.nx, z = row / R.ny;
     const long o = R.off + (long)z * a.sz + (long)(row - z * R.ny) * a.sy + (q - row * R.nx);
     const double eta = a.eta ? a.eta[o] : P.eta;
-    const StageUpdate<FORM, KT> update{a, S, o, ko, K};
+    const StageUpdate<FORM, KT> update{a, S, o, c.ko, K};
     // (the stage's inputs and outputs are different arrays, so a cell that turns
     // out to need the FP64 form is simply written again)
     if (!z4c_rhs_fixed(a.Y, S, a.fs, o, P, eta, c, mem, K, update)) {
@@ -962,7 +947,8 @@ namespace {
 template <int BPS>
 void launch_stage_bps(const StageArgs& a, const double* scratch, const Z4cParams& p, const CellRun* runs, int nruns,
                       int grid, cudaStream_t s, const FmaK& K, bool op_class) {
-  const FxScales c = fx_scales(a.ds);
+  FxScales c = fx_scales(a.ds);
+  c.ko = p.ko_sigma / (64.0 * a.h);
   if (op_class)
     z4c_stage_kernel<kStageSingle, BPS, PlainK><<<grid, kRunCells, 0, s>>>(a, scratch, p, runs, nruns, c, PlainK{});
   else if (a.form == kStageRk4) z4c_stage_kernel<kStageRk4, BPS><<<grid, kRunCells, 0, s>>>(a, scratch, p, runs, nruns, c, K);

@@ -318,9 +318,10 @@ struct FxScales {
   FxC kP3, kM3;      // a third of those
   FxC twothird;      // exponent -59
   int poff;          // in place
+  double ko;         // sigma / (64 h) of the dissipation sum
 };
 inline FxScales fx_scales(const DerivScales& ds) {
-  FxScales c;
+  FxScales c{};
   c.s1 = fx_const(ds.s1);
   c.ts1 = fx_const(ds.ts1);
   // s2p / s2m = 12 (4th order) or 140 (8th): the power of two above it goes with the values
