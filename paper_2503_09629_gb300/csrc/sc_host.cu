@@ -2392,7 +2392,7 @@ sc_status sc_get_constraints(sc_ctx* c, int level, int box, double* dst) {
     CU(launch_z4c_derivs_split(Y, c->scratch, L.g.fs, sy, sz, L.dtiles + L.box_dtile_begin[box],
                                L.box_dtile_begin[box + 1] - L.box_dtile_begin[box], c->stream, c->order));
   }
-  CU(launch_z4c_constraints(Y, c->scratch, c->staging, L.g.fs, sy, sz, c->zp, deriv_scales(c->order, L.g.h), dt, (int)tl.size(), ncell, blo, n,
+  CU(launch_z4c_constraints(Y, c->scratch, c->staging, L.g.fs, sy, sz, c->zp, deriv_scales(c->order, L.g.h), ncell, blo, n,
                             c->stream));
   CU(cudaMemcpyAsync(dst, c->staging, bytes, cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));

@@ -771,7 +771,7 @@ __global__ void __launch_bounds__(kRunCells, 2 * BPS) z4c_stage_kernel(StageArgs
     const StageUpdate<FORM, KT> update{a, S, o, c.ko, K};
     // (the stage's inputs and outputs are different arrays, so a cell that turns
     // out to need the FP64 form is simply written again)
-    if (!z4c_rhs_fixed(a.Y, S, a.fs, o, P, eta, c, mem, K, update)) {
+    if (!z4c_rhs_fixed<false>(a.Y, S, a.fs, o, P, eta, c, mem, K, update)) {
       double rhs[kNZ4c];
       z4c_rhs_fp64(a.Y, S, a.fs, o, P, eta, a.ds, rhs, K);
 #pragma unroll 1
@@ -784,87 +784,101 @@ __global__ void __launch_bounds__(kRunCells, 2 * BPS) z4c_stage_kernel(StageArgs
 //   H   = R + 2/3 (Khat + 2 Theta)^2 - At_ij At^ij      (R the Ricci scalar of gamma)
 //   M^i = d_j At^ij + Gamt^i_jk At^jk - 3 At^ij d_j W / W - 2/3 gt^ij d_j (Khat + 2 Theta)
 //   G^i = Gamt^i - gt^jk Gamt^i_jk
-// out[c * out_stride + cell], cells numbered x-fastest within the box.
-__global__ void __launch_bounds__(128) z4c_constraints_kernel(const double* __restrict__ Y,
-                                                             const double* __restrict__ S, double* __restrict__ out,
-                                                             long fs, int sy, int sz, Z4cParams P, DerivScales ds,
-                                                             const Tile* __restrict__ tiles, int ntiles,
-                                                             long out_stride, int bx, int by, int bz, int nbx,
-                                                             int nby, FmaK K) {
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const Tile T = tiles[t];
-    const int n = T.nx * T.ny * T.nz;
-    for (int q = threadIdx.x; q < n; q += blockDim.x) {
-      const int ax = T.x0 + q % T.nx, ay = T.y0 + (q / T.nx) % T.ny, az = T.z0 + q / (T.nx * T.ny);
-      const long o = (long)az * sz + (long)ay * sy + ax;
-      const long cell = ((long)(az - bz) * nby + (ay - by)) * nbx + (ax - bx);
+// out[c * out_stride + cell], cells numbered x-fastest within the box.  The
+// FP64 form, for the cells that the fixed-point form does not take.
+__device__ __noinline__ void z4c_constraints_fp64(const double* __restrict__ Y, const double* __restrict__ S, long fs,
+                                                  long o, Z4cParams P, DerivScales ds, double* out, FmaK K) {
 #define FLD(f) Y[(long)(f) * fs + o]
 #define D1(f, d) (ds.s1 * S[(long)(Q_D1 + 3 * (f) + (d)) * fs + o])
-      double rhs[kNZ4c], diag[3];
-      z4c_rhs_point<true>(Y, S, fs, o, P, P.eta, ds, rhs, diag, K);
-      out[cell] = diag[0] + (2.0 / 3.0) * diag[2] * diag[2] - diag[1];
-      double g[6], A[6], gu[6];
-      for (int s = 0; s < 6; ++s) {
-        g[s] = FLD(ZG + s);
-        A[s] = FLD(ZA + s);
-      }
-      gu[0] = fma(g[3], g[5], -g[4] * g[4]);
-      gu[1] = fma(g[2], g[4], -g[1] * g[5]);
-      gu[2] = fma(g[1], g[4], -g[2] * g[3]);
-      gu[3] = fma(g[0], g[5], -g[2] * g[2]);
-      gu[4] = fma(g[1], g[2], -g[0] * g[4]);
-      gu[5] = fma(g[0], g[3], -g[1] * g[1]);
-      const double idet = 1.0 / fma(g[0], gu[0], fma(g[1], gu[1], g[2] * gu[2]));
-      for (int s = 0; s < 6; ++s) gu[s] *= idet;
-      const double iW = 1.0 / FLD(ZW);
-      double Gu[3][6];
-      for (int k = 0; k < 3; ++k)
-        for (int a = 0; a < 3; ++a)
-          for (int b = a; b < 3; ++b) {
-            double v = 0.0;
-            for (int l = 0; l < 3; ++l)
-              v += gu[sidx(k, l)] * 0.5 * (D1(ZG + sidx(b, l), a) + D1(ZG + sidx(a, l), b) - D1(ZG + sidx(a, b), l));
-            Gu[k][sidx(a, b)] = v;
-          }
-      double Auu[3][3];
-      for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) {
-          double v = 0.0;
-          for (int c = 0; c < 3; ++c)
-            for (int d = 0; d < 3; ++d) v += gu[sidx(a, c)] * gu[sidx(b, d)] * A[sidx(c, d)];
-          Auu[a][b] = v;
-        }
-      double dgu[3][6];  // d_m gt^{ab} = -gt^{ac} gt^{bd} d_m gt_cd
-      for (int m = 0; m < 3; ++m)
-        for (int a = 0; a < 3; ++a)
-          for (int b = a; b < 3; ++b) {
-            double v = 0.0;
-            for (int c = 0; c < 3; ++c)
-              for (int d = 0; d < 3; ++d) v -= gu[sidx(a, c)] * gu[sidx(b, d)] * D1(ZG + sidx(c, d), m);
-            dgu[m][sidx(a, b)] = v;
-          }
-      for (int a = 0; a < 3; ++a) {
+  double rhs[kNZ4c], diag[3];
+  z4c_rhs_point<true>(Y, S, fs, o, P, P.eta, ds, rhs, diag, K);
+  out[0] = diag[0] + (2.0 / 3.0) * diag[2] * diag[2] - diag[1];
+  double g[6], A[6], gu[6];
+  for (int s = 0; s < 6; ++s) {
+    g[s] = FLD(ZG + s);
+    A[s] = FLD(ZA + s);
+  }
+  gu[0] = fma(g[3], g[5], -g[4] * g[4]);
+  gu[1] = fma(g[2], g[4], -g[1] * g[5]);
+  gu[2] = fma(g[1], g[4], -g[2] * g[3]);
+  gu[3] = fma(g[0], g[5], -g[2] * g[2]);
+  gu[4] = fma(g[1], g[2], -g[0] * g[4]);
+  gu[5] = fma(g[0], g[3], -g[1] * g[1]);
+  const double idet = 1.0 / fma(g[0], gu[0], fma(g[1], gu[1], g[2] * gu[2]));
+  for (int s = 0; s < 6; ++s) gu[s] *= idet;
+  const double iW = 1.0 / FLD(ZW);
+  double Gu[3][6];
+  for (int k = 0; k < 3; ++k)
+    for (int a = 0; a < 3; ++a)
+      for (int b = a; b < 3; ++b) {
         double v = 0.0;
-        for (int j = 0; j < 3; ++j)  // d_j At^{aj}
-          for (int m = 0; m < 3; ++m)
-            for (int p = 0; p < 3; ++p)
-              v += dgu[j][sidx(a, m)] * gu[sidx(j, p)] * A[sidx(m, p)] +
-                   gu[sidx(a, m)] * dgu[j][sidx(j, p)] * A[sidx(m, p)] +
-                   gu[sidx(a, m)] * gu[sidx(j, p)] * D1(ZA + sidx(m, p), j);
-        for (int b = 0; b < 3; ++b)
-          for (int c = 0; c < 3; ++c) v += Gu[a][sidx(b, c)] * Auu[b][c];
-        for (int b = 0; b < 3; ++b) {
-          v -= 3.0 * Auu[a][b] * D1(ZW, b) * iW;
-          v -= (2.0 / 3.0) * gu[sidx(a, b)] * (D1(ZK, b) + 2.0 * D1(ZTH, b));
-        }
-        out[(1 + a) * out_stride + cell] = v;
-        double gd = 0.0;
-        for (int b = 0; b < 3; ++b)
-          for (int c = 0; c < 3; ++c) gd += gu[sidx(b, c)] * Gu[a][sidx(b, c)];
-        out[(4 + a) * out_stride + cell] = FLD(ZGAM + a) - gd;
+        for (int l = 0; l < 3; ++l)
+          v += gu[sidx(k, l)] * 0.5 * (D1(ZG + sidx(b, l), a) + D1(ZG + sidx(a, l), b) - D1(ZG + sidx(a, b), l));
+        Gu[k][sidx(a, b)] = v;
       }
+  double Auu[3][3];
+  for (int a = 0; a < 3; ++a)
+    for (int b = 0; b < 3; ++b) {
+      double v = 0.0;
+      for (int c = 0; c < 3; ++c)
+        for (int d = 0; d < 3; ++d) v += gu[sidx(a, c)] * gu[sidx(b, d)] * A[sidx(c, d)];
+      Auu[a][b] = v;
+    }
+  double dgu[3][6];  // d_m gt^{ab} = -gt^{ac} gt^{bd} d_m gt_cd
+  for (int m = 0; m < 3; ++m)
+    for (int a = 0; a < 3; ++a)
+      for (int b = a; b < 3; ++b) {
+        double v = 0.0;
+        for (int c = 0; c < 3; ++c)
+          for (int d = 0; d < 3; ++d) v -= gu[sidx(a, c)] * gu[sidx(b, d)] * D1(ZG + sidx(c, d), m);
+        dgu[m][sidx(a, b)] = v;
+      }
+  for (int a = 0; a < 3; ++a) {
+    double v = 0.0;
+    for (int j = 0; j < 3; ++j)  // d_j At^{aj}
+      for (int m = 0; m < 3; ++m)
+        for (int p = 0; p < 3; ++p)
+          v += dgu[j][sidx(a, m)] * gu[sidx(j, p)] * A[sidx(m, p)] +
+               gu[sidx(a, m)] * dgu[j][sidx(j, p)] * A[sidx(m, p)] +
+               gu[sidx(a, m)] * gu[sidx(j, p)] * D1(ZA + sidx(m, p), j);
+    for (int b = 0; b < 3; ++b)
+      for (int c = 0; c < 3; ++c) v += Gu[a][sidx(b, c)] * Auu[b][c];
+    for (int b = 0; b < 3; ++b) {
+      v -= 3.0 * Auu[a][b] * D1(ZW, b) * iW;
+      v -= (2.0 / 3.0) * gu[sidx(a, b)] * (D1(ZK, b) + 2.0 * D1(ZTH, b));
+    }
+    out[1 + a] = v;
+    double gd = 0.0;
+    for (int b = 0; b < 3; ++b)
+      for (int c = 0; c < 3; ++c) gd += gu[sidx(b, c)] * Gu[a][sidx(b, c)];
+    out[4 + a] = FLD(ZGAM + a) - gd;
+  }
 #undef FLD
 #undef D1
+}
+
+// One thread per cell of the box, 64 cells a block, so that an 11,000-cell box
+// reaches every SM.  Bound by the latency of one warp's instructions on such a box.
+__global__ void __launch_bounds__(kRunCells, 4)
+    z4c_constraints_kernel(const double* __restrict__ Y, const double* __restrict__ S, double* __restrict__ out, long fs,
+                           int sy, int sz, Z4cParams P, DerivScales ds, long out_stride, int bx, int by, int bz, int nbx,
+                           int nby, int nbz, const __grid_constant__ FxScales c, FmaK K) {
+  __shared__ long long slots[FM_SLOTS * kRunCells];
+  const FxMem<kRunCells> mem{slots + threadIdx.x};
+  const long cells = (long)nbx * nby * nbz;
+  for (long cell = (long)blockIdx.x * kRunCells + threadIdx.x; cell < cells; cell += (long)gridDim.x * kRunCells) {
+    const int x = (int)(cell % nbx), y = (int)(cell / nbx % nby), z = (int)(cell / ((long)nbx * nby));
+    const long o = (long)(bz + z) * sz + (long)(by + y) * sy + bx + x;
+    struct Out {
+      double* p;
+      long stride;
+      struct Pre {};
+      __device__ __forceinline__ void operator()(int q, double v) const { p[q * stride] = v; }
+    };
+    if (!z4c_rhs_fixed<true>(Y, S, fs, o, P, 0.0, c, mem, K, Out{out + cell, out_stride})) {
+      double v[kNCons];
+      z4c_constraints_fp64(Y, S, fs, o, P, ds, v, K);
+      for (int q = 0; q < kNCons; ++q) out[q * out_stride + cell] = v[q];
     }
   }
 }
@@ -974,12 +988,13 @@ cudaError_t launch_z4c_stage(const StageArgs& a, const double* scratch, const Z4
 }
 
 cudaError_t launch_z4c_constraints(const double* Y, const double* scratch, double* out, long fs, int sy, int sz,
-                                   const Z4cParams& p, const DerivScales& ds, const Tile* tiles, int ntiles,
-                                   long out_stride, const int* box_lo, const int* box_n, cudaStream_t s) {
-  if (ntiles == 0) return cudaSuccess;
-  const int grid = ntiles < sm_count() * 16 ? ntiles : sm_count() * 16;
-  z4c_constraints_kernel<<<grid, 128, 0, s>>>(Y, scratch, out, fs, sy, sz, p, ds, tiles, ntiles, out_stride, box_lo[0],
-                                              box_lo[1], box_lo[2], box_n[0], box_n[1], FmaK{1.0, -1.0, -0.0});
+                                   const Z4cParams& p, const DerivScales& ds, long out_stride, const int* box_lo,
+                                   const int* box_n, cudaStream_t s) {
+  const long blocks = ((long)box_n[0] * box_n[1] * box_n[2] + kRunCells - 1) / kRunCells;
+  const int grid = (int)(blocks < sm_count() * 16L ? blocks : sm_count() * 16L);
+  z4c_constraints_kernel<<<grid, kRunCells, 0, s>>>(Y, scratch, out, fs, sy, sz, p, ds, out_stride, box_lo[0],
+                                                    box_lo[1], box_lo[2], box_n[0], box_n[1], box_n[2], fx_scales(ds),
+                                                    FmaK{1.0, -1.0, -0.0});
   return cudaGetLastError();
 }
 

@@ -410,7 +410,12 @@ enum {
 // FP64.  So the tensors that several loops share live in shared memory, and
 // the loops over tensor components are rolled: 0.327 ms, and 0.269 with the
 // global loads issued a loop iteration or a section ahead.
-template <int T, class KT, class OUT>
+// CONS: instead of the right-hand side the seven constraints of
+// z4c_constraints_kernel, out(q, value), from the same Ricci tensor; with
+// d_k gt_ij = Gamma_{i,jk} + Gamma_{j,ik} and At^ij's own derivatives,
+//   M^i = gt^im (gt^jp d_j At_mp - Gamma^n_mj At_n^j) - At^id Gamma^j_dj - At^i_p (Gamma_d)^p
+//         - 3 At^ij d_j W / W - 2/3 gt^ij d_j (Khat + 2 Theta)
+template <bool CONS, int T, class KT, class OUT>
 FXD bool z4c_rhs_fixed(const double* __restrict__ Y, const double* __restrict__ S, long fs, long o, const Z4cParams& P,
                        double eta, const FxScales& c, const FxMem<T>& mem, const KT& K, const OUT& out) {
 #define FLD(f) Y[(long)(f) * fs + o]
@@ -701,112 +706,32 @@ FXD bool z4c_rhs_fixed(const double* __restrict__ Y, const double* __restrict__ 
     mem.stm(FM_DDW + s, e);
     em = em > e ? em : e;
   }
-  // second derivatives of the shift: gt^jk d_j d_k beta^i + 1/3 gt^ij d_j d_k beta^k
-  int eTB;
-  {
-    const FxBlk<18> h = fx_load<59, 18>(xbe, bad, c.poff);
-    FxSum<3> dv, sB, sL;
-    dv.e = h.e + c.kP3.e + 61;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      FxDot d;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) d.mac(h.v[6 * k + sidx(j, k)], j == k ? c.kP3.v : c.kM3.v);
-      dv.m[j] = d.fin<61>();  // 58.6
-    }
-    const FxBlk<3> ddivb = fx_norm<59>(dv);  // 1/3 d_j d_k beta^k
-    sL.e = gu.e + ddivb.e + 61;
-    sB.e = guk.e + h.e + 61;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      sL.m[i] = fx_row(gu, i, ddivb.v).fin<61>();        // 58.6
-      sB.m[i] = fx_trace(guk.v, h.v + 6 * i).fin<61>();  // 60.2
-    }
-    fx_add(sB, sL);
-    eTB = sB.e;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) mem.stm(FM_TB + i, sB.m[i]);  // 60.6
-  }
-  double xA[6], xdb[9];
-#pragma unroll
-  for (int s = 0; s < 6; ++s) xA[s] = FLD(ZA + s);
-#pragma unroll
-  for (int q = 0; q < 9; ++q) xdb[q] = D1(ZB + q / 3, q % 3);
-  const FxBlk<1> fal = scalar(al);
-  double trR, trDDa;
-  int eTF;
-  {
-    FxBlk<6> R, DDa;
-    FxSum<6> a, b, w;
+  if constexpr (CONS) {
+    FxSum<6> a;
     a.e = em;
 #pragma unroll
     for (int s = 0; s < 6; ++s) a.m[s] = fx_shr(mem.ldm(FM_R + s), em - (int)mem.ldm(FM_DDW + s));
-    R = fx_norm_any(a);
-    // D_i D_j alpha with Gamma^k_ij - (delta^k_i d_j W + delta^k_j d_i W - gt_ij gt^kl d_l W) / W
-    FxSum<1> zz;
-    zz.m[0] = fx_dot3(gdWi.v, dal.v).fin<61>();
-    zz.e = gdWi.e + dal.e + 61;
-    const FxBlk<1> za = fx_norm<59>(zz);
-    const FxBlk<6> h = fx_load<59, 6>(xh.v, bad, c.poff);
-    a.e = h.e + c.kP.e + 59;
-    b.e = eGu + dal.e + 60;
-    w.e = dWi.e + dal.e + 60;
+    const FxBlk<6> R = fx_norm_any(a);
+    const double trR = fx_double(fx_trace(gu.v, R.v).fin<63>(), gu.e + R.e + 63);
+    double x[6], xg[3], xd[18], xk[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int s = 0; s < 6; ++s) x[s] = FLD(ZA + s);
 #pragma unroll
-      for (int j = i; j < 3; ++j) {
-        const int s = sidx(i, j);
-        FxDot p, q, u;
-        p.mac(h.v[s], fx_pure(s) ? c.kP.v : c.kM.v);
-        a.m[s] = p.fin<59>();  // 59
+    for (int q = 0; q < 18; ++q) xd[q] = D1(ZA + q / 3, q % 3);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) q.mac(mem.ld(FM_GU + 6 * k + s), dal.v[k]);
-        b.m[s] = -q.fin<60>();  // 59.6
-        u.mac(dWi.v[j], dal.v[i]);
-        u.mac(dWi.v[i], dal.v[j]);
-        w.m[s] = u.fin<60>();  // 59
-      }
-    fx_add(a, b);
-    fx_add(a, w);
-    const FxBlk<6> g = mem.template get<6>(FM_G, eG);
-    b = fx_times<60>(g, za.v[0], za.e);  // 58
-#pragma unroll
-    for (int s = 0; s < 6; ++s) b.m[s] = -b.m[s];
-    fx_add(a, b);  // 61
-    DDa = fx_norm_any(a);
-    trR = fx_double(fx_trace(gu.v, R.v).fin<63>(), gu.e + R.e + 63);
-    trDDa = fx_double(fx_trace(gu.v, DDa.v).fin<63>(), gu.e + DDa.e + 63);
-    // the trace-free part of alpha R_ij - D_i D_j alpha
-    const FxBlk<1> zt = scalar(fmul(-1.0 / 3.0, fma(al, trR, -trDDa), K));
-    a = fx_times<59>(R, fal.v[0], fal.e);
-    b = fx_times<59>(g, zt.v[0], zt.e);
-    fx_add(a, b);
-    b.e = DDa.e;
-#pragma unroll
-    for (int s = 0; s < 6; ++s) b.m[s] = -fx_join(DDa.v[s]);
-    fx_add(a, b);
-    const FxBlk<6> tf = fx_norm_any(a);  // from 60.6
-    mem.put(FM_TF, tf);
-    eTF = tf.e;
-  }
-  const double W2 = fmul(W, W, K), Kt = fma(2.0, Th, Kh);
-
-  const X3 xK = get_d1(ZK), xT = get_d1(ZTH);
-  const double be[3] = {FLD(ZB), FLD(ZB + 1), FLD(ZB + 2)};
-  const double gam[3] = {FLD(ZGAM), FLD(ZGAM + 1), FLD(ZGAM + 2)};
-  // At with raised indices: Am[3 i + j] = At^i_j, Auu = At^ij
-  double AA;
-  int eA, eAU, eAB;
-  {
-    const FxBlk<6> A = fx_load<59, 6>(xA, bad);
-    FxSum<9> m, kt;
+    for (int i = 0; i < 3; ++i) {
+      xg[i] = FLD(ZGAM + i);
+      xk[i] = fma(2.0, D1(ZTH, i), D1(ZK, i));
+    }
+    const FxBlk<6> A = fx_load<59, 6>(x, bad);
+    FxSum<9> m;
     m.e = gu.e + A.e + 61;
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
       const FxP b[3] = {A.v[sidx(0, q % 3)], A.v[sidx(1, q % 3)], A.v[sidx(2, q % 3)]};
       m.m[q] = fx_row(gu, q / 3, b).fin<61>();  // 58.6
     }
-    const FxBlk<9> Am = fx_norm<59>(m);
+    const FxBlk<9> Am = fx_norm<59>(m);  // At^i_j, 3 i + j
     FxSum<6> u;
     u.e = gu.e + Am.e + 61;
 #pragma unroll
@@ -814,190 +739,360 @@ FXD bool z4c_rhs_fixed(const double* __restrict__ Y, const double* __restrict__ 
 #pragma unroll
       for (int j = i; j < 3; ++j) u.m[sidx(i, j)] = fx_row(gu, j, Am.v + 3 * i).fin<61>();
     const FxBlk<6> Auu = fx_norm<59>(u);
-    AA = fx_double(fx_trace(A.v, Auu.v).fin<63>(), A.e + Auu.e + 63);
-    // (Kt delta^k_i - 2 At^k_i) At_kj
-    const FxBlk<1> fKt = scalar(Kt);
-    m.e = Am.e + 1;
-    kt.e = fKt.e;
+    const double AA = fx_double(fx_trace(A.v, Auu.v).fin<63>(), A.e + Auu.e + 63), Kt = fma(2.0, Th, Kh);
+    out(0, fma(fmul(W, W, K), trR, fma(fmul(2.0 / 3.0, Kt, K), Kt, -AA)));
+    const FxBlk<18> dA = fx_load<59, 18>(xd, bad);
+    const FxBlk<6> gs = fx_norm<59>(fx_times<60>(gu, c.s1.v, c.s1.e));
+    const FxBlk<3> dd = fx_norm<59>(fx_times<60>(fx_load<59, 3>(xk, bad), c.ts1.v, c.ts1.e + 1));
+    FxSum<3> t, b, d;
+    t.e = eGu;
+    b.e = gs.e + dA.e + 62;
+    d.e = eGu + Am.e + 62;
 #pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      m.m[q] = -fx_join(Am.v[q]);
-      kt.m[q] = q % 4 == 0 ? fx_join(fKt.v[0]) : 0;
+    for (int i = 0; i < 3; ++i) {
+      FxDot p, q;
+      t.m[i] = 0;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          p.mac(gs.v[sidx(j, k)], dA.v[3 * sidx(i, k) + j]);
+          q.mac(mem.ld(FM_GU + 6 * k + sidx(i, j)), Am.v[3 * j + k]);
+        }
+        t.m[i] += fx_join(mem.ld(FM_GU + 6 * j + sidx(i, j)));  // Gamma^j_ij, 60.6
+      }
+      b.m[i] = p.fin<62>();   // 59.2
+      d.m[i] = -q.fin<62>();  // 59.2
     }
-    fx_add(m, kt);
-    const FxBlk<9> ak = fx_norm_any(m);
-    u.e = ak.e + A.e + 61;
+    fx_add(b, d);
+    const FxBlk<3> bn = fx_norm_any(b), tn = fx_norm_any(t);
+    FxSum<3> M, v;
+    M.e = gu.e + bn.e + 61;
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int i = 0; i < 3; ++i) M.m[i] = fx_row(gu, i, bn.v).fin<61>();  // 58.6
+    auto less = [&](const FxBlk<6>& a6, const FxBlk<3>& w, int times) {
+      v.e = a6.e + w.e + 61;
 #pragma unroll
-      for (int j = i; j < 3; ++j) {
+      for (int i = 0; i < 3; ++i) v.m[i] = -times * fx_row(a6, i, w.v).fin<61>();
+      fx_add(M, v);
+    };
+    less(Auu, tn, 1);
+    less(Auu, dWi, 3);  // 60.2
+    less(gu, dd, 1);
+    v.e = Am.e + Gd.e + 61;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) v.m[i] = -fx_dot3(Am.v + 3 * i, Gd.v).fin<61>();
+    fx_add(M, v);
+    fx_load_raw<59, 3>(xg, t, bad);
+    v.e = Gd.e;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) v.m[i] = -fx_join(Gd.v[i]);
+    fx_add(t, v);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      out(1 + i, fx_double(M.m[i], M.e));
+      out(4 + i, fx_double(t.m[i], t.e));
+    }
+    return !bad;
+  } else {
+    // second derivatives of the shift: gt^jk d_j d_k beta^i + 1/3 gt^ij d_j d_k beta^k
+    int eTB;
+    {
+      const FxBlk<18> h = fx_load<59, 18>(xbe, bad, c.poff);
+      FxSum<3> dv, sB, sL;
+      dv.e = h.e + c.kP3.e + 61;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
         FxDot d;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) d.mac(ak.v[3 * k + i], A.v[sidx(k, j)]);
-        u.m[sidx(i, j)] = d.fin<61>();  // 58.6
+        for (int k = 0; k < 3; ++k) d.mac(h.v[6 * k + sidx(j, k)], j == k ? c.kP3.v : c.kM3.v);
+        dv.m[j] = d.fin<61>();  // 58.6
       }
-    const FxBlk<6> ab = fx_norm<59>(u);
-    mem.put(FM_A, A);
-    mem.put(FM_AU, Auu);
-    mem.put(FM_AB, ab);
-    eA = A.e;
-    eAU = Auu.e;
-    eAB = ab.e;
-  }
-
-  // d_j beta^i, its trace, and -2/3 of that
-  FxP p23, m23;
-  double divb;
-  int eDB;
-  {
-    const FxBlk<9> db = fx_norm<59>(fx_times<60>(fx_load<59, 9>(xdb, bad), c.s1.v, c.s1.e));
-    const long long t = fx_join(db.v[0]) + fx_join(db.v[4]) + fx_join(db.v[8]);  // 60.6
-    divb = fx_double(t, db.e);
-    FxDot d;
-    d.mac(fx_split(t), c.twothird.v);
-    const long long u = d.fin<59>();  // 60, the units of db
-    p23 = fx_split(u);
-    m23 = fx_split(-u);
-    mem.put(FM_DB, db);
-    eDB = db.e;
-  }
-  // beta^i s1, for the advection terms
-  const FxBlk<3> bes = fx_norm<59>(fx_times<60>(fx_load<59, 3>(be, bad), c.s1.v, c.s1.e));
-  // The loops from here on finish one field after the other; next holds the
-  // coming field's first derivatives and what out needs of it.
-  struct Next {
-    X3 d;
-    typename OUT::Pre p;
-  };
-  auto get = [&](int f) { return Next{get_d1(f), out.load(f)}; };
-  Next next = get(ZGAM);
-  auto adv = [&](const X3& x, long long& m, int& e) {  // beta^i d_i f
-    const FxBlk<3> d = fx_load<59, 3>(x.v, bad);
-    m = fx_dot3(bes.v, d.v).fin<61>();  // 58.6
-    e = bes.e + d.e + 61;
-  };
-
-  // Gamt^i
-  {
-    double x[3];
+      const FxBlk<3> ddivb = fx_norm<59>(dv);  // 1/3 d_j d_k beta^k
+      sL.e = gu.e + ddivb.e + 61;
+      sB.e = guk.e + h.e + 61;
 #pragma unroll
-    for (int j = 0; j < 3; ++j) x[j] = fma(2.0, xK.v[j], xT.v[j]);  // d_j (2 Khat + Theta)
-    const FxBlk<3> dd = fx_norm<59>(fx_times<60>(fx_load<59, 3>(x, bad), c.ts1.v, c.ts1.e));
-    const FxBlk<6> Auu = mem.template get<6>(FM_AU, eAU);
-    const FxBlk<1> k2 = scalar(fmul(-2.0 * P.kappa1, al, K));
-#pragma unroll 1
-    for (int i = 0; i < 3; ++i) {
-      const Next now = next;
-      next = get(i < 2 ? ZGAM + 1 + i : ZG);
-      const double gami = i == 0 ? gam[0] : i == 1 ? gam[1] : gam[2];
-      FxP v[6], r[3], ra[3];
+      for (int i = 0; i < 3; ++i) {
+        sL.m[i] = fx_row(gu, i, ddivb.v).fin<61>();        // 58.6
+        sB.m[i] = fx_trace(guk.v, h.v + 6 * i).fin<61>();  // 60.2
+      }
+      fx_add(sB, sL);
+      eTB = sB.e;
 #pragma unroll
-      for (int s = 0; s < 6; ++s) v[s] = mem.ld(FM_GU + 6 * i + s);
-      mem.row(FM_GI, i, r);
-      mem.row(FM_AU, i, ra);
-      FxSum<1> br, t;
-      br.m[0] = fx_trace(v, Auu.v).fin<62>();  // Gamt^i_jk At^jk, 59.2
-      br.e = eGu + Auu.e + 62;
-      t.m[0] = -3 * fx_dot3(ra, dWi.v).fin<61>();  // 60.2
-      t.e = Auu.e + dWi.e + 61;
-      fx_add(br, t);
-      t.m[0] = -fx_dot3(r, dd.v).fin<61>();  // 58.6
-      t.e = gu.e + dd.e + 61;
-      fx_add(br, t);
-      const FxBlk<1> b = fx_norm_any(br);
-      long long m;
-      int e;
-      adv(now.d, m, e);
-      fx_add1(m, e, fx_times<59>(b, fal.v[0], 0).m[0], b.e + fal.e + 60);       // 2 alpha (...), 59
-      fx_add1(m, e, -fx_dot3(ra, dal.v).fin<61>(), Auu.e + dal.e + 62);         // -2 At^ij d_j alpha, 58.6
-      fx_add1(m, e, mem.ldm(FM_TB + i), eTB);                                   // 60.6
-      const FxP gd = mem.ld(FM_GD + i);
-      FxDot p;  // 2/3 (Gamma_d)^i div beta - (Gamma_d)^j d_j beta^i
-      p.mac(gd, p23);
-      const FxP w[3] = {mem.ld(FM_DB + 3 * i), mem.ld(FM_DB + 3 * i + 1), mem.ld(FM_DB + 3 * i + 2)};
-      p.sub(fx_dot3(Gd.v, w));
-      fx_add1(m, e, p.fin<60>(), Gd.e + eDB + 60);  // 60.4
-      // -2 kappa1 alpha (Gamt^i - (Gamma_d)^i)
-      FxSum<1> gm, gc;
-      fx_load_raw<59, 1>(&gami, gm, bad);
-      gc.m[0] = -fx_join(gd);
-      gc.e = Gd.e;
-      fx_add(gm, gc);
-      const FxBlk<1> gn = fx_norm_any(gm);
-      fx_add1(m, e, fx_times<60>(gn, k2.v[0], 0).m[0], gn.e + k2.e + 60);  // 58, 62 in all
-      out(ZGAM + i, fx_double(m, e), now.p);
+      for (int i = 0; i < 3; ++i) mem.stm(FM_TB + i, sB.m[i]);  // 60.6
     }
-  }
-  // gt_ij and At_ij
-  {
-    const FxBlk<1> fW2 = scalar(W2);
-#pragma unroll 1
-    for (int s = 0; s < 6; ++s) {
-      const int i = fx_slot_i(s), j = fx_slot_j(s);
-      Next now = next;
-      next = get(ZA + s);
-      FxP ri[3], rj[3];
-      const FxP di[3] = {mem.ld(FM_DB + i), mem.ld(FM_DB + 3 + i), mem.ld(FM_DB + 6 + i)};
-      const FxP dj[3] = {mem.ld(FM_DB + j), mem.ld(FM_DB + 3 + j), mem.ld(FM_DB + 6 + j)};
-      const FxP A = mem.ld(FM_A + s);
-      long long m;
-      int e;
-      FxDot l, p, q, w;
-      mem.row(FM_G, i, ri);
-      mem.row(FM_G, j, rj);
-      l = fx_dot3(ri, dj);
-      l.add(fx_dot3(rj, di));
-      l.mac(mem.ld(FM_G + s), m23);
-      adv(now.d, m, e);
-      fx_add1(m, e, l.fin<60>(), eG + eDB + 60);  // 61
-      p.mac(fal.v[0], A);
-      fx_add1(m, e, -p.fin<60>(), fal.e + eA + 61);  // 58
-      out(ZG + s, fx_double(m, e), now.p);
-      now = next;
-      next = get(s < 5 ? ZG + 1 + s : ZW);
-      mem.row(FM_A, i, ri);
-      mem.row(FM_A, j, rj);
-      l = fx_dot3(ri, dj);
-      l.add(fx_dot3(rj, di));
-      l.mac(A, m23);
-      adv(now.d, m, e);
-      fx_add1(m, e, l.fin<60>(), eA + eDB + 60);  // 61
-      q.mac(fal.v[0], mem.ld(FM_AB + s));
-      fx_add1(m, e, q.fin<59>(), fal.e + eAB + 59);  // 59
-      w.mac(fW2.v[0], mem.ld(FM_TF + s));
-      fx_add1(m, e, w.fin<59>(), fW2.e + eTF + 59);  // 59
-      out(ZA + s, fx_double(m, e), now.p);
+    double xA[6], xdb[9];
+#pragma unroll
+    for (int s = 0; s < 6; ++s) xA[s] = FLD(ZA + s);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) xdb[q] = D1(ZB + q / 3, q % 3);
+    const FxBlk<1> fal = scalar(al);
+    double trR, trDDa;
+    int eTF;
+    {
+      FxBlk<6> R, DDa;
+      FxSum<6> a, b, w;
+      a.e = em;
+#pragma unroll
+      for (int s = 0; s < 6; ++s) a.m[s] = fx_shr(mem.ldm(FM_R + s), em - (int)mem.ldm(FM_DDW + s));
+      R = fx_norm_any(a);
+      // D_i D_j alpha with Gamma^k_ij - (delta^k_i d_j W + delta^k_j d_i W - gt_ij gt^kl d_l W) / W
+      FxSum<1> zz;
+      zz.m[0] = fx_dot3(gdWi.v, dal.v).fin<61>();
+      zz.e = gdWi.e + dal.e + 61;
+      const FxBlk<1> za = fx_norm<59>(zz);
+      const FxBlk<6> h = fx_load<59, 6>(xh.v, bad, c.poff);
+      a.e = h.e + c.kP.e + 59;
+      b.e = eGu + dal.e + 60;
+      w.e = dWi.e + dal.e + 60;
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = i; j < 3; ++j) {
+          const int s = sidx(i, j);
+          FxDot p, q, u;
+          p.mac(h.v[s], fx_pure(s) ? c.kP.v : c.kM.v);
+          a.m[s] = p.fin<59>();  // 59
+#pragma unroll
+          for (int k = 0; k < 3; ++k) q.mac(mem.ld(FM_GU + 6 * k + s), dal.v[k]);
+          b.m[s] = -q.fin<60>();  // 59.6
+          u.mac(dWi.v[j], dal.v[i]);
+          u.mac(dWi.v[i], dal.v[j]);
+          w.m[s] = u.fin<60>();  // 59
+        }
+      fx_add(a, b);
+      fx_add(a, w);
+      const FxBlk<6> g = mem.template get<6>(FM_G, eG);
+      b = fx_times<60>(g, za.v[0], za.e);  // 58
+#pragma unroll
+      for (int s = 0; s < 6; ++s) b.m[s] = -b.m[s];
+      fx_add(a, b);  // 61
+      DDa = fx_norm_any(a);
+      trR = fx_double(fx_trace(gu.v, R.v).fin<63>(), gu.e + R.e + 63);
+      trDDa = fx_double(fx_trace(gu.v, DDa.v).fin<63>(), gu.e + DDa.e + 63);
+      // the trace-free part of alpha R_ij - D_i D_j alpha
+      const FxBlk<1> zt = scalar(fmul(-1.0 / 3.0, fma(al, trR, -trDDa), K));
+      a = fx_times<59>(R, fal.v[0], fal.e);
+      b = fx_times<59>(g, zt.v[0], zt.e);
+      fx_add(a, b);
+      b.e = DDa.e;
+#pragma unroll
+      for (int s = 0; s < 6; ++s) b.m[s] = -fx_join(DDa.v[s]);
+      fx_add(a, b);
+      const FxBlk<6> tf = fx_norm_any(a);  // from 60.6
+      mem.put(FM_TF, tf);
+      eTF = tf.e;
     }
-  }
-  // W, Khat, Theta, alpha and beta^i: the scalar parts in FP64
-  {
-    const double third = 1.0 / 3.0, twothird = 2.0 / 3.0;
-    auto put = [&](int q, double v) {
-      mem.stm(FM_GU + q, fx_shl((long long)fx_dhi(v), 32) | fx_dlo(v));
+    const double W2 = fmul(W, W, K), Kt = fma(2.0, Th, Kh);
+
+    const X3 xK = get_d1(ZK), xT = get_d1(ZTH);
+    const double be[3] = {FLD(ZB), FLD(ZB + 1), FLD(ZB + 2)};
+    const double gam[3] = {FLD(ZGAM), FLD(ZGAM + 1), FLD(ZGAM + 2)};
+    // At with raised indices: Am[3 i + j] = At^i_j, Auu = At^ij
+    double AA;
+    int eA, eAU, eAB;
+    {
+      const FxBlk<6> A = fx_load<59, 6>(xA, bad);
+      FxSum<9> m, kt;
+      m.e = gu.e + A.e + 61;
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        const FxP b[3] = {A.v[sidx(0, q % 3)], A.v[sidx(1, q % 3)], A.v[sidx(2, q % 3)]};
+        m.m[q] = fx_row(gu, q / 3, b).fin<61>();  // 58.6
+      }
+      const FxBlk<9> Am = fx_norm<59>(m);
+      FxSum<6> u;
+      u.e = gu.e + Am.e + 61;
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = i; j < 3; ++j) u.m[sidx(i, j)] = fx_row(gu, j, Am.v + 3 * i).fin<61>();
+      const FxBlk<6> Auu = fx_norm<59>(u);
+      AA = fx_double(fx_trace(A.v, Auu.v).fin<63>(), A.e + Auu.e + 63);
+      // (Kt delta^k_i - 2 At^k_i) At_kj
+      const FxBlk<1> fKt = scalar(Kt);
+      m.e = Am.e + 1;
+      kt.e = fKt.e;
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        m.m[q] = -fx_join(Am.v[q]);
+        kt.m[q] = q % 4 == 0 ? fx_join(fKt.v[0]) : 0;
+      }
+      fx_add(m, kt);
+      const FxBlk<9> ak = fx_norm_any(m);
+      u.e = ak.e + A.e + 61;
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = i; j < 3; ++j) {
+          FxDot d;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) d.mac(ak.v[3 * k + i], A.v[sidx(k, j)]);
+          u.m[sidx(i, j)] = d.fin<61>();  // 58.6
+        }
+      const FxBlk<6> ab = fx_norm<59>(u);
+      mem.put(FM_A, A);
+      mem.put(FM_AU, Auu);
+      mem.put(FM_AB, ab);
+      eA = A.e;
+      eAU = Auu.e;
+      eAB = ab.e;
+    }
+
+    // d_j beta^i, its trace, and -2/3 of that
+    FxP p23, m23;
+    double divb;
+    int eDB;
+    {
+      const FxBlk<9> db = fx_norm<59>(fx_times<60>(fx_load<59, 9>(xdb, bad), c.s1.v, c.s1.e));
+      const long long t = fx_join(db.v[0]) + fx_join(db.v[4]) + fx_join(db.v[8]);  // 60.6
+      divb = fx_double(t, db.e);
+      FxDot d;
+      d.mac(fx_split(t), c.twothird.v);
+      const long long u = d.fin<59>();  // 60, the units of db
+      p23 = fx_split(u);
+      m23 = fx_split(-u);
+      mem.put(FM_DB, db);
+      eDB = db.e;
+    }
+    // beta^i s1, for the advection terms
+    const FxBlk<3> bes = fx_norm<59>(fx_times<60>(fx_load<59, 3>(be, bad), c.s1.v, c.s1.e));
+    // The loops from here on finish one field after the other; next holds the
+    // coming field's first derivatives and what out needs of it.
+    struct Next {
+      X3 d;
+      typename OUT::Pre p;
     };
-    put(0, fmul(fmul(third, W, K), fma(al, Kt, -divb), K));
-    put(1, fma(al, fma(fmul(third, Kt, K), Kt, AA), fma(fmul(al, P.kappa1 * (1.0 - P.kappa2), K), Th, fmul(-W2, trDDa, K))));
-    put(2, fma(fmul(0.5, al, K), fma(fmul(twothird, Kt, K), Kt, fma(W2, trR, -AA)),
-               fmul(fmul(-al, P.kappa1 * (2.0 + P.kappa2), K), Th, K)));
-    put(3, fmul(fmul(-2.0, al, K), Kh, K));
+    auto get = [&](int f) { return Next{get_d1(f), out.load(f)}; };
+    Next next = get(ZGAM);
+    auto adv = [&](const X3& x, long long& m, int& e) {  // beta^i d_i f
+      const FxBlk<3> d = fx_load<59, 3>(x.v, bad);
+      m = fx_dot3(bes.v, d.v).fin<61>();  // 58.6
+      e = bes.e + d.e + 61;
+    };
+
+    // Gamt^i
+    {
+      double x[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) put(4 + i, fma(0.75, gam[i], fmul(-eta, be[i], K)));
+      for (int j = 0; j < 3; ++j) x[j] = fma(2.0, xK.v[j], xT.v[j]);  // d_j (2 Khat + Theta)
+      const FxBlk<3> dd = fx_norm<59>(fx_times<60>(fx_load<59, 3>(x, bad), c.ts1.v, c.ts1.e));
+      const FxBlk<6> Auu = mem.template get<6>(FM_AU, eAU);
+      const FxBlk<1> k2 = scalar(fmul(-2.0 * P.kappa1, al, K));
 #pragma unroll 1
-    for (int q = 0; q < 7; ++q) {
-      const int f = q < 2 ? 7 * q : q + 15;
-      const Next now = next;
-      next = get(q < 1 ? ZK : q < 6 ? q + 16 : ZB + 2);
-      long long m;
-      int e;
-      adv(now.d, m, e);
-      const long long v = mem.ldm(FM_GU + q);
-      out(f, fadd(fx_make((int)(v >> 32), (int)v), fx_double(m, e), K), now.p);
+      for (int i = 0; i < 3; ++i) {
+        const Next now = next;
+        next = get(i < 2 ? ZGAM + 1 + i : ZG);
+        const double gami = i == 0 ? gam[0] : i == 1 ? gam[1] : gam[2];
+        FxP v[6], r[3], ra[3];
+#pragma unroll
+        for (int s = 0; s < 6; ++s) v[s] = mem.ld(FM_GU + 6 * i + s);
+        mem.row(FM_GI, i, r);
+        mem.row(FM_AU, i, ra);
+        FxSum<1> br, t;
+        br.m[0] = fx_trace(v, Auu.v).fin<62>();  // Gamt^i_jk At^jk, 59.2
+        br.e = eGu + Auu.e + 62;
+        t.m[0] = -3 * fx_dot3(ra, dWi.v).fin<61>();  // 60.2
+        t.e = Auu.e + dWi.e + 61;
+        fx_add(br, t);
+        t.m[0] = -fx_dot3(r, dd.v).fin<61>();  // 58.6
+        t.e = gu.e + dd.e + 61;
+        fx_add(br, t);
+        const FxBlk<1> b = fx_norm_any(br);
+        long long m;
+        int e;
+        adv(now.d, m, e);
+        fx_add1(m, e, fx_times<59>(b, fal.v[0], 0).m[0], b.e + fal.e + 60);       // 2 alpha (...), 59
+        fx_add1(m, e, -fx_dot3(ra, dal.v).fin<61>(), Auu.e + dal.e + 62);         // -2 At^ij d_j alpha, 58.6
+        fx_add1(m, e, mem.ldm(FM_TB + i), eTB);                                   // 60.6
+        const FxP gd = mem.ld(FM_GD + i);
+        FxDot p;  // 2/3 (Gamma_d)^i div beta - (Gamma_d)^j d_j beta^i
+        p.mac(gd, p23);
+        const FxP w[3] = {mem.ld(FM_DB + 3 * i), mem.ld(FM_DB + 3 * i + 1), mem.ld(FM_DB + 3 * i + 2)};
+        p.sub(fx_dot3(Gd.v, w));
+        fx_add1(m, e, p.fin<60>(), Gd.e + eDB + 60);  // 60.4
+        // -2 kappa1 alpha (Gamt^i - (Gamma_d)^i)
+        FxSum<1> gm, gc;
+        fx_load_raw<59, 1>(&gami, gm, bad);
+        gc.m[0] = -fx_join(gd);
+        gc.e = Gd.e;
+        fx_add(gm, gc);
+        const FxBlk<1> gn = fx_norm_any(gm);
+        fx_add1(m, e, fx_times<60>(gn, k2.v[0], 0).m[0], gn.e + k2.e + 60);  // 58, 62 in all
+        out(ZGAM + i, fx_double(m, e), now.p);
+      }
     }
+    // gt_ij and At_ij
+    {
+      const FxBlk<1> fW2 = scalar(W2);
+#pragma unroll 1
+      for (int s = 0; s < 6; ++s) {
+        const int i = fx_slot_i(s), j = fx_slot_j(s);
+        Next now = next;
+        next = get(ZA + s);
+        FxP ri[3], rj[3];
+        const FxP di[3] = {mem.ld(FM_DB + i), mem.ld(FM_DB + 3 + i), mem.ld(FM_DB + 6 + i)};
+        const FxP dj[3] = {mem.ld(FM_DB + j), mem.ld(FM_DB + 3 + j), mem.ld(FM_DB + 6 + j)};
+        const FxP A = mem.ld(FM_A + s);
+        long long m;
+        int e;
+        FxDot l, p, q, w;
+        mem.row(FM_G, i, ri);
+        mem.row(FM_G, j, rj);
+        l = fx_dot3(ri, dj);
+        l.add(fx_dot3(rj, di));
+        l.mac(mem.ld(FM_G + s), m23);
+        adv(now.d, m, e);
+        fx_add1(m, e, l.fin<60>(), eG + eDB + 60);  // 61
+        p.mac(fal.v[0], A);
+        fx_add1(m, e, -p.fin<60>(), fal.e + eA + 61);  // 58
+        out(ZG + s, fx_double(m, e), now.p);
+        now = next;
+        next = get(s < 5 ? ZG + 1 + s : ZW);
+        mem.row(FM_A, i, ri);
+        mem.row(FM_A, j, rj);
+        l = fx_dot3(ri, dj);
+        l.add(fx_dot3(rj, di));
+        l.mac(A, m23);
+        adv(now.d, m, e);
+        fx_add1(m, e, l.fin<60>(), eA + eDB + 60);  // 61
+        q.mac(fal.v[0], mem.ld(FM_AB + s));
+        fx_add1(m, e, q.fin<59>(), fal.e + eAB + 59);  // 59
+        w.mac(fW2.v[0], mem.ld(FM_TF + s));
+        fx_add1(m, e, w.fin<59>(), fW2.e + eTF + 59);  // 59
+        out(ZA + s, fx_double(m, e), now.p);
+      }
+    }
+    // W, Khat, Theta, alpha and beta^i: the scalar parts in FP64
+    {
+      const double third = 1.0 / 3.0, twothird = 2.0 / 3.0;
+      auto put = [&](int q, double v) {
+        mem.stm(FM_GU + q, fx_shl((long long)fx_dhi(v), 32) | fx_dlo(v));
+      };
+      put(0, fmul(fmul(third, W, K), fma(al, Kt, -divb), K));
+      put(1, fma(al, fma(fmul(third, Kt, K), Kt, AA), fma(fmul(al, P.kappa1 * (1.0 - P.kappa2), K), Th, fmul(-W2, trDDa, K))));
+      put(2, fma(fmul(0.5, al, K), fma(fmul(twothird, Kt, K), Kt, fma(W2, trR, -AA)),
+                 fmul(fmul(-al, P.kappa1 * (2.0 + P.kappa2), K), Th, K)));
+      put(3, fmul(fmul(-2.0, al, K), Kh, K));
+#pragma unroll
+      for (int i = 0; i < 3; ++i) put(4 + i, fma(0.75, gam[i], fmul(-eta, be[i], K)));
+#pragma unroll 1
+      for (int q = 0; q < 7; ++q) {
+        const int f = q < 2 ? 7 * q : q + 15;
+        const Next now = next;
+        next = get(q < 1 ? ZK : q < 6 ? q + 16 : ZB + 2);
+        long long m;
+        int e;
+        adv(now.d, m, e);
+        const long long v = mem.ldm(FM_GU + q);
+        out(f, fadd(fx_make((int)(v >> 32), (int)v), fx_double(m, e), K), now.p);
+      }
+    }
+    return !bad;
   }
 #undef FLD
 #undef D1
 #undef D2
-  return !bad;
 }
 
 }  // namespace sc
