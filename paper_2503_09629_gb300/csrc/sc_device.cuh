@@ -87,7 +87,8 @@ __device__ __forceinline__ void prolong_pair(const long long* __restrict__ v, co
   int e[7], mid = 0;
 #pragma unroll
   for (int m = 0; m < 7; ++m) {
-    const int n = min(max(n0 + m, 0), N - 1) * stride;
+    // (n0 is at least -1 and n0 + 5 at most N - 1)
+    const int n = (m == 0 ? max(n0, 0) : m == 6 ? min(n0 + 6, N - 1) : n0 + m) * stride;
     x[m] = v[n];
     e[m] = ve[n];
     if (m > 0 && m < 6) mid = max(mid, e[m]);
@@ -114,19 +115,28 @@ __device__ __forceinline__ void prolong_pair(const long long* __restrict__ v, co
   *elo = E0;
   *ehi = E1;
 }
-// A tile's lines along one axis: lines * pairs work items, line l's nodes at
-// line_base(l) + n * stride, its fine positions written by out(l, i, v, e).
-template <class BASE, class OUT>
+// q / d by a multiplication, exact for q (d - 1) < 65536.
+struct SmallDiv {
+  unsigned m;
+  __device__ __forceinline__ explicit SmallDiv(int d) : m((65535u + (unsigned)d) / (unsigned)d) {}
+  __device__ __forceinline__ int operator()(int q) const { return (int)((unsigned)q * m >> 16); }
+};
+// A tile's lines along one axis: lines * pairs work items (at most 500), line l's
+// nodes at lay(l, &dst) + n * stride, its fine positions written by out(dst, i, v, e).
+template <class LAY, class OUT>
 __device__ __forceinline__ void prolong_axis(const long long* v, const short* ve, int t, int lines, int p0, int ext,
-                                             int N, int stride, const BASE& base, const OUT& out) {
-  const int pairs = ((p0 + ext - 1) >> 1) + 1;
-  for (int q = t; q < lines * pairs; q += 128) {
-    const int c = q / lines, l = q - c * lines, b = base(l), i = 2 * c - p0;
+                                             int N, int stride, const LAY& lay, const OUT& out) {
+  const int items = lines * (((p0 + ext - 1) >> 1) + 1);
+  const SmallDiv by_lines(lines);
+  for (int q = t; q < items; q += 128) {
+    const int c = by_lines(q), l = q - c * lines, i = 2 * c - p0;
+    int dst;
+    const int b = lay(l, &dst);
     long long lo, hi;
     int elo, ehi;
     prolong_pair(v + b, ve + b, c - p0, N, stride, &lo, &hi, &elo, &ehi);
-    if (i >= 0) out(l, i, lo, elo);
-    if (i + 1 < ext) out(l, i + 1, hi, ehi);
+    if (i >= 0) out(dst, i, lo, elo);
+    if (i + 1 < ext) out(dst, i + 1, hi, ehi);
   }
 }
 
@@ -174,10 +184,11 @@ __device__ __forceinline__ void amr_prolong_tiles_body(const double* __restrict_
     const int v = active ? combo / F : 0, f = active ? combo % F : 0;
     const double* base = (v == 0 ? yn : v == 1 ? k1 : v == 2 ? k2 : v == 3 ? k3 : k4) + (long)f * pfs + T.pbase;
     int bad = 0;
+    const SmallDiv by_x(Nx), by_y(Ny), by_e(ex);
     if (active)
       for (int q = t; q < Nx * Ny * Nz; q += 128) {
-        const int x = q % Nx, r = q / Nx;
-        const double d = __ldg(base + (long)(r / Ny) * psz + (long)(r % Ny) * psy + x);  // [z][y][x]
+        const int r = by_x(q), x = q - r * Nx, z = by_y(r);
+        const double d = __ldg(base + (long)z * psz + (long)(r - z * Ny) * psy + x);  // [z][y][x]
         const int h = __double2hiint(d), e = (h >> 20) & 0x7ff;
         const long long s = h >> 31;
         const long long bits = __double_as_longlong(d), m = (bits & 0xfffffffffffffll) | 0x10000000000000ll;
@@ -188,24 +199,36 @@ __device__ __forceinline__ void amr_prolong_tiles_body(const double* __restrict_
       }
     if (!__syncthreads_or(bad)) {
       if (active)
-        prolong_axis(iR, eR, t, Ny * Nz, px, ex, Nx, 1, [&](int l) { return l * Nx; },
-                     [&](int l, int i, long long x, int e) {
-                       iX[l * ex + i] = x;  // [z][y][i]
-                       eX[l * ex + i] = (short)e;
+        prolong_axis(iR, eR, t, Ny * Nz, px, ex, Nx, 1,
+                     [&](int l, int* dst) {
+                       *dst = l * ex;  // [z][y][i]
+                       return l * Nx;
+                     },
+                     [&](int dst, int i, long long x, int e) {
+                       iX[dst + i] = x;
+                       eX[dst + i] = (short)e;
                      });
       __syncthreads();
       if (active)
-        prolong_axis(iX, eX, t, ex * Nz, py, ey, Ny, ex, [&](int l) { return (l / ex) * Ny * ex + l % ex; },
-                     [&](int l, int j, long long x, int e) {
-                       const int o = ((l / ex) * ey + j) * ex + l % ex;  // [z][j][i]
-                       iY[o] = x;
-                       eY[o] = (short)e;
+        prolong_axis(iX, eX, t, ex * Nz, py, ey, Ny, ex,
+                     [&](int l, int* dst) {
+                       const int z = by_e(l), i = l - z * ex;
+                       *dst = z * ey * ex + i;  // [z][j][i]
+                       return z * Ny * ex + i;
+                     },
+                     [&](int dst, int j, long long x, int e) {
+                       iY[dst + j * ex] = x;
+                       eY[dst + j * ex] = (short)e;
                      });
       __syncthreads();
       if (active)
-        prolong_axis(iY, eY, t, ex * ey, pz, ez, Nz, ex * ey, [&](int l) { return l; },
-                     [&](int l, int k, long long x, int e) {
-                       const int slot = slots[T.slot_base + k * ex * ey + l];
+        prolong_axis(iY, eY, t, ex * ey, pz, ez, Nz, ex * ey,
+                     [&](int l, int* dst) {
+                       *dst = l;
+                       return l;
+                     },
+                     [&](int dst, int k, long long x, int e) {
+                       const int slot = slots[T.slot_base + k * ex * ey + dst];
                        if (slot >= 0) store[((long)v * F + f) * ncells + slot] = fx_back<6, 0>(x, e << 20);
                      });
       __syncthreads();
