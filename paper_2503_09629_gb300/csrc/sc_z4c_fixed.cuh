@@ -318,7 +318,6 @@ struct FxScales {
   FxC kP3, kM3;      // a third of those
   FxC twothird;      // exponent -59
   int poff;          // in place
-  double ko;         // sigma / (64 h) of the dissipation sum
 };
 inline FxScales fx_scales(const DerivScales& ds) {
   FxScales c{};
