@@ -12,10 +12,68 @@
 
 namespace sc {
 
+// Prolongation sums.  Values are v * 2^e with |v| < 2^60.2 (59 bits at a node,
+// grown by less than 1.3 per axis: the weights' magnitudes sum to 10568 / 8192).
+// A position's six nodes are aligned to their largest exponent and the weights are
+// integers over 2^13, so a sum is exact to the last place of that alignment and
+// depends on the six values alone.  Nodes that hold an infinity, a NaN or a value
+// near the ends of the exponent range carry kNodeFp64, which spreads to every
+// sum they enter; such a position is computed in FP64.
+constexpr int kNodeFp64 = 0x7fff;
+__device__ __forceinline__ void prolong_node(double d, long long* v, int* e) {
+  const long long bits = __double_as_longlong(d), s = bits >> 63;
+  const int t = (int)(bits >> 52) & 0x7ff;
+  const long long m = (bits & 0xfffffffffffffll) | 0x10000000000000ll;
+  const bool zero = (bits << 1) == 0;
+  *v = zero ? 0 : ((m << 6) ^ s) - s;
+  *e = zero || (unsigned)(t - 120) <= 1880u ? t : kNodeFp64;
+}
+__device__ __forceinline__ long long prolong_align(long long v, int n) {
+  long long r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+}
+// weight * 2^13 of node m for parity 0 (-1/4 from cell c, nodes c-3..c+2); parity 1 mirrored
+__device__ __forceinline__ constexpr int prolong_weight(int m) {
+  constexpr int w[6] = {63, -495, 2310, 6930, -693, 77};
+  return w[m];
+}
+__device__ __forceinline__ void prolong_one(const long long* v, const int* e, int parity, long long* r, int* E) {
+  int em = 0;
+#pragma unroll
+  for (int m = 0; m < 6; ++m) em = max(em, e[m]);
+  FxWide a;
+#pragma unroll
+  for (int m = 0; m < 6; ++m)
+    a.add(parity ? prolong_weight(5 - m) : prolong_weight(m), prolong_align(v[m], em - e[m]));
+  *r = a.get<13>();
+  *E = em;
+}
+// One value in FP64 chains: x sums over six nodes from zero, then y sums of those, then z sums.
+static __device__ __noinline__ double prolong_fp64(const double* p, long psy, long psz, const double* wx, const double* wy,
+                                            const double* wz) {
+  double sz = 0.0;
+#pragma unroll 1
+  for (int kz = 0; kz < kPN; ++kz) {
+    double sy = 0.0;
+#pragma unroll 1
+    for (int ky = 0; ky < kPN; ++ky) {
+      const double* row = p + (long)kz * psz + (long)ky * psy;
+      double sx = 0.0;
+#pragma unroll
+      for (int kx = 0; kx < kPN; ++kx) sx = fma(wx[kx], row[kx], sx);
+      sy = fma(wy[ky], sx, sy);
+    }
+    sz = fma(wz[kz], sy, sz);
+  }
+  return sz;
+}
+
 // Sec. II step 2, per-cell form: tensor-product quintic Lagrange prolongation
 // of y_n and the stage vectors the dense output reads (the first nvec of yn,
 // k1..k4) from 6x6x6 parent cells to refinement-boundary ghost cells
-// [first, ncells); results go to store[(v * F + f) * ncells + cell].
+// [first, ncells); results go to store[(v * F + f) * ncells + cell].  The sums of
+// the tile form below, so both give identical results.
 __device__ __forceinline__ void amr_prolong_cells_body(const double* __restrict__ yn, const double* __restrict__ k1,
                                                        const double* __restrict__ k2, const double* __restrict__ k3,
                                                        const double* __restrict__ k4, long pfs, int psy, int psz,
@@ -28,28 +86,27 @@ __device__ __forceinline__ void amr_prolong_cells_body(const double* __restrict_
     const int a = first + (int)(idx % nc);
     const int f = (int)(idx / nc);
     const AmrCell c = cells[a];
-    const double* wx = w.prolong[c.parity & 1];
-    const double* wy = w.prolong[(c.parity >> 1) & 1];
-    const double* wz = w.prolong[(c.parity >> 2) & 1];
+    const int px = c.parity & 1, py = (c.parity >> 1) & 1, pz = (c.parity >> 2) & 1;
     const double* src[5] = {yn, k1, k2, k3, k4};
 #pragma unroll 1
     for (int v = 0; v < nvec; ++v) {
       const double* p = src[v] + (long)f * pfs + c.pbase;
-      double sz = 0.0;
+      long long z[kPN], y[kPN], x[kPN], r;
+      int ez[kPN], ey[kPN], ex[kPN], e;
 #pragma unroll
       for (int kz = 0; kz < kPN; ++kz) {
-        double sy = 0.0;
 #pragma unroll
         for (int ky = 0; ky < kPN; ++ky) {
           const double* row = p + (long)kz * psz + (long)ky * psy;
-          double sx = 0.0;
 #pragma unroll
-          for (int kx = 0; kx < kPN; ++kx) sx = fma(wx[kx], __ldg(row + kx), sx);
-          sy = fma(wy[ky], sx, sy);
+          for (int kx = 0; kx < kPN; ++kx) prolong_node(__ldg(row + kx), &x[kx], &ex[kx]);
+          prolong_one(x, ex, px, &y[ky], &ey[ky]);
         }
-        sz = fma(wz[kz], sy, sz);
+        prolong_one(y, ey, py, &z[kz], &ez[kz]);
       }
-      store[((long)v * F + f) * ncells + a] = sz;
+      prolong_one(z, ez, pz, &r, &e);
+      store[((long)v * F + f) * ncells + a] =
+          e == kNodeFp64 ? prolong_fp64(p, psy, psz, w.prolong[px], w.prolong[py], w.prolong[pz]) : fx_back<6, 0>(r, e << 20);
     }
   }
 }
@@ -71,18 +128,10 @@ constexpr int kProlongSmemPerGroup = kTileValues + kTileValues / 4;
 // The two fine positions of parent cell c of a line (parities 0 and 1, at -1/4
 // and +1/4) from the seven nodes their stencils cover: nodes n0..n0 + 6 of the
 // line's N (those outside it belong to a position that the tile does not have).
-// Values are v * 2^e with |v| < 2^60.2 (59 bits, grown by less than 1.3 per axis:
-// the weights' magnitudes sum to 10568 / 8192).  Each position's six nodes are
-// aligned to their own largest exponent, so that its value does not depend on
-// the tile it is in, and the weights are integers over 2^13: a sum is exact to
-// the last place of that alignment.
+// Each position has its own alignment (prolong_one), so that its value does not
+// depend on the tile it is in.
 __device__ __forceinline__ void prolong_pair(const long long* __restrict__ v, const short* __restrict__ ve, int n0,
                                              int N, int stride, long long* lo, long long* hi, int* elo, int* ehi) {
-  auto align = [](long long x, int n) {
-    long long r;
-    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
-    return r;
-  };
   long long x[7];
   int e[7], mid = 0;
 #pragma unroll
@@ -94,22 +143,21 @@ __device__ __forceinline__ void prolong_pair(const long long* __restrict__ v, co
     if (m > 0 && m < 6) mid = max(mid, e[m]);
   }
   const int E0 = max(e[0], mid), E1 = max(mid, e[6]);
-  constexpr int w[6] = {63, -495, 2310, 6930, -693, 77};  // parity 0: -1/4 from cell c, nodes c-3..c+2; parity 1 mirrored
   FxWide a, b;
-  a.add(w[0], align(x[0], E0 - e[0]));
-  b.add(w[0], align(x[6], E1 - e[6]));
+  a.add(prolong_weight(0), prolong_align(x[0], E0 - e[0]));
+  b.add(prolong_weight(0), prolong_align(x[6], E1 - e[6]));
   long long y[5];
 #pragma unroll
   for (int m = 1; m < 6; ++m) {
-    y[m - 1] = align(x[m], E0 - e[m]);
-    a.add(w[m], y[m - 1]);
+    y[m - 1] = prolong_align(x[m], E0 - e[m]);
+    a.add(prolong_weight(m), y[m - 1]);
   }
   if (E0 != E1) {
 #pragma unroll
-    for (int m = 1; m < 6; ++m) y[m - 1] = align(x[m], E1 - e[m]);
+    for (int m = 1; m < 6; ++m) y[m - 1] = prolong_align(x[m], E1 - e[m]);
   }
 #pragma unroll
-  for (int m = 1; m < 6; ++m) b.add(w[6 - m], y[m - 1]);
+  for (int m = 1; m < 6; ++m) b.add(prolong_weight(6 - m), y[m - 1]);
   *lo = a.get<13>();
   *hi = b.get<13>();
   *elo = E0;
@@ -146,9 +194,10 @@ __device__ __forceinline__ void prolong_axis(const long long* v, const short* ve
 // then z.  Along the thin axis of a slab tile (the ghost width) the sums shrink
 // 7-8 nodes to 3-4 values, so a ghost value costs 20-40 multiplications instead
 // of the 216 + 42 of the per-cell form.  The sums are integers (prolong_pair), two
-// fine positions of a parent cell at a time: in FP64 chains (which stay for
-// tiles that hold an infinity, a NaN or a value near the ends of the exponent
-// range) the kernel was bound by that pipe, 82% of its rate.
+// fine positions of a parent cell at a time: in FP64 chains the kernel was bound
+// by that pipe, 82% of its rate.  Now integer issue: 684,504 ghost cells of two
+// fields and five vectors, 0.443 ms in FP64, 0.343 with run-time divisions for the
+// work items' places, 0.281 so; 46,872 ghost cells 0.054, 0.039, 0.033.
 // ngrp groups of 128 threads (threads beyond them idle); sm: ngrp *
 // kProlongSmemPerGroup doubles.  Every thread of the block must call this
 // function (it synchronises the block).
@@ -160,13 +209,10 @@ __device__ __forceinline__ void amr_prolong_tiles_body(const double* __restrict_
                                                        double* __restrict__ store, int F, const Weights& w, int nvec,
                                                        int bid, int nb, double* sm, int ngrp) {
   const int grp = threadIdx.x >> 7, t = threadIdx.x & 127;
-  double* sR = sm + grp * kProlongSmemPerGroup;
-  double* sX = sR + kTileRegion;
-  double* sY = sX + kTileXSums;
-  long long* iR = reinterpret_cast<long long*>(sR);  // the same places for the integer form
+  long long* iR = reinterpret_cast<long long*>(sm + grp * kProlongSmemPerGroup);
   long long* iX = iR + kTileRegion;
   long long* iY = iX + kTileXSums;
-  short* eR = reinterpret_cast<short*>(sR + kTileValues);
+  short* eR = reinterpret_cast<short*>(iR + kTileValues);
   short* eX = eR + kTileRegion;
   short* eY = eX + kTileXSums;
   const int combos = nvec * F;
@@ -183,99 +229,59 @@ __device__ __forceinline__ void amr_prolong_tiles_body(const double* __restrict_
     const int Nz = tile_node_offset(pz, ez - 1) + kPN;
     const int v = active ? combo / F : 0, f = active ? combo % F : 0;
     const double* base = (v == 0 ? yn : v == 1 ? k1 : v == 2 ? k2 : v == 3 ? k3 : k4) + (long)f * pfs + T.pbase;
-    int bad = 0;
     const SmallDiv by_x(Nx), by_y(Ny), by_e(ex);
     if (active)
       for (int q = t; q < Nx * Ny * Nz; q += 128) {
         const int r = by_x(q), x = q - r * Nx, z = by_y(r);
-        const double d = __ldg(base + (long)z * psz + (long)(r - z * Ny) * psy + x);  // [z][y][x]
-        const int h = __double2hiint(d), e = (h >> 20) & 0x7ff;
-        const long long s = h >> 31;
-        const long long bits = __double_as_longlong(d), m = (bits & 0xfffffffffffffll) | 0x10000000000000ll;
-        const bool zero = (bits << 1) == 0;
-        iR[q] = zero ? 0 : ((m << 6) ^ s) - s;
+        int e;
+        prolong_node(__ldg(base + (long)z * psz + (long)(r - z * Ny) * psy + x), iR + q, &e);  // [z][y][x]
         eR[q] = (short)e;
-        bad |= (unsigned)(e - 120) > 1880u && !zero;
       }
-    if (!__syncthreads_or(bad)) {
-      if (active)
-        prolong_axis(iR, eR, t, Ny * Nz, px, ex, Nx, 1,
-                     [&](int l, int* dst) {
-                       *dst = l * ex;  // [z][y][i]
-                       return l * Nx;
-                     },
-                     [&](int dst, int i, long long x, int e) {
-                       iX[dst + i] = x;
-                       eX[dst + i] = (short)e;
-                     });
-      __syncthreads();
-      if (active)
-        prolong_axis(iX, eX, t, ex * Nz, py, ey, Ny, ex,
-                     [&](int l, int* dst) {
-                       const int z = by_e(l), i = l - z * ex;
-                       *dst = z * ey * ex + i;  // [z][j][i]
-                       return z * Ny * ex + i;
-                     },
-                     [&](int dst, int j, long long x, int e) {
-                       iY[dst + j * ex] = x;
-                       eY[dst + j * ex] = (short)e;
-                     });
-      __syncthreads();
-      if (active)
-        prolong_axis(iY, eY, t, ex * ey, pz, ez, Nz, ex * ey,
-                     [&](int l, int* dst) {
-                       *dst = l;
-                       return l;
-                     },
-                     [&](int dst, int k, long long x, int e) {
-                       const int slot = slots[T.slot_base + k * ex * ey + dst];
-                       if (slot >= 0) store[((long)v * F + f) * ncells + slot] = fx_back<6, 0>(x, e << 20);
-                     });
-      __syncthreads();
-      continue;
-    }
+    __syncthreads();
     if (active)
-      for (int q = t; q < Nx * Ny * Nz; q += 128) {
-        const int x = q % Nx, r = q / Nx;
-        sR[q] = __ldg(base + (long)(r / Ny) * psz + (long)(r % Ny) * psy + x);
-      }
+      prolong_axis(iR, eR, t, Ny * Nz, px, ex, Nx, 1,
+                   [&](int l, int* dst) {
+                     *dst = l * ex;  // [z][y][i]
+                     return l * Nx;
+                   },
+                   [&](int dst, int i, long long x, int e) {
+                     iX[dst + i] = x;
+                     eX[dst + i] = (short)e;
+                   });
     __syncthreads();
-    if (active) {  // x: each (y, z) row of nodes to the tile's ex fine positions
-      for (int q = t; q < ex * Ny * Nz; q += 128) {
-        const int i = q % ex, r = q / ex;
-        const int p = (px + i) & 1;
-        const double* row = sR + r * Nx + tile_node_offset(px, i);
-        double s = 0.0;
-#pragma unroll
-        for (int m = 0; m < kPN; ++m) s = fma(w.prolong[p][m], row[m], s);
-        sX[q] = s;  // [z][y][i]
-      }
-    }
+    if (active)
+      prolong_axis(iX, eX, t, ex * Nz, py, ey, Ny, ex,
+                   [&](int l, int* dst) {
+                     const int z = by_e(l), i = l - z * ex;
+                     *dst = z * ey * ex + i;  // [z][j][i]
+                     return z * Ny * ex + i;
+                   },
+                   [&](int dst, int j, long long x, int e) {
+                     iY[dst + j * ex] = x;
+                     eY[dst + j * ex] = (short)e;
+                   });
     __syncthreads();
-    if (active) {  // y
-      for (int q = t; q < ex * ey * Nz; q += 128) {
-        const int i = q % ex, j = (q / ex) % ey, z = q / (ex * ey);
-        const int p = (py + j) & 1;
-        const double* col = sX + (z * Ny + tile_node_offset(py, j)) * ex + i;
-        double s = 0.0;
-#pragma unroll
-        for (int m = 0; m < kPN; ++m) s = fma(w.prolong[p][m], col[m * ex], s);
-        sY[q] = s;  // [z][j][i]
-      }
-    }
-    __syncthreads();
-    if (active) {  // z, then store the claimed positions
-      for (int q = t; q < ex * ey * ez; q += 128) {
-        const int ij = q % (ex * ey), k = q / (ex * ey);
-        const int p = (pz + k) & 1;
-        const double* col = sY + tile_node_offset(pz, k) * ex * ey + ij;
-        double s = 0.0;
-#pragma unroll
-        for (int m = 0; m < kPN; ++m) s = fma(w.prolong[p][m], col[m * ex * ey], s);
-        const int slot = slots[T.slot_base + q];
-        if (slot >= 0) store[((long)v * F + f) * ncells + slot] = s;
-      }
-    }
+    if (active)
+      prolong_axis(iY, eY, t, ex * ey, pz, ez, Nz, ex * ey,
+                   [&](int l, int* dst) {
+                     *dst = l;
+                     return l;
+                   },
+                   [&](int dst, int k, long long x, int e) {
+                     const int slot = slots[T.slot_base + k * ex * ey + dst];
+                     if (slot < 0) return;
+                     double d;
+                     if (e == kNodeFp64) {
+                       const int j = by_e(dst), i = dst - j * ex;
+                       d = prolong_fp64(base + (long)tile_node_offset(pz, k) * psz +
+                                            (long)tile_node_offset(py, j) * psy + tile_node_offset(px, i),
+                                        psy, psz, w.prolong[(px + i) & 1], w.prolong[(py + j) & 1],
+                                        w.prolong[(pz + k) & 1]);
+                     } else {
+                       d = fx_back<6, 0>(x, e << 20);
+                     }
+                     store[((long)v * F + f) * ncells + slot] = d;
+                   });
     __syncthreads();
   }
 }

@@ -110,10 +110,10 @@ __device__ void run_phase(const POp& op, const Weights& w, double* sm, int bid, 
   }
 }
 
-// Three blocks per SM (at most 80 registers): more warps to hide the
-// latency of the memory-bound phases than the two an unconstrained build
-// allows.
-__global__ void __launch_bounds__(kPThreads, 3) persistent_step_kernel(PBatch B) {
+// Two blocks per SM (at most 128 registers): with three, the integer sums spill
+// (2-level 32^3 / 3-level 64^3 / 128^3 step: 0.159 / 0.583 / 2.298 ms, against
+// 0.135 / 0.537 / 1.934 with two).
+__global__ void __launch_bounds__(kPThreads, 2) persistent_step_kernel(PBatch B) {
   extern __shared__ double sm[];
   // the phase record, staged in shared memory: one coalesced read per block
   // instead of one dependent global load per field
