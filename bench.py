@@ -63,19 +63,12 @@ HBM_GBS = _measured_hbm_gbs()
 # multiplies and fused multiply-adds (2 flops) of the formulation as first
 # written, counted by ncu (z4c_derivs = row-segment D_x/D_y pass 133 +
 # per-cell pass 1047).  Later rewrites evaluate the same right-hand side with
-# fewer FP64 instructions (FP64_INSTR_PER_CELL); the flop counts stay fixed so
-# that achieved rates measure the method's work, and the issue fractions
-# measure the current instruction stream.
+# fewer FP64 instructions (FP64_INSTR_PER_CELL) and then in integers; the flop
+# counts stay fixed so that achieved rates measure the method's work.
 FLOPS_PER_CELL = {"z4c_derivs": 1180.0, "z4c_stage": 1971.0}
-# DRAM bytes (read + write) per interior cell of each kernel from a
-# cold-cache ncu capture of a 262,144-cell launch (ncu flushes the caches
-# before the launch; profiles/z4c_kernels_bl3level64_ncu.md), scaled to a
-# launch by its cell count; None once the kernel has changed since the
-# counters were taken.
-DRAM_BYTES_PER_CELL = {"z4c_derivs": (32.003584e6 + 5.960192e6 + 150.886144e6 + 247.183104e6) / 262144,
-                       "z4c_stage": (525.380608e6 + 289.159168e6) / 262144}
 # FP64 instructions (DFMA + DMUL + DADD, thread-level / cell) per interior
-# cell of each pass, counted by ncu on the 3-level 64^3 case
+# cell of each pass in its FP64 form, which the production kernels keep for the
+# cells that their integer forms do not take, counted by ncu on the 3-level 64^3 case
 # (profiles/z4c_kernels_bl3level64_ncu.md, profiles/z4c_fp64_op_classes_bl3level64_ncu.md).
 FP64_INSTR_PER_CELL = {4: {"z4c_derivs": 72.1875 + 693.0, "z4c_stage": 1072.0},
                        8: {"z4c_derivs": 209.0 + 1210.0, "z4c_stage": 1072.0}}
@@ -509,7 +502,8 @@ def run_gpu(args, rank: int, world: int):
     launches = ctx.sc_launches_per_step() * args.steps
     state_finite = ctx.sc_check_finite()
 
-    # Roofline of the dominant kernels: FP64-ALU bound.  Per-launch durations
+    # Roofline of the dominant kernels against the FP64 peak: the method's flops,
+    # which the kernels compute in integers (a fraction may exceed 1).  Per-launch durations
     # from CUDA events on the library's stream, on the finest level; peaks
     # read from this device (nominal from its SM count and clock, and the
     # measured DFMA and DADD issue rates).
@@ -523,23 +517,18 @@ def run_gpu(args, rank: int, world: int):
     for name, t in (("z4c_derivs", t_der), ("z4c_stage", t_stage)):
         fpc = FLOPS_PER_CELL[name] if (h.fd_order == 4 or name == "z4c_stage") else None
         ipc = FP64_INSTR_PER_CELL[h.fd_order][name]
-        issue = cells * ipc / (t * 1e-3) / 1e9
         gen, slow = FP64_OP_CLASSES[h.fd_order][name]
-        # shortest time of this instruction mix at the measured issue rates
+        # shortest time of the FP64 form's instruction mix at the measured issue rates: the production
+        # kernels sum in integers and are not bound by it
         t_mix = cells * (gen / pk["dfma_g_per_s"] + slow / pk["dadd_g_per_s"]) / 1e9 * 1e3
         r = {"ms_per_launch": t, "cells_per_launch": cells, "flops_per_cell": fpc,
-             "fp64_issue": {"achieved_g_instr_per_s": issue, "instr_per_cell": ipc,
-                            "general_fma_per_cell": gen, "dadd_rate_ops_per_cell": slow,
-                            "frac_of_nominal_dfma_issue": issue / (nominal_tflops * 1e3 / 2),
-                            "frac_of_measured_dfma_issue": issue / pk["dfma_g_per_s"],
-                            "frac_of_measured_dadd_issue": issue / pk["dadd_g_per_s"],
-                            "mix_ceiling_ms": t_mix, "frac_of_mix_ceiling": t_mix / t}}
+             "fp64_form": {"instr_per_cell": ipc, "general_fma_per_cell": gen, "dadd_rate_ops_per_cell": slow,
+                           "mix_ceiling_ms": t_mix, "speedup_over_mix_ceiling": t_mix / t}}
         if fpc is not None:
             ach = cells * fpc / (t * 1e-3) / 1e12
-            tb = DRAM_BYTES_PER_CELL.get(name) if h.fd_order == 4 else None
             r.update({"bound": "alu", "achieved": ach, "peak": nominal_tflops, "unit": "TFLOP/s",
                       "frac": ach / nominal_tflops, "frac_of_measured_dfma": ach / dfma_tflops,
-                      "traffic": (tb * cells if tb else None)})
+                      "traffic": None})
         roof[name] = r
     # Refinement-boundary ghost fill on the finest level: the tile-separable
     # prolongation (FP64: the FMAs its tiles execute, counted by the library)
