@@ -1693,8 +1693,8 @@ sc_status apply_tuning(sc_ctx* c, const int* shape, int deriv_form, int bps) {
 
 }  // namespace
 
-// Autotuner (the search space: tile shape x derivative-pass split x stage
-// kernel blocks per SM).  On the context's largest level it times every tile
+// Autotuner (the search space: derivative-pass split x stage kernel blocks per
+// SM; the wave stage and the two-kernel derivative pass have tiles of their own).  On the context's largest level it times every tile
 // shape of the stencil kernel (the wave's fused stage, or the Z4c derivative
 // pass in its two-kernel form), the one-kernel Z4c derivative pass (4th
 // order, default tiles), and the Z4c stage kernel built for 2 and for 3 blocks

@@ -168,7 +168,7 @@ struct StageArgs {
 // multiply-adds with constants the compiler cannot see (+1, -1, -0 arrive as
 // kernel arguments): fma(a, 1, b) = a + b, fma(b, -1, a) = a - b and
 // fma(x, y, -0) = x * y exactly, so the results are bitwise those of the
-// plain operations.  Measured on this GPU: the Z4c derivative and stage
+// plain operations.  Measured on this GPU: the FP64 forms of the Z4c derivative and stage
 // kernels run about 5% faster this way than in their op-class build below,
 // the same arithmetic with DADD/DSUB/DMUL (ncu on a 262,144-cell level:
 // 339 against 358 us and 538 against 564 us), although an isolated chain of
