@@ -38,7 +38,7 @@ def _stale(target: str, deps) -> bool:
 
 def build(verbose: bool = False) -> str:
     os.makedirs(OUT_DIR, exist_ok=True)
-    headers = [os.path.join(SRC, h) for h in ("sc_internal.h", "sc_device.cuh", "sc_fixed.cuh", "sc_z4c_fixed.cuh", "sc_persist.h")] + [os.path.join(ROOT, "include", "subcyc.h")]
+    headers = [os.path.join(SRC, h) for h in ("sc_internal.h", "sc_device.cuh", "sc_fixed.cuh", "sc_z4c_point.cuh", "sc_persist.h")] + [os.path.join(ROOT, "include", "subcyc.h")]
     srcs = [s for s in SOURCES if os.path.exists(os.path.join(SRC, s))]
     objs = []
     jobs = []

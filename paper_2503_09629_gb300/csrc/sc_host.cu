@@ -340,9 +340,9 @@ struct sc_ctx {
   // pass that differentiates them for the mixed derivatives), 1 = one kernel
   // per (cell, field) with direct 16-point mixed stencils (4th order only);
   // stage kernel build: registers for 2 or 3 blocks of 128 threads per SM
-  // (autotuned; 2 measured faster from 8,000 to 262,144 cells)
+  // (autotuned; 262,144 cells: 0.329 ms with 3, 0.361 with 2; 8,000 cells: 0.035 with both)
   int deriv_form = 0;
-  int stage_bps = 2;
+  int stage_bps = 3;
   int eta_profile = 0;
   double eta_c = 0, eta_s = 0, eta_o = 0;
   std::vector<Op> plain_ops[2];  // per-box form: the schedule, run directly
@@ -2392,8 +2392,7 @@ sc_status sc_get_constraints(sc_ctx* c, int level, int box, double* dst) {
     CU(launch_z4c_derivs_split(Y, c->scratch, L.g.fs, sy, sz, L.dtiles + L.box_dtile_begin[box],
                                L.box_dtile_begin[box + 1] - L.box_dtile_begin[box], c->stream, c->order));
   }
-  CU(launch_z4c_constraints(Y, c->scratch, c->staging, L.g.fs, sy, sz, c->zp, deriv_scales(c->order, L.g.h), ncell, blo, n,
-                            c->stream));
+  CU(launch_z4c_constraints(Y, c->scratch, c->staging, L.g.fs, sy, sz, deriv_scales(c->order, L.g.h), L.g.h, ncell, blo, n, c->stream));
   CU(cudaMemcpyAsync(dst, c->staging, bytes, cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));
   c->dfree(dt);  // the per-call tile list (the stream is idle)

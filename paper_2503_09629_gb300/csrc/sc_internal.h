@@ -251,9 +251,9 @@ cudaError_t launch_z4c_stage(const StageArgs& a, const double* scratch, const Z4
                              int nruns, cudaStream_t s, int bps, bool op_class = false);
 cudaError_t launch_radiative_stage(const StageArgs& a, const int32_t* cells, int ncells, int F,
                                    const Geom& g, int system, cudaStream_t s);
-cudaError_t launch_z4c_constraints(const double* Y, const double* scratch, double* out, long fs, int sy,
-                                   int sz, const Z4cParams& p, const DerivScales& ds, long out_stride,
-                                   const int* box_lo, const int* box_n, cudaStream_t s);
+cudaError_t launch_z4c_constraints(const double* Y, const double* scratch, double* out, long fs, int sy, int sz,
+                                   const DerivScales& ds, double h, long out_stride, const int* box_lo,
+                                   const int* box_n, cudaStream_t s);
 
 cudaError_t launch_periodic_copy(double* vec, long fs, int F, const int2* pairs, int npairs, cudaStream_t s);
 // per-cell prolongation of AMR cells [first, ncells) of the list (store has ncells slots per vector-field);
