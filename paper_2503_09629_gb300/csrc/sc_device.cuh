@@ -459,7 +459,7 @@ template <int ORD>
 __device__ __forceinline__ void wave_stage_body(const StageArgs& a, const Tile* __restrict__ tiles, int ntiles,
                                                 const FmaK& K, int bid, int nb, long long* planes) {
   using F = FxSums<ORD>;
-  constexpr int R = ORD / 2, NW = 2 * R + 1, G = F::kGuard;
+  constexpr int R = ORD / 2, NW = 2 * R + 1;
   const long sy = a.sy, sz = a.sz;
   int buf = 0;
   for (int t = bid; t < ntiles; t += nb) {
@@ -520,7 +520,7 @@ __device__ __forceinline__ void wave_stage_body(const StageArgs& a, const Tile* 
       __syncthreads();
       if (!active) continue;
       long long v[R][6];
-      int E = fx_pexp(w[R]);
+      int Ei = fx_pexp(w[R]), E = 0;
 #pragma unroll
       for (int m = 0; m < R; ++m) {
         v[m][0] = pl[own - (m + 1)];
@@ -530,18 +530,15 @@ __device__ __forceinline__ void wave_stage_body(const StageArgs& a, const Tile* 
         v[m][4] = w[R - (m + 1)];
         v[m][5] = w[R + (m + 1)];
 #pragma unroll
-        for (int q = 0; q < 6; ++q) E = max(E, fx_pexp(v[m][q]));
-      }
-      double lap;
-      if (packed_ok(E)) {
-        typename F::Val s[R];
-#pragma unroll
-        for (int m = 0; m < R; ++m) {
-          s[m] = fx_palign<G>(v[m][0], E);
-#pragma unroll
-          for (int q = 1; q < 6; ++q) s[m] += fx_palign<G>(v[m][q], E);
+        for (int q = 0; q < 6; ++q) {
+          if (m == 0) Ei = max(Ei, fx_pexp(v[m][q]));
+          else E = max(E, fx_pexp(v[m][q]));
         }
-        lap = F::laplacian(s, fx_palign<G>(w[R], E), packed_field(E));
+      }
+      E = max(E, Ei);
+      double lap;
+      if (packed_ok(E) && E - Ei <= F::kLaplacianExcess) {
+        lap = F::laplacian(v, w[R], E);
       } else {
         const double* c = u + k * sz;
         double s[4];

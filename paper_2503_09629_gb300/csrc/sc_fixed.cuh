@@ -4,19 +4,27 @@
 // integer pipes about 110 (measured: 60.9 IADD3 and 61.0 IMAD per SM and
 // clock, on two pipes that run side by side, beside FP64 instructions too).  A
 // finite-difference stencil has small integer weights, so its sum needs no
-// floating point until the end: the stencil's values are aligned to the
-// exponent of the largest of them, as signed integers with 2 (4th order) or 6
-// (8th order) bits below that value's last place, summed exactly, and the sum
-// is rounded once on its way back to FP64.  The alignment drops what lies
-// below 2^-54 (2^-58) of the stencil's own largest value, always downwards, so
-// that its mean cancels in sums whose weights add up to zero; the halves of an
-// 8th-order sum are joined at 2^-47 of its largest term or less.  A chain of FP64
-// additions instead rounds every partial sum at 2^-53 of its size, which the
-// weights make several (8th order: thousands of) times the largest value.
+// floating point until the end: the values are aligned to the exponent of the largest
+// of them, as signed integers with some bits below that value's last place,
+// summed exactly, and the sum is rounded once on its way back to FP64.  The
+// alignment drops what lies below the last of these bits, always downwards, so
+// that its mean cancels in sums whose weights add up to zero.
+//
+// What is aligned together is what the sum weighs: the values along one axis for
+// its derivatives, all of the star for its Laplacian and the Kreiss-Oliger sum.  At
+// 4th order the weights multiply before the alignment cuts, or the weighted
+// values keep more bits, so that a sum's error is a few units of its smallest
+// weight: at most 2^-54 of its largest weighted term.  At 8th order the weights
+// are too far apart for that (1 to 8192), and sums whose lightly weighted outer
+// values are 2^3 to 2^5 times the inner ones are left to FP64, whose error
+// is relative to the weighted values (kFirstExcess and so on; inside these limits the
+// integer sums were the more accurate ones: on random values 1.4e-16 against
+// 2.3e-14 for a Laplacian of 4th order, 4.7e-17 against 2.8e-14 of 8th).
 // The result depends on the stencil's values alone, not on tiles or boxes.
 //
-// Stencils that hold an infinity or a NaN, or whose largest value lies near
-// either end of the exponent range, are left to the FP64 form (aligned_ok).
+// Stencils that hold an infinity or a NaN, that vanish, or whose largest value
+// lies near either end of the exponent range are left to the FP64 form too
+// (aligned_ok, packed_ok).
 #pragma once
 
 #include "sc_internal.h"
@@ -47,14 +55,18 @@ __device__ __forceinline__ Fx fx_unpack(double v) {
 // The exponent field of a value, in place.
 __device__ __forceinline__ int fx_exp(double v) { return __double2hiint(v) & 0x7ff00000; }
 
-// The value in units of 2^(exponent of E - 52 - GUARD), rounded down.  E is at
-// least the value's own t.  (PTX defines shr.s64 for every count: 64 and more
-// give the sign, which is how zeros and denormals, t = 0, become 0 or -1.)
-__device__ __forceinline__ long long fx_align(const Fx& f, int E) {
-  const long long x = ((long long)f.hi << 32) | f.lo;
+// (PTX defines shr.s64 for every count: 64 and more give the sign.)
+__device__ __forceinline__ long long fx_shift(long long x, int n) {
   long long r;
-  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"((E - f.t) >> 20));
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
   return r;
+}
+
+// The value in units of 2^(exponent of E - 52 - GUARD), rounded down.  E is at
+// least the value's own t.  (Shifts of 64 and more are how zeros and denormals,
+// t = 0, become 0 or -1.)
+__device__ __forceinline__ long long fx_align(const Fx& f, int E) {
+  return fx_shift(((long long)f.hi << 32) | f.lo, (E - f.t) >> 20);
 }
 
 // Whether stencils whose largest value has exponent field E may be summed in
@@ -74,12 +86,11 @@ __device__ __forceinline__ long long fx_pack(double v) {
   return ((x ^ s) - s) | t;
 }
 __device__ __forceinline__ int fx_pexp(long long p) { return (int)p & 1023; }
-// The same as fx_align(fx_unpack<GUARD>) of a packed value.
+// The same for a packed value (a negative one that loses no bits comes out as it is,
+// where fx_unpack's is one unit lower).
 template <int GUARD>
 __device__ __forceinline__ long long fx_palign(long long p, int E) {
-  long long r;
-  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(p & ~1023ll), "r"(E + (10 - GUARD) - fx_pexp(p)));
-  return r;
+  return fx_shift(p & ~1023ll, E + (10 - GUARD) - fx_pexp(p));
 }
 // As aligned_ok, for the largest packed exponent of a stencil.
 __device__ __forceinline__ bool packed_ok(int E) { return (unsigned)(E - 120) <= 902u; }
@@ -119,70 +130,139 @@ struct FxSums;
 
 template <>
 struct FxSums<4> {
-  static constexpr int kGuard = 2;  // 53 + 2 bits, weights of the Kreiss-Oliger sum 192 < 2^8
-  using Val = long long;
-  __device__ static __forceinline__ Val val(double v, int E) { return fx_align(fx_unpack<kGuard>(v), E); }
+  static constexpr int kInner = 2;         // first derivatives: every value counts as an inner one
+  static constexpr int kFirstExcess = 0;
+  // One axis of a star: u0 and the values at +-3 (Kreiss-Oliger) may be 2^2 times those of the
+  // first derivative; its error is then 2^-57 of their largest, FP64's 2^-55 of the latter's.
+  static constexpr int kAxisExcess = 2;
+  static constexpr int kLaplacianExcess = 1023;
   // 8 (v_1 - v_-1) - (v_2 - v_-2) = 12 h u'
-  __device__ static __forceinline__ double first(const Val* lo, const Val* hi, int E) {
-    return fx_back<kGuard, 0>(((hi[0] - lo[0]) << 3) + (lo[1] - hi[1]), E);
+  __device__ static __forceinline__ double first(const double* lo, const double* hi, int E) {
+    const long long l0 = fx_align(fx_unpack<7>(lo[0]), E), h0 = fx_align(fx_unpack<7>(hi[0]), E);
+    const long long l1 = fx_align(fx_unpack<4>(lo[1]), E), h1 = fx_align(fx_unpack<4>(hi[1]), E);
+    return fx_back<4, 0>((h0 - l0) + (l1 - h1), E);
   }
-  // 16 p1 - p2 - 30 u0 = 12 h^2 u'', pm = v_m + v_-m
-  __device__ static __forceinline__ double second(const Val* p, Val u0, int E) {
-    return fx_back<kGuard, 0>((p[0] << 4) - p[1] - ((u0 << 5) - (u0 << 1)), E);
-  }
-  // the three second derivatives' sum, Pm the sum over the six neighbours at distance m (weights: 192)
-  __device__ static __forceinline__ double laplacian(const Val* P, Val u0, int E) {
-    return fx_back<kGuard, 0>((P[0] << 4) - P[1] - 90 * u0, E);
-  }
-  // P3 - 6 P2 + 15 P1 - 60 u0, Pm the sum over the six neighbours at distance m
-  __device__ static __forceinline__ double ko(Val P1, Val P2, Val P3, Val u0, int E) {
-    const Val u60 = (u0 << 6) - (u0 << 2);
-    return fx_back<kGuard, 0>(((P1 << 4) - P1) - ((P2 << 2) + (P2 << 1)) + P3 - u60, E);
+  // Packed values of one axis, E their largest exponent (u0's among them), with 4 bits
+  // below the last place: 12 h u', 12 h^2 u'' = 16 p1 - p2 - 30 u0 (pm = v_m + v_-m) and the axis's share
+  // 15 p1 - 6 p2 + p3 - 20 u0 of the Kreiss-Oliger sum.  Weights up to 64, 63 bits.
+  struct Axis {
+    long long a, b, c, u10;
+    long long d;  // 8 (v_1 - v_-1) - (v_2 - v_-2)
+    __device__ __forceinline__ Axis(const long long* lo, const long long* hi, long long u0, int E) {
+      const long long l0 = fx_palign<7>(lo[0], E), h0 = fx_palign<7>(hi[0], E);
+      const long long l1 = fx_palign<4>(lo[1], E), h1 = fx_palign<4>(hi[1], E);
+      const long long x = u0 >> 10;  // 160 x: u0 times 10
+      a = l0 + h0;                   // 8 p1
+      b = l1 + h1;
+      c = fx_palign<4>(lo[2], E) + fx_palign<4>(hi[2], E);
+      d = (h0 - l0) + (l1 - h1);
+      u10 = fx_shift((x << 7) + (x << 5), E - fx_pexp(u0));
+    }
+    __device__ __forceinline__ double first(int Ef) const { return fx_back<4, 0>(d, Ef); }
+    __device__ __forceinline__ double second(int Ef) const { return fx_back<4, 0>((a << 1) - b - ((u10 << 1) + u10), Ef); }
+    __device__ __forceinline__ long long ko() const {
+      const long long p1 = a >> 3;
+      return ((p1 << 4) - p1) - ((b << 2) + (b << 1)) + c - (u10 << 1);
+    }
+  };
+  // The Kreiss-Oliger sum from the axes' shares; E: the star's largest exponent, Ed: the axis's.
+  struct Ko {
+    long long s = 0;
+    __device__ __forceinline__ void add(const Axis& A, int Ed, int E) { s += fx_shift(A.ko(), E - Ed + 2); }
+    __device__ __forceinline__ double get(long long, int E) const { return fx_back<4, 2>(s, packed_field(E)); }
+  };
+  // 12 h^2 times the Laplacian: 16 P1 - P2 - 90 u0, Pm the sum over the six neighbours at distance
+  // m, v[m - 1]: packed values, E their largest exponent (weights 192, 2 bits below the last place: 63 bits)
+  __device__ static __forceinline__ double laplacian(const long long (*v)[6], long long u0, int E) {
+    const long long x = u0 >> 10;  // 360 x: u0 times 90
+    long long s = -fx_shift((x << 8) + (x << 6) + (x << 5) + (x << 3), E - fx_pexp(u0));
+#pragma unroll
+    for (int q = 0; q < 6; ++q) s += fx_palign<6>(v[0][q], E) - fx_palign<2>(v[1][q], E);
+    return fx_back<2, 0>(s, packed_field(E));
   }
 };
 
 template <>
 struct FxSums<8> {
   static constexpr int kGuard = 6;  // 59 bits: sums of six values and their halves stay in range
-  using Val = long long;
-  __device__ static __forceinline__ Val val(double v, int E) { return fx_align(fx_unpack<kGuard>(v), E); }
+  // Outer values (+-3, +-4, weights 32 and 3) against those at +-1 and +-2 (672, 168): error of
+  // the integers 9 2^-53 of the largest value, of FP64 67 to 270 2^-53 of the inner ones.
+  static constexpr int kInner = 2, kFirstExcess = 3, kAxisExcess = 3;
+  // Values at +-2, +-3, +-4 (1008, 128, 9) against u0 and those at +-1 (43050, 8064):
+  // 430 2^-53 against 2e4 2^-53.
+  static constexpr int kLaplacianExcess = 5;
   // 672 d1 - 168 d2 + 32 d3 - 3 d4 = 840 h u', dm = v_m - v_-m (weights: 1750 < 2^11)
-  __device__ static __forceinline__ double first(const Val* lo, const Val* hi, int E) {
+  __device__ static __forceinline__ double first_of(const long long* l, const long long* h, int Ef) {
     FxWide s;
-    s.add(672, hi[0] - lo[0]);
-    s.add(-168, hi[1] - lo[1]);
-    s.add(32, hi[2] - lo[2]);
-    s.add(-3, hi[3] - lo[3]);
-    return fx_back<kGuard, 8>(s.get<8>(), E);
+    s.add(672, h[0] - l[0]);
+    s.add(-168, h[1] - l[1]);
+    s.add(32, h[2] - l[2]);
+    s.add(-3, h[3] - l[3]);
+    return fx_back<kGuard, 8>(s.get<8>(), Ef);
   }
-  // 8064 p1 - 1008 p2 + 128 p3 - 9 p4 - 14350 u0 = 5040 h^2 u'' (weights: 2^15)
-  __device__ static __forceinline__ double second(const Val* p, Val u0, int E) {
-    FxWide s;
-    s.add(8064, p[0]);
-    s.add(-1008, p[1]);
-    s.add(128, p[2]);
-    s.add(-9, p[3]);
-    s.add(-14350, u0);
-    return fx_back<kGuard, 12>(s.get<12>(), E);
+  __device__ static __forceinline__ double first(const double* lo, const double* hi, int E) {
+    long long l[4], h[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      l[m] = fx_align(fx_unpack<kGuard>(lo[m]), E);
+      h[m] = fx_align(fx_unpack<kGuard>(hi[m]), E);
+    }
+    return first_of(l, h, E);
   }
-  // the three second derivatives' sum, Pm the sum over the six neighbours at distance m (weights: 98304)
-  __device__ static __forceinline__ double laplacian(const Val* P, Val u0, int E) {
+  struct Axis {
+    long long l[4], h[4], u0;
+    __device__ __forceinline__ Axis(const long long* lo, const long long* hi, long long u, int E) {
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        l[m] = fx_palign<kGuard>(lo[m], E);
+        h[m] = fx_palign<kGuard>(hi[m], E);
+      }
+      u0 = fx_palign<kGuard>(u, E);
+    }
+    __device__ __forceinline__ double first(int Ef) const { return first_of(l, h, Ef); }
+    // 8064 p1 - 1008 p2 + 128 p3 - 9 p4 - 14350 u0 = 5040 h^2 u'' (weights: 2^15)
+    __device__ __forceinline__ double second(int Ef) const {
+      FxWide s;
+      s.add(8064, l[0] + h[0]);
+      s.add(-1008, l[1] + h[1]);
+      s.add(128, l[2] + h[2]);
+      s.add(-9, l[3] + h[3]);
+      s.add(-14350, u0);
+      return fx_back<kGuard, 12>(s.get<12>(), Ef);
+    }
+  };
+  // (weights: 192)
+  struct Ko {
+    long long P[3] = {0, 0, 0};
+    __device__ __forceinline__ void add(const Axis& A, int Ed, int E) {
+#pragma unroll
+      for (int m = 0; m < 3; ++m) P[m] += fx_shift(A.l[m] + A.h[m], E - Ed);
+    }
+    __device__ __forceinline__ double get(long long u0, int E) const {
+      FxWide s;
+      s.add(15, P[0]);
+      s.add(-6, P[1]);
+      s.add(1, P[2]);
+      s.add(-60, fx_palign<kGuard>(u0, E));
+      return fx_back<kGuard, 5>(s.get<5>(), packed_field(E));
+    }
+  };
+  // 5040 h^2 times the Laplacian (weights: 98304)
+  __device__ static __forceinline__ double laplacian(const long long (*v)[6], long long u0, int E) {
+    long long P[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      P[m] = fx_palign<kGuard>(v[m][0], E);
+#pragma unroll
+      for (int q = 1; q < 6; ++q) P[m] += fx_palign<kGuard>(v[m][q], E);
+    }
     FxWide s;
     s.add(8064, P[0]);
     s.add(-1008, P[1]);
     s.add(128, P[2]);
     s.add(-9, P[3]);
-    s.add(-43050, u0);
-    return fx_back<kGuard, 14>(s.get<14>(), E);
-  }
-  // (weights: 192)
-  __device__ static __forceinline__ double ko(Val P1, Val P2, Val P3, Val u0, int E) {
-    FxWide s;
-    s.add(15, P1);
-    s.add(-6, P2);
-    s.add(1, P3);
-    s.add(-60, u0);
-    return fx_back<kGuard, 5>(s.get<5>(), E);
+    s.add(-43050, fx_palign<kGuard>(u0, E));
+    return fx_back<kGuard, 14>(s.get<14>(), packed_field(E));
   }
 };
 

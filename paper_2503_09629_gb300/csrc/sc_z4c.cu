@@ -122,19 +122,15 @@ __device__ __forceinline__ double dfirst_fp64(const double* lo, const double* hi
 template <int ORD>
 __device__ __forceinline__ double dfirst(const double* lo, const double* hi) {
   using F = FxSums<ORD>;
-  constexpr int R = ORD / 2;
-  int E = 0;
+  int Ei = 0, E = 0;
 #pragma unroll
-  for (int m = 0; m < R; ++m) E = max(E, max(fx_exp(lo[m]), fx_exp(hi[m])));
-  if (aligned_ok(E)) {
-    typename F::Val l[R], h[R];
-#pragma unroll
-    for (int m = 0; m < R; ++m) {
-      l[m] = F::val(lo[m], E);
-      h[m] = F::val(hi[m], E);
-    }
-    return F::first(l, h, E);
+  for (int m = 0; m < ORD / 2; ++m) {
+    const int e = max(fx_exp(lo[m]), fx_exp(hi[m]));
+    if (m < F::kInner) Ei = max(Ei, e);
+    else E = max(E, e);
   }
+  E = max(E, Ei);
+  if (aligned_ok(E) && E - Ei <= F::kFirstExcess << 20) return F::first(lo, hi, E);
   return dfirst_fp64<ORD>(lo, hi);
 }
 
@@ -207,10 +203,12 @@ __device__ __forceinline__ void cell_sums_fp64(double u0, const double (*lo)[ORD
 // 32 high; a plane then holds at most 38 x 14 (40 x 16) values.  At 4th order D_x
 // and D_y along z are windows in registers too; at 8th order these would spill,
 // and are read again (L1).  Integer ALU 45%, latency of 16 warps: 262,144 cells with
-// the row pass before it, 0.251 ms with a thread per column and no sharing, 0.197
-// so; 110,592 cells 0.119 and 0.104; 8th order, 262,144 cells, 0.347 and 0.332.  With
-// the mixed derivatives in FP64 instead: 0.211 and 0.444; with three or four blocks
-// per SM and reads in place of the windows: 0.219 and 0.238.
+// the row pass before it, 0.251 ms with a thread per column and no sharing, 0.207
+// so (0.200 with one alignment for a cell's whole star, whose error in a derivative was
+// relative to the values along the other axes too); 110,592 cells 0.119 and 0.110; 8th order, 262,144
+// cells, 0.347 and 0.353 (0.329).  With the mixed derivatives in FP64 instead: 0.211 and
+// 0.444 (star alignment); with three or four blocks per SM and reads in place of the
+// windows: 0.219 and 0.238.
 template <int ORD>
 __global__ void __launch_bounds__(kDerivCols, 2)
     z4c_derivs_split_kernel(const double* __restrict__ Y, double* __restrict__ S, long fs, int sy_, int sz_,
@@ -220,7 +218,6 @@ __global__ void __launch_bounds__(kDerivCols, 2)
   constexpr int WR = R > 3 ? R : 3;
   constexpr int NW = 2 * WR + 1;
   constexpr int ND = 2 * R + 1;
-  constexpr int G = F::kGuard;
   constexpr bool kWindows = ORD == 4;
   __shared__ long long planes[2][plane_values(WR)];
   const long sy = sy_, sz = sz_;
@@ -288,35 +285,44 @@ __global__ void __launch_bounds__(kDerivCols, 2)
       auto at = [&](int dim, int m) {
         return dim == 0 ? pl[own + m] : dim == 1 ? pl[own + m * pitch] : w[WR + m];
       };
-      int E = fx_pexp(w[WR]);
+      // Each axis has an alignment of its own; one whose first derivative would lose by
+      // that (its values far below u0 or those at +-3), and one of zeros, sends the cell to FP64.
+      int Ed[3];
+      bool ok = true;
 #pragma unroll
-      for (int dim = 0; dim < 3; ++dim)
+      for (int dim = 0; dim < 3; ++dim) {
+        int Ei = 0, E = fx_pexp(w[WR]);
 #pragma unroll
-        for (int m = 1; m <= WR; ++m) E = max(E, max(fx_pexp(at(dim, -m)), fx_pexp(at(dim, m))));
+        for (int m = 1; m <= WR; ++m) {
+          const int e = max(fx_pexp(at(dim, -m)), fx_pexp(at(dim, m)));
+          if (m <= F::kInner) Ei = max(Ei, e);
+          else E = max(E, e);
+        }
+        Ed[dim] = max(E, Ei);
+        ok = ok && packed_ok(Ed[dim]) && Ed[dim] - Ei <= F::kAxisExcess;
+      }
       double* d1 = S + (long)(Q_D1 + 3 * f) * fs + o;
       double* d2 = S + (long)(Q_D2 + 6 * sl) * fs + o;
       double* ko = S + (long)(Q_KO + f) * fs + o;
-      if (packed_ok(E)) {
-        // One alignment for every sum of the cell.
-        const int Ef = packed_field(E);
-        typename F::Val P[3];
-        const typename F::Val x0 = fx_palign<G>(w[WR], E);
+      if (ok) {
+        const int E = max(max(Ed[0], Ed[1]), Ed[2]);
+        typename F::Ko sum;
 #pragma unroll
         for (int dim = 0; dim < 3; ++dim) {
-          typename F::Val l[WR], h[WR], p[WR];
+          long long l[WR], h[WR];
 #pragma unroll
           for (int m = 0; m < WR; ++m) {
-            l[m] = fx_palign<G>(at(dim, -m - 1), E);
-            h[m] = fx_palign<G>(at(dim, m + 1), E);
-            p[m] = l[m] + h[m];
+            l[m] = at(dim, -m - 1);
+            h[m] = at(dim, m + 1);
           }
+          const typename F::Axis A(l, h, w[WR], Ed[dim]);
+          const int Ef = packed_field(Ed[dim]);
           // D_x, D_y of the Hessian fields are there already (z4c_dxy_kernel)
-          if (sl < 0 || dim == 2) d1[dim * fs] = F::first(l, h, Ef);
-          if (sl >= 0) d2[(dim == 0 ? 0 : dim == 1 ? 3 : 5) * fs] = F::second(p, x0, Ef);
-#pragma unroll
-          for (int m = 0; m < 3; ++m) P[m] = dim == 0 ? p[m] : P[m] + p[m];
+          if (sl < 0 || dim == 2) d1[dim * fs] = A.first(Ef);
+          if (sl >= 0) d2[(dim == 0 ? 0 : dim == 1 ? 3 : 5) * fs] = A.second(Ef);
+          sum.add(A, Ed[dim], E);
         }
-        *ko = F::ko(P[0], P[1], P[2], x0, Ef);
+        *ko = sum.get(w[WR], E);
       } else {
         const double* v = u + k * sz;
         double fl[3][ORD == 4 ? 3 : 4], fh[3][ORD == 4 ? 3 : 4], e1[3], e2[3], eko;
