@@ -2474,8 +2474,8 @@ sc_status sc_run_op_class_pass(sc_ctx* c, int level) {
   Level& L = c->lev[level];
   const Geom& g = L.g;
   const StageArgs a = tuning_stage_args(L, c->order);
-  CU(launch_z4c_dxy(a.Y, c->scratch, g.fs, a.sy, L.dxy, L.ndxy, c->stream, c->order));
-  CU(launch_z4c_derivs_split(a.Y, c->scratch, g.fs, a.sy, a.sz, L.dtiles, L.ndtiles, c->stream, c->order));
+  CU(launch_z4c_dxy(a.Y, c->scratch, g.fs, a.sy, L.dxy, L.ndxy, c->stream, c->order, true));
+  CU(launch_z4c_derivs_split(a.Y, c->scratch, g.fs, a.sy, a.sz, L.dtiles, L.ndtiles, c->stream, c->order, true));
   CU(launch_z4c_stage(a, c->scratch, c->zp, L.runs, L.nruns, c->stream, c->stage_bps, true));
   CU(cudaStreamSynchronize(c->stream));
   return SC_OK;

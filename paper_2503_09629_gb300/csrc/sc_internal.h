@@ -239,11 +239,12 @@ cudaError_t launch_z4c_derivs(const double* Y, double* scratch, long fs, int sy,
 // before any graph capture).
 cudaError_t z4c_init_launch_config();
 // order: finite-difference order of the derivatives, 4 or 8 (Kreiss-Oliger stays r = 4).
+// op_class: the PlainK build of the kernel (same results; see PlainK).
 cudaError_t launch_z4c_dxy(const double* Y, double* scratch, long fs, int sy, const RowSeg* segs, int nsegs,
-                           cudaStream_t s, int order = 4);
+                           cudaStream_t s, int order = 4, bool op_class = false);
 // tiles: of a deriv_tiles list (at most kDerivCols columns, 32 wide, 32 high).
 cudaError_t launch_z4c_derivs_split(const double* Y, double* scratch, long fs, int sy, int sz,
-                                    const Tile* tiles, int ntiles, cudaStream_t s, int order);
+                                    const Tile* tiles, int ntiles, cudaStream_t s, int order, bool op_class = false);
 // bps: warps per scheduler that the stage kernel's build leaves registers for, 2
 // or 3 (a tuning choice); cudaErrorInvalidValue otherwise.  op_class: the PlainK
 // build (stage form kStageSingle only, cudaErrorInvalidValue for the others).

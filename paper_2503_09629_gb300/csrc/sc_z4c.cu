@@ -112,15 +112,17 @@ __device__ __forceinline__ int d2_field(int s) { return s <= 6 ? s : s + 11; }
 // Centred first derivative as the integer-weight sum, lo[m - 1] = v_-m, hi[m - 1] = v_m:
 // 4th order 8 (v_1 - v_-1) - (v_2 - v_-2) (= 12 h u'), 8th order
 // 672 d1 - 168 d2 + 32 d3 - 3 d4 (= 840 h u'), dm = v_m - v_-m, in FP64.
-template <int ORD>
-__device__ __forceinline__ double dfirst_fp64(const double* lo, const double* hi) {
-  if (ORD == 4) return fma(8.0, hi[0], fma(-8.0, lo[0], lo[1] - hi[1]));
-  return fma(672.0, hi[0] - lo[0], fma(-168.0, hi[1] - lo[1], fma(32.0, hi[2] - lo[2], -3.0 * (hi[3] - lo[3]))));
+template <int ORD, class KT>
+__device__ __forceinline__ double dfirst_fp64(const double* lo, const double* hi, const KT& K) {
+  if (ORD == 4) return fma(8.0, hi[0], fma(-8.0, lo[0], fsub(lo[1], hi[1], K)));
+  return fma(672.0, fsub(hi[0], lo[0], K),
+             fma(-168.0, fsub(hi[1], lo[1], K),
+                 fma(32.0, fsub(hi[2], lo[2], K), fmul(-3.0, fsub(hi[3], lo[3], K), K))));
 }
 
 // The same in aligned integers (sc_fixed.cuh), or in FP64 where the values do not allow that.
-template <int ORD>
-__device__ __forceinline__ double dfirst(const double* lo, const double* hi) {
+template <int ORD, class KT>
+__device__ __forceinline__ double dfirst(const double* lo, const double* hi, const KT& K) {
   using F = FxSums<ORD>;
   int Ei = 0, E = 0;
 #pragma unroll
@@ -131,12 +133,12 @@ __device__ __forceinline__ double dfirst(const double* lo, const double* hi) {
   }
   E = max(E, Ei);
   if (aligned_ok(E) && E - Ei <= F::kFirstExcess << 20) return F::first(lo, hi, E);
-  return dfirst_fp64<ORD>(lo, hi);
+  return dfirst_fp64<ORD>(lo, hi, K);
 }
 
-template <int ORD>
+template <int ORD, class KT = FmaK>
 __global__ void __launch_bounds__(128) z4c_dxy_kernel(const double* __restrict__ Y, double* __restrict__ S, long fs,
-                                                     int sy_, const RowSeg* __restrict__ segs, int nsegs) {
+                                                     int sy_, const RowSeg* __restrict__ segs, int nsegs, KT K) {
   constexpr int R = ORD / 2;
   const long sy = sy_;
   for (int sgi = blockIdx.x; sgi < nsegs; sgi += gridDim.x) {
@@ -153,7 +155,7 @@ __global__ void __launch_bounds__(128) z4c_dxy_kernel(const double* __restrict__
           lo[m - 1] = u[-m];
           hi[m - 1] = u[m];
         }
-        S[(long)(Q_D1 + 3 * f + 0) * fs + o] = dfirst<ORD>(lo, hi);
+        S[(long)(Q_D1 + 3 * f + 0) * fs + o] = dfirst<ORD>(lo, hi, K);
       }
       if (sg.which & 2) {
 #pragma unroll
@@ -161,7 +163,7 @@ __global__ void __launch_bounds__(128) z4c_dxy_kernel(const double* __restrict__
           lo[m - 1] = u[-m * sy];
           hi[m - 1] = u[m * sy];
         }
-        S[(long)(Q_D1 + 3 * f + 1) * fs + o] = dfirst<ORD>(lo, hi);
+        S[(long)(Q_D1 + 3 * f + 1) * fs + o] = dfirst<ORD>(lo, hi, K);
       }
     }
   }
@@ -171,26 +173,21 @@ __global__ void __launch_bounds__(128) z4c_dxy_kernel(const double* __restrict__
 // three axes (lo[d][m - 1] = u at -m along d), in FP64: D_d of the axes in
 // dmask, the Kreiss-Oliger sum and, for d2 != null, the pure second
 // derivatives.  The form of the cells that aligned_ok refuses.
-template <int ORD>
+template <int ORD, class KT>
 __device__ __forceinline__ void cell_sums_fp64(double u0, const double (*lo)[ORD == 4 ? 3 : 4],
                                                const double (*hi)[ORD == 4 ? 3 : 4], double* d1, double* ko,
-                                               double* d2) {
+                                               double* d2, const KT& K) {
   double P[3] = {0.0, 0.0, 0.0};
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     double p[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-    for (int m = 0; m < (ORD == 4 ? 3 : 4); ++m) p[m] = lo[d][m] + hi[d][m];
-    if (ORD == 4) {
-      d1[d] = fma(8.0, hi[d][0], fma(-8.0, lo[d][0], lo[d][1] - hi[d][1]));
-      d2[d] = fma(16.0, p[0], fma(-30.0, u0, -p[1]));
-    } else {
-      d1[d] = fma(672.0, hi[d][0] - lo[d][0],
-                  fma(-168.0, hi[d][1] - lo[d][1], fma(32.0, hi[d][2] - lo[d][2], -3.0 * (hi[d][ORD == 4 ? 0 : 3] - lo[d][ORD == 4 ? 0 : 3]))));
-      d2[d] = fma(-14350.0, u0, fma(8064.0, p[0], fma(-1008.0, p[1], fma(128.0, p[2], -9.0 * p[3]))));
-    }
+    for (int m = 0; m < (ORD == 4 ? 3 : 4); ++m) p[m] = fadd(lo[d][m], hi[d][m], K);
+    d1[d] = dfirst_fp64<ORD>(lo[d], hi[d], K);
+    if (ORD == 4) d2[d] = fma(16.0, p[0], fma(-30.0, u0, -p[1]));
+    else d2[d] = fma(-14350.0, u0, fma(8064.0, p[0], fma(-1008.0, p[1], fma(128.0, p[2], fmul(-9.0, p[3], K)))));
 #pragma unroll
-    for (int m = 0; m < 3; ++m) P[m] += p[m];
+    for (int m = 0; m < 3; ++m) P[m] = d == 0 ? p[m] : fadd(P[m], p[m], K);
   }
   *ko = fma(15.0, P[0], fma(-6.0, P[1], fma(-60.0, u0, P[2])));
 }
@@ -209,10 +206,10 @@ __device__ __forceinline__ void cell_sums_fp64(double u0, const double (*lo)[ORD
 // cells, 0.347 and 0.353 (0.329).  With the mixed derivatives in FP64 instead: 0.211 and
 // 0.444 (star alignment); with three or four blocks per SM and reads in place of the
 // windows: 0.219 and 0.238.
-template <int ORD>
+template <int ORD, class KT = FmaK>
 __global__ void __launch_bounds__(kDerivCols, 2)
     z4c_derivs_split_kernel(const double* __restrict__ Y, double* __restrict__ S, long fs, int sy_, int sz_,
-                            const Tile* __restrict__ tiles, int ntiles) {
+                            const Tile* __restrict__ tiles, int ntiles, KT K) {
   using F = FxSums<ORD>;
   constexpr int R = ORD / 2;
   constexpr int WR = R > 3 ? R : 3;
@@ -334,7 +331,7 @@ __global__ void __launch_bounds__(kDerivCols, 2)
             fl[dim][m - 1] = v[-m * st[dim]];
             fh[dim][m - 1] = v[m * st[dim]];
           }
-        cell_sums_fp64<ORD>(v[0], fl, fh, e1, &eko, e2);
+        cell_sums_fp64<ORD>(v[0], fl, fh, e1, &eko, e2, K);
         *ko = eko;
 #pragma unroll
         for (int dim = 0; dim < 3; ++dim) {
@@ -351,7 +348,7 @@ __global__ void __launch_bounds__(kDerivCols, 2)
             ml[m - 1] = d[-m * st];
             mh[m - 1] = d[m * st];
           }
-          return dfirst<ORD>(ml, mh);
+          return dfirst<ORD>(ml, mh, K);
         };
         d2[1 * fs] = mixed(Dx + k * sz, sy);
         if (kWindows) {
@@ -364,7 +361,7 @@ __global__ void __launch_bounds__(kDerivCols, 2)
             }
 #pragma unroll
             for (int m = 0; m < ND - 1; ++m) v[m] = v[m + 1];
-            return dfirst<ORD>(ml, mh);
+            return dfirst<ORD>(ml, mh, K);
           };
           d2[2 * fs] = window(wx);
           d2[4 * fs] = window(wy);
@@ -518,23 +515,41 @@ cudaError_t launch_z4c_derivs(const double* Y, double* scratch, long fs, int sy,
   return cudaGetLastError();
 }
 
+namespace {
+
+template <class KT>
+void launch_dxy(const double* Y, double* scratch, long fs, int sy, const RowSeg* segs, int nsegs, int grid,
+                cudaStream_t s, int order, const KT& K) {
+  if (order == 8) z4c_dxy_kernel<8, KT><<<grid, 128, 0, s>>>(Y, scratch, fs, sy, segs, nsegs, K);
+  else z4c_dxy_kernel<4, KT><<<grid, 128, 0, s>>>(Y, scratch, fs, sy, segs, nsegs, K);
+}
+
+template <class KT>
+void launch_derivs(const double* Y, double* scratch, long fs, int sy, int sz, const Tile* tiles, int ntiles, int grid,
+                   cudaStream_t s, int order, const KT& K) {
+  if (order == 8) z4c_derivs_split_kernel<8, KT><<<grid, kDerivCols, 0, s>>>(Y, scratch, fs, sy, sz, tiles, ntiles, K);
+  else z4c_derivs_split_kernel<4, KT><<<grid, kDerivCols, 0, s>>>(Y, scratch, fs, sy, sz, tiles, ntiles, K);
+}
+
+}  // namespace
+
 cudaError_t launch_z4c_dxy(const double* Y, double* scratch, long fs, int sy, const RowSeg* segs, int nsegs,
-                           cudaStream_t s, int order) {
+                           cudaStream_t s, int order, bool op_class) {
   if (nsegs == 0) return cudaSuccess;
   const int grid = nsegs < caps().dxy ? nsegs : caps().dxy;
-  if (order == 8) z4c_dxy_kernel<8><<<grid, 128, 0, s>>>(Y, scratch, fs, sy, segs, nsegs);
-  else z4c_dxy_kernel<4><<<grid, 128, 0, s>>>(Y, scratch, fs, sy, segs, nsegs);
+  if (op_class) launch_dxy(Y, scratch, fs, sy, segs, nsegs, grid, s, order, PlainK{});
+  else launch_dxy(Y, scratch, fs, sy, segs, nsegs, grid, s, order, FmaK{1.0, -1.0, -0.0});
   return cudaGetLastError();
 }
 
 cudaError_t launch_z4c_derivs_split(const double* Y, double* scratch, long fs, int sy, int sz, const Tile* tiles,
-                                    int ntiles, cudaStream_t s, int order) {
+                                    int ntiles, cudaStream_t s, int order, bool op_class) {
   if (ntiles == 0) return cudaSuccess;
   const long items = (long)ntiles * kNZ4c;
   const int cap = caps().derivs[order == 8];
   const int grid = items < cap ? (int)items : cap;
-  if (order == 8) z4c_derivs_split_kernel<8><<<grid, kDerivCols, 0, s>>>(Y, scratch, fs, sy, sz, tiles, ntiles);
-  else z4c_derivs_split_kernel<4><<<grid, kDerivCols, 0, s>>>(Y, scratch, fs, sy, sz, tiles, ntiles);
+  if (op_class) launch_derivs(Y, scratch, fs, sy, sz, tiles, ntiles, grid, s, order, PlainK{});
+  else launch_derivs(Y, scratch, fs, sy, sz, tiles, ntiles, grid, s, order, FmaK{1.0, -1.0, -0.0});
   return cudaGetLastError();
 }
 
