@@ -541,12 +541,25 @@ __device__ __forceinline__ void wave_stage_body(const StageArgs& a, const Tile* 
         lap = F::laplacian(v, w[R], E);
       } else {
         const double* c = u + k * sz;
-        double s[4];
+        double p[R][6];
+        unsigned any = zero_bits(c[0]);
 #pragma unroll
-        for (int m = 1; m <= R; ++m)
-          s[m - 1] = ((c[-m] + c[m]) + (c[-m * sy] + c[m * sy])) + (c[-m * sz] + c[m * sz]);
-        if (ORD == 4) lap = fma(-90.0, c[0], fma(16.0, s[0], -s[1]));
-        else lap = fma(-43050.0, c[0], fma(8064.0, s[0], fma(-1008.0, s[1], fma(128.0, s[2], -9.0 * s[3]))));
+        for (int m = 1; m <= R; ++m) {
+          const double q[6] = {c[-m], c[m], c[-m * sy], c[m * sy], c[-m * sz], c[m * sz]};
+#pragma unroll
+          for (int n = 0; n < 6; ++n) {
+            p[m - 1][n] = q[n];
+            any |= zero_bits(q[n]);
+          }
+        }
+        lap = 0.0;
+        if (any) {
+          double s[4];
+#pragma unroll
+          for (int m = 0; m < R; ++m) s[m] = ((p[m][0] + p[m][1]) + (p[m][2] + p[m][3])) + (p[m][4] + p[m][5]);
+          if (ORD == 4) lap = fma(-90.0, c[0], fma(16.0, s[0], -s[1]));
+          else lap = fma(-43050.0, c[0], fma(8064.0, s[0], fma(-1008.0, s[1], fma(128.0, s[2], -9.0 * s[3]))));
+        }
       }
       const double kp = fmul(lap, a.ds.s2p, K);  // d_t Pi = Laplacian u, its sum over 12 h^2 or 5040 h^2
       a.k[o] = ku;

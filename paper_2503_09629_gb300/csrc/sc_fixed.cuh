@@ -22,9 +22,9 @@
 // 2.3e-14 for a Laplacian of 4th order, 4.7e-17 against 2.8e-14 of 8th).
 // The result depends on the stencil's values alone, not on tiles or boxes.
 //
-// Stencils that hold an infinity or a NaN, that vanish, or whose largest value
-// lies near either end of the exponent range are left to the FP64 form too
-// (aligned_ok, packed_ok).
+// Stencils that hold an infinity or a NaN, or whose largest value lies near either
+// end of the exponent range are left to the FP64 form too (aligned_ok,
+// packed_ok), unless they are all zeros (zero_bits), as fields at rest are.
 #pragma once
 
 #include "sc_internal.h"
@@ -52,6 +52,10 @@ __device__ __forceinline__ Fx fx_unpack(double v) {
   return r;
 }
 
+// Zero for zeros of either sign only.
+__device__ __forceinline__ unsigned zero_bits(double v) {
+  return (unsigned)__double2hiint(v) << 1 | (unsigned)__double2loint(v);
+}
 // The exponent field of a value, in place.
 __device__ __forceinline__ int fx_exp(double v) { return __double2hiint(v) & 0x7ff00000; }
 

@@ -133,6 +133,10 @@ __device__ __forceinline__ double dfirst(const double* lo, const double* hi, con
   }
   E = max(E, Ei);
   if (aligned_ok(E) && E - Ei <= F::kFirstExcess << 20) return F::first(lo, hi, E);
+  unsigned any = 0;
+#pragma unroll
+  for (int m = 0; m < ORD / 2; ++m) any |= zero_bits(lo[m]) | zero_bits(hi[m]);
+  if (any == 0) return 0.0;
   return dfirst_fp64<ORD>(lo, hi, K);
 }
 
@@ -324,14 +328,22 @@ __global__ void __launch_bounds__(kDerivCols, 2)
         const double* v = u + k * sz;
         double fl[3][ORD == 4 ? 3 : 4], fh[3][ORD == 4 ? 3 : 4], e1[3], e2[3], eko;
         const long st[3] = {1, sy, sz};
+        unsigned any = zero_bits(v[0]);
 #pragma unroll
         for (int dim = 0; dim < 3; ++dim)
 #pragma unroll
           for (int m = 1; m <= WR; ++m) {
             fl[dim][m - 1] = v[-m * st[dim]];
             fh[dim][m - 1] = v[m * st[dim]];
+            any |= zero_bits(fl[dim][m - 1]) | zero_bits(fh[dim][m - 1]);
           }
-        cell_sums_fp64<ORD>(v[0], fl, fh, e1, &eko, e2, K);
+        if (any) {
+          cell_sums_fp64<ORD>(v[0], fl, fh, e1, &eko, e2, K);
+        } else {
+          eko = 0.0;
+#pragma unroll
+          for (int dim = 0; dim < 3; ++dim) e1[dim] = e2[dim] = 0.0;
+        }
         *ko = eko;
 #pragma unroll
         for (int dim = 0; dim < 3; ++dim) {
