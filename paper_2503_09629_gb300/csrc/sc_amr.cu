@@ -250,6 +250,18 @@ __global__ void __launch_bounds__(kThreads) pack_fields_kernel(double* __restric
   }
 }
 
+// Data to time kernels on: flat space (Z4c) or zero plus a thousandth of noise.
+__global__ void __launch_bounds__(kThreads) sample_kernel(double* __restrict__ vec, long fs, int F, int system) {
+  const long n = fs * F;
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
+    const int f = (int)(i / fs);
+    const bool one = system == SC_Z4C && (f == ZW || f == ZG || f == ZG + 3 || f == ZG + 5 || f == ZAL);
+    unsigned h = (unsigned)i * 2654435761u;
+    h = (h ^ (h >> 15)) * 2246822519u;
+    vec[i] = (one ? 1.0 : 0.0) + 1e-3 * (int)h * 0x1p-31;
+  }
+}
+
 __global__ void __launch_bounds__(kThreads) nonfinite_kernel(const double* __restrict__ vec, long fs, int F,
                                                             const Tile* __restrict__ tiles, int ntiles,
                                                             int sy, int sz, int* flag) {
@@ -384,6 +396,11 @@ cudaError_t launch_pack_fields(double* vec, long fs, int F, const Geom& g, const
   if (blocks > sm_count() * 16L) blocks = sm_count() * 16L;
   pack_fields_kernel<<<(int)blocks, kThreads, 0, s>>>(vec, fs, F, g.pitch, g.ext[1], lo[0] - g.org[0], lo[1] - g.org[1],
                                                       lo[2] - g.org[2], n[0], n[1], n[2], buf, unpack);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sample_data(double* vec, long fs, int F, int system, cudaStream_t s) {
+  sample_kernel<<<grid_for(fs * F, kThreads), kThreads, 0, s>>>(vec, fs, F, system);
   return cudaGetLastError();
 }
 

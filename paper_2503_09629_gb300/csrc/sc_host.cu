@@ -1598,7 +1598,7 @@ sc_status sc::set_last_error(sc_status code, const char* msg) { return fail(code
 namespace {
 
 std::mutex g_tune_mutex;
-// per (system, level shapes): tile shape, derivative form, stage blocks per SM
+// per (system, order, level shapes): tile shape, derivative form, stage kernel build
 std::map<std::string, std::array<int, 5>> g_tune_cache;
 
 std::string tune_key(const sc_ctx* c) {
@@ -1636,9 +1636,9 @@ StageArgs tuning_stage_args(const Level& L, int order) {
 }
 
 // Time one candidate on one level with CUDA events on the context's stream
-// (one untimed launch first, then reps): kind 0 = the stencil kernel with the
-// given tiles (the wave's fused stage, or the Z4c derivative pass in the form
-// deriv_form), kind 1 = the Z4c stage kernel built for bps blocks per SM.
+// (one untimed launch first, then reps): kind 0 = the stencil kernel (the wave's
+// fused stage, or the Z4c derivative pass in the form deriv_form, its one-kernel
+// form with the given tiles), kind 1 = the Z4c stage kernel's build bps.
 sc_status time_candidate(sc_ctx* c, Level& L, int kind, const Tile* tiles, int ntiles, int deriv_form,
                          int bps, int reps, double* ms) {
   const Geom& g = L.g;
@@ -1693,18 +1693,17 @@ sc_status apply_tuning(sc_ctx* c, const int* shape, int deriv_form, int bps) {
 
 }  // namespace
 
-// Autotuner (the search space: derivative-pass split x stage kernel blocks per
-// SM; the wave stage and the two-kernel derivative pass have tiles of their own).  On the context's largest level it times every tile
-// shape of the stencil kernel (the wave's fused stage, or the Z4c derivative
-// pass in its two-kernel form), the one-kernel Z4c derivative pass (4th
-// order, default tiles), and the Z4c stage kernel built for 2 and for 3 blocks
-// per SM; it keeps the fastest derivative configuration and the faster stage
-// build.  All forms compute the same derivatives (the one-kernel form sums the
-// mixed stencils in another order, so its results differ by rounding).
+// Autotuner.  On the context's largest level it times the Z4c derivative pass in
+// its two-kernel and (4th order) one-kernel forms and the Z4c stage kernel built
+// for 2 and for 3 warps per scheduler, on sample data in the stage buffer (its kernels
+// are faster on ordinary values than on the zeros of a new context), and keeps the
+// faster ones.  All forms compute the same derivatives (the one-kernel form sums
+// the mixed stencils in another order, so its results differ by rounding).  The
+// wave stage has nothing to tune: it is timed only.
 extern "C" sc_status sc_autotune(sc_ctx* c, int* tile_out, double* ms_out) {
   if (!c) return fail(SC_EINVAL, "null context");
   const std::string key = tune_key(c);
-  std::array<int, 5> best{c->tile[0], c->tile[1], c->tile[2], c->deriv_form, c->stage_bps};
+  std::array<int, 5> best{32, 4, 2, 0, c->stage_bps};
   double best_ms = -1.0;
   bool cached = false;
   {
@@ -1720,33 +1719,22 @@ extern "C" sc_status sc_autotune(sc_ctx* c, int* tile_out, double* ms_out) {
     for (int l = 1; l < c->nlev; ++l)
       if (c->lev[l].interior_cells > c->lev[big].interior_cells) big = l;
     Level& L = c->lev[big];
-    static const int cand[][3] = {{32, 4, 2}, {32, 2, 4}, {32, 1, 8}, {32, 4, 4}, {32, 2, 8}, {32, 1, 16},
-                                  {16, 4, 8}, {64, 1, 8}, {16, 2, 16}, {32, 1, 32}};
+    std::vector<Tile> t;  // of the one-kernel form
+    build_stencil_tiles(L, best.data(), t);
+    Tile* d = (Tile*)c->dalloc(t.size() * sizeof(Tile));
+    if (!d) return fail(SC_ENOMEM, "autotune tile buffer");
+    CU(cudaMemcpyAsync(d, t.data(), t.size() * sizeof(Tile), cudaMemcpyHostToDevice, c->stream));
+    CU(launch_sample_data(L.A, L.g.fs, c->F, c->system, c->stream));
     const int nform = (c->system == SC_Z4C && c->order == 4) ? 2 : 1;
-    std::vector<Tile> t;
-    Tile* d = nullptr;
-    size_t cap = 0;
-    std::vector<void*> scratch_lists;
-    for (int form = 0; form < nform; ++form)
-      for (const auto& cd : cand) {
-        // the wave stage and the two-kernel Z4c form have tiles of their own, the one-kernel form takes these
-        if (cd[0] != 32 || cd[1] != 4 || cd[2] != 2) continue;
-        build_stencil_tiles(L, cd, t);
-        if (t.size() > cap) {
-          cap = t.size() * 2;
-          d = (Tile*)c->dalloc(cap * sizeof(Tile));
-          if (!d) return fail(SC_ENOMEM, "autotune tile buffer");
-          scratch_lists.push_back(d);
-        }
-        CU(cudaMemcpyAsync(d, t.data(), t.size() * sizeof(Tile), cudaMemcpyHostToDevice, c->stream));
-        double ms = 0;
-        sc_status st = time_candidate(c, L, 0, d, (int)t.size(), form, 0, 3, &ms);
-        if (st) return st;
-        if (best_ms < 0 || ms < best_ms) {
-          best_ms = ms;
-          best = {cd[0], cd[1], cd[2], form, best[4]};
-        }
+    for (int form = 0; form < nform; ++form) {
+      double ms = 0;
+      sc_status st = time_candidate(c, L, 0, d, (int)t.size(), form, 0, 3, &ms);
+      if (st) return st;
+      if (best_ms < 0 || ms < best_ms) {
+        best_ms = ms;
+        best[3] = form;
       }
+    }
     if (c->system == SC_Z4C) {
       double ms2 = 0, ms3 = 0;
       sc_status st = time_candidate(c, L, 1, nullptr, 0, 0, 2, 3, &ms2);
@@ -1754,8 +1742,10 @@ extern "C" sc_status sc_autotune(sc_ctx* c, int* tile_out, double* ms_out) {
       if (st) return st;
       best[4] = ms2 < ms3 ? 2 : 3;
     }
+    // (as at creation: ghost cells that no stage writes are zero)
+    CU(cudaMemsetAsync(L.A, 0, sizeof(double) * (size_t)c->F * L.g.fs, c->stream));
     CU(cudaStreamSynchronize(c->stream));
-    for (void* p : scratch_lists) c->dfree(p);
+    c->dfree(d);
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     g_tune_cache[key] = best;
   }

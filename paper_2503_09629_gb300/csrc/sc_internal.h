@@ -294,6 +294,7 @@ cudaError_t launch_unpack(double* vec, const Geom& g, const int* lo, const int* 
 // consecutive x-fastest blocks); unpack = 1 writes the array.
 cudaError_t launch_pack_fields(double* vec, long fs, int F, const Geom& g, const int* lo, const int* n, double* buf,
                                int unpack, cudaStream_t s);
+cudaError_t launch_sample_data(double* vec, long fs, int F, int system, cudaStream_t s);
 cudaError_t launch_nonfinite_check(const double* vec, long fs, int F, const Tile* tiles, int ntiles, int sy,
                                    int sz, int* flag, cudaStream_t s);
 
