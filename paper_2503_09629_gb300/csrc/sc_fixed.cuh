@@ -17,7 +17,7 @@
 // weight: at most 2^-54 of its largest weighted term.  At 8th order the weights
 // are too far apart for that (1 to 8192), and sums whose lightly weighted outer
 // values are 2^3 to 2^5 times the inner ones are left to FP64, whose error
-// is relative to the weighted values (kFirstExcess and so on; inside these limits the
+// is relative to the weighted values (kExcess1 and so on; inside these limits the
 // integer sums were the more accurate ones: on random values 1.4e-16 against
 // 2.3e-14 for a Laplacian of 4th order, 4.7e-17 against 2.8e-14 of 8th).
 // The result depends on the stencil's values alone, not on tiles or boxes.
@@ -134,11 +134,10 @@ struct FxSums;
 
 template <>
 struct FxSums<4> {
-  static constexpr int kInner = 2;         // first derivatives: every value counts as an inner one
-  static constexpr int kFirstExcess = 0;
-  // One axis of a star: u0 and the values at +-3 (Kreiss-Oliger) may be 2^2 times those of the
-  // first derivative; its error is then 2^-57 of their largest, FP64's 2^-55 of the latter's.
-  static constexpr int kAxisExcess = 2;
+  // One axis of a star: by how many powers of two its largest value, u0 or one at +-3, may
+  // exceed those at +-1 and those at +-2 (one of the two; RMS error of the first
+  // derivative 0.07 units of 2^-53 of the largest, FP64: 3.3 of v_1 or 0.5 of v_2).
+  static constexpr int kExcess1 = 4, kExcess2 = 2;
   static constexpr int kLaplacianExcess = 1023;
   // 8 (v_1 - v_-1) - (v_2 - v_-2) = 12 h u'
   __device__ static __forceinline__ double first(const double* lo, const double* hi, int E) {
@@ -189,9 +188,9 @@ struct FxSums<4> {
 template <>
 struct FxSums<8> {
   static constexpr int kGuard = 6;  // 59 bits: sums of six values and their halves stay in range
-  // Outer values (+-3, +-4, weights 32 and 3) against those at +-1 and +-2 (672, 168): error of
-  // the integers 9 2^-53 of the largest value, of FP64 67 to 270 2^-53 of the inner ones.
-  static constexpr int kInner = 2, kFirstExcess = 3, kAxisExcess = 3;
+  // As at 4th order, with the outer values of the derivative itself (+-3, +-4, weights 32 and 3
+  // against 672 and 168): 9 units of 2^-53 of the largest, FP64: 270 of v_1 or 67 of v_2.
+  static constexpr int kExcess1 = 4, kExcess2 = 3;
   // Values at +-2, +-3, +-4 (1008, 128, 9) against u0 and those at +-1 (43050, 8064):
   // 430 2^-53 against 2e4 2^-53.
   static constexpr int kLaplacianExcess = 5;

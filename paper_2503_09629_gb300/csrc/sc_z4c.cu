@@ -124,15 +124,11 @@ __device__ __forceinline__ double dfirst_fp64(const double* lo, const double* hi
 template <int ORD, class KT>
 __device__ __forceinline__ double dfirst(const double* lo, const double* hi, const KT& K) {
   using F = FxSums<ORD>;
-  int Ei = 0, E = 0;
+  const int E1 = max(fx_exp(lo[0]), fx_exp(hi[0])), E2 = max(fx_exp(lo[1]), fx_exp(hi[1]));
+  int E = max(E1, E2);
 #pragma unroll
-  for (int m = 0; m < ORD / 2; ++m) {
-    const int e = max(fx_exp(lo[m]), fx_exp(hi[m]));
-    if (m < F::kInner) Ei = max(Ei, e);
-    else E = max(E, e);
-  }
-  E = max(E, Ei);
-  if (aligned_ok(E) && E - Ei <= F::kFirstExcess << 20) return F::first(lo, hi, E);
+  for (int m = 2; m < ORD / 2; ++m) E = max(E, max(fx_exp(lo[m]), fx_exp(hi[m])));
+  if (aligned_ok(E) && (ORD == 4 || E - E1 <= F::kExcess1 << 20 || E - E2 <= F::kExcess2 << 20)) return F::first(lo, hi, E);
   unsigned any = 0;
 #pragma unroll
   for (int m = 0; m < ORD / 2; ++m) any |= zero_bits(lo[m]) | zero_bits(hi[m]);
@@ -204,10 +200,10 @@ __device__ __forceinline__ void cell_sums_fp64(double u0, const double (*lo)[ORD
 // 32 high; a plane then holds at most 38 x 14 (40 x 16) values.  At 4th order D_x
 // and D_y along z are windows in registers too; at 8th order these would spill,
 // and are read again (L1).  Integer ALU 45%, latency of 16 warps: 262,144 cells with
-// the row pass before it, 0.251 ms with a thread per column and no sharing, 0.207
+// the row pass before it, 0.251 ms with a thread per column and no sharing, 0.209
 // so (0.200 with one alignment for a cell's whole star, whose error in a derivative was
-// relative to the values along the other axes too); 110,592 cells 0.119 and 0.110; 8th order, 262,144
-// cells, 0.347 and 0.353 (0.329).  With the mixed derivatives in FP64 instead: 0.211 and
+// relative to the values along the other axes too); 110,592 cells 0.119 and 0.111; 8th order, 262,144
+// cells, 0.347 and 0.357 (0.329).  With the mixed derivatives in FP64 instead: 0.211 and
 // 0.444 (star alignment); with three or four blocks per SM and reads in place of the
 // windows: 0.219 and 0.238.
 template <int ORD, class KT = FmaK>
@@ -292,15 +288,13 @@ __global__ void __launch_bounds__(kDerivCols, 2)
       bool ok = true;
 #pragma unroll
       for (int dim = 0; dim < 3; ++dim) {
-        int Ei = 0, E = fx_pexp(w[WR]);
+        const int E1 = max(fx_pexp(at(dim, -1)), fx_pexp(at(dim, 1)));
+        const int E2 = max(fx_pexp(at(dim, -2)), fx_pexp(at(dim, 2)));
+        int E = max(fx_pexp(w[WR]), max(E1, E2));
 #pragma unroll
-        for (int m = 1; m <= WR; ++m) {
-          const int e = max(fx_pexp(at(dim, -m)), fx_pexp(at(dim, m)));
-          if (m <= F::kInner) Ei = max(Ei, e);
-          else E = max(E, e);
-        }
-        Ed[dim] = max(E, Ei);
-        ok = ok && packed_ok(Ed[dim]) && Ed[dim] - Ei <= F::kAxisExcess;
+        for (int m = 3; m <= WR; ++m) E = max(E, max(fx_pexp(at(dim, -m)), fx_pexp(at(dim, m))));
+        Ed[dim] = E;
+        ok = ok && packed_ok(E) && (E - E1 <= F::kExcess1 || E - E2 <= F::kExcess2);
       }
       double* d1 = S + (long)(Q_D1 + 3 * f) * fs + o;
       double* d2 = S + (long)(Q_D2 + 6 * sl) * fs + o;
