@@ -2355,37 +2355,38 @@ sc_status sc_get_constraints(sc_ctx* c, int level, int box, double* dst) {
   const long ncell = (long)n[0] * n[1] * n[2];
   const size_t bytes = sizeof(double) * kNCons * (size_t)ncell;
   if ((st = ensure_staging(c, bytes))) return st;
-  // tiles of this box only
-  std::vector<Tile> tl;
-  for (int z = B.lo[2]; z <= B.hi[2]; z += 2)
-    for (int y = B.lo[1]; y <= B.hi[1]; y += 4)
-      for (int x = B.lo[0]; x <= B.hi[0]; x += 32) {
-        Tile t;
-        t.x0 = x - L.g.org[0];
-        t.y0 = y - L.g.org[1];
-        t.z0 = z - L.g.org[2];
-        t.nx = std::min(32, B.hi[0] - x + 1);
-        t.ny = std::min(4, B.hi[1] - y + 1);
-        t.nz = std::min(2, B.hi[2] - z + 1);
-        tl.push_back(t);
-      }
-  Tile* dt = (Tile*)c->dalloc(tl.size() * sizeof(Tile));
-  if (!dt) return fail(SC_ENOMEM, "tile list allocation failed");
-  CU(cudaMemcpyAsync(dt, tl.data(), tl.size() * sizeof(Tile), cudaMemcpyHostToDevice, c->stream));
   const double* Y = L.S[L.parity];
   const int sy = L.g.pitch, sz = L.g.pitch * L.g.ext[1];
   const int blo[3] = {B.lo[0] - L.g.org[0], B.lo[1] - L.g.org[1], B.lo[2] - L.g.org[2]};
+  Tile* dt = nullptr;  // 4th order: a list of this box's tiles for the one-kernel form
   if (c->order == 4) {
+    std::vector<Tile> tl;
+    for (int z = B.lo[2]; z <= B.hi[2]; z += 2)
+      for (int y = B.lo[1]; y <= B.hi[1]; y += 4)
+        for (int x = B.lo[0]; x <= B.hi[0]; x += 32) {
+          Tile t;
+          t.x0 = x - L.g.org[0];
+          t.y0 = y - L.g.org[1];
+          t.z0 = z - L.g.org[2];
+          t.nx = std::min(32, B.hi[0] - x + 1);
+          t.ny = std::min(4, B.hi[1] - y + 1);
+          t.nz = std::min(2, B.hi[2] - z + 1);
+          tl.push_back(t);
+        }
+    dt = (Tile*)c->dalloc(tl.size() * sizeof(Tile));
+    if (!dt) return fail(SC_ENOMEM, "tile list allocation failed");
+    CU(cudaMemcpyAsync(dt, tl.data(), tl.size() * sizeof(Tile), cudaMemcpyHostToDevice, c->stream));
     CU(launch_z4c_derivs(Y, c->scratch, L.g.fs, sy, sz, dt, (int)tl.size(), c->stream));
   } else {
     CU(launch_z4c_dxy(Y, c->scratch, L.g.fs, sy, L.dxy, L.ndxy, c->stream, c->order));
     CU(launch_z4c_derivs_split(Y, c->scratch, L.g.fs, sy, sz, L.dtiles + L.box_dtile_begin[box],
                                L.box_dtile_begin[box + 1] - L.box_dtile_begin[box], c->stream, c->order));
   }
-  CU(launch_z4c_constraints(Y, c->scratch, c->staging, L.g.fs, sy, sz, deriv_scales(c->order, L.g.h), L.g.h, ncell, blo, n, c->stream));
+  CU(launch_z4c_constraints(Y, c->scratch, c->staging, L.g.fs, sy, sz, deriv_scales(c->order, L.g.h), L.g.h, ncell, blo,
+                            n, c->stream));
   CU(cudaMemcpyAsync(dst, c->staging, bytes, cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));
-  c->dfree(dt);  // the per-call tile list (the stream is idle)
+  if (dt) c->dfree(dt);  // the per-call tile list (the stream is idle)
   return SC_OK;
 }
 

@@ -37,12 +37,18 @@ def _steep(rng, shape, axis, bits):
 
 @pytest.mark.parametrize("order", [4, 8])
 @pytest.mark.parametrize("axis", [0, 1, 2])
-@pytest.mark.parametrize("bits", [0, 1, 3, 10])
+@pytest.mark.parametrize("bits", [0, 1, 3, 10, "mixed", "large"])
 def test_laplacian_against_exact_sums(sc, order, axis, bits):
     n = 16
     h = W.Hierarchy(system=W.WAVE, boxes=[[((0, 0, 0), (n - 1,) * 3)]], ncells0=(n,) * 3, origin=(0.0,) * 3, h0=1.0 / n,
                     fd_order=order)
-    u = _steep(np.random.default_rng(5), (n,) * 3, axis, bits)
+    rng = np.random.default_rng(5)
+    if bits == "mixed":  # inside and outside of the range of the integers, cell by cell
+        u = rng.uniform(-1, 1, (n,) * 3) * rng.choice([1.0, 1.0, 0.0, 1e-290, 1e-200, 1e-20], size=(n,) * 3)
+    elif bits == "large":
+        u = rng.uniform(-1, 1, (n,) * 3) * rng.choice([1e300, 1e290, 1.0, -0.0], size=(n,) * 3)
+    else:
+        u = _steep(rng, (n,) * 3, axis, bits)
     ctx = sc.Context(h)
     ctx.sc_set_field(0, 0, 0, u)
     ctx.sc_set_field(0, 0, 1, np.zeros_like(u))
@@ -58,7 +64,8 @@ def test_laplacian_against_exact_sums(sc, order, axis, bits):
                 v = np.roll(exact, s, axis=d)
                 lap, size = lap + c * v, size + abs(c) * abs(v)
     scale = Fraction(n * n, den)
-    worst = max(abs(Fraction(g) - a * scale) / (t * scale) for g, a, t in zip(got.flat, lap.flat, size.flat))
+    worst = max(abs(Fraction(g) - a * scale) / (t * scale) for g, a, t in zip(got.flat, lap.flat, size.flat) if t)
+    assert not any(g for g, t in zip(got.flat, size.flat) if not t)
     assert float(worst) <= BOUND[order]
 
 
