@@ -63,19 +63,27 @@ HBM_GBS = _measured_hbm_gbs()
 # multiplies and fused multiply-adds (2 flops) of the formulation as first
 # written, counted by ncu (z4c_derivs = row-segment D_x/D_y pass 133 +
 # per-cell pass 1047).  Later rewrites evaluate the same right-hand side with
-# fewer FP64 instructions (FP64_INSTR_PER_CELL) and then in integers; the flop
-# counts stay fixed so that achieved rates measure the method's work.
+# fewer FP64 instructions and in part in integers; the flop counts stay fixed so
+# that achieved rates measure the method's work.
 FLOPS_PER_CELL = {"z4c_derivs": 1180.0, "z4c_stage": 1971.0}
+# What the kernels execute and move per interior cell, counted by ncu on a launch over
+# 262,144 cells with cold caches (profiles/integer_kernels_ncu.md): thread-level
+# instructions, those of the FP64 pipe (conversions among them), DRAM bytes read and
+# written.  z4c_derivs = row pass + per-cell pass.
+INSTR_PER_CELL = {4: {"z4c_derivs": 2575.0 + 13876.0, "z4c_stage": 11793.0},
+                  8: {"z4c_derivs": 5291.0 + 21109.0, "z4c_stage": 11793.0}}
+FP64_PIPE_PER_CELL = {4: {"z4c_derivs": 24.1 + 132.0, "z4c_stage": 564.0},
+                      8: {"z4c_derivs": 26.1 + 132.2, "z4c_stage": 564.0}}
+DRAM_BYTES_PER_CELL = {4: {"z4c_derivs": 122.1 + 21.8 + 587.8 + 917.8, "z4c_stage": 1949.3 + 436.5},
+                       8: {"z4c_derivs": 125.6 + 44.8 + 530.5 + 902.3, "z4c_stage": 1882.4 + 424.8}}
 # FP64 instructions (DFMA + DMUL + DADD, thread-level / cell) per interior
-# cell of each pass in its FP64 form, which the production kernels keep for the
-# cells that their integer forms do not take, counted by ncu on the 3-level 64^3 case
+# cell of each pass when all of it was FP64, counted by ncu on the 3-level 64^3 case
 # (profiles/z4c_kernels_bl3level64_ncu.md, profiles/z4c_fp64_op_classes_bl3level64_ncu.md).
 FP64_INSTR_PER_CELL = {4: {"z4c_derivs": 72.1875 + 693.0, "z4c_stage": 1072.0},
                        8: {"z4c_derivs": 209.0 + 1210.0, "z4c_stage": 1072.0}}
 # The same passes split by issue rate (general FMAs, DADD-rate operations:
-# additions, multiplications, unit-multiplier FMAs), counted by ncu on their
-# op-class build (sc_run_op_class_pass, which issues every such operation as
-# a DADD or DMUL; profiles/z4c_fp64_op_classes_bl3level64_ncu.md).
+# additions, multiplications, unit-multiplier FMAs), counted by ncu on the
+# op-class build of that time (profiles/z4c_fp64_op_classes_bl3level64_ncu.md).
 FP64_OP_CLASSES = {4: {"z4c_derivs": (48.125 + 451.0, 24.0625 + 242.0), "z4c_stage": (830.559, 13.0 + 235.445)},
                    8: {"z4c_derivs": (156.75 + 429.0, 52.25 + 781.0), "z4c_stage": (830.559, 13.0 + 235.445)}}
 # Kernel with the largest share of a coarse step in the ncu launch list
@@ -502,8 +510,9 @@ def run_gpu(args, rank: int, world: int):
     launches = ctx.sc_launches_per_step() * args.steps
     state_finite = ctx.sc_check_finite()
 
-    # Roofline of the dominant kernels against the FP64 peak: the method's flops,
-    # which the kernels compute in integers (a fraction may exceed 1).  Per-launch durations
+    # Roofline of the dominant kernels against what binds them: the Z4c stage kernel the
+    # FP64 pipe, the derivative pass the instruction issue (counted instructions over the
+    # measured time).  Per-launch durations
     # from CUDA events on the library's stream, on the finest level; peaks
     # read from this device (nominal from its SM count and clock, and the
     # measured DFMA and DADD issue rates).
@@ -516,19 +525,28 @@ def run_gpu(args, rank: int, world: int):
     roof = {}
     for name, t in (("z4c_derivs", t_der), ("z4c_stage", t_stage)):
         fpc = FLOPS_PER_CELL[name] if (h.fd_order == 4 or name == "z4c_stage") else None
-        ipc = FP64_INSTR_PER_CELL[h.fd_order][name]
         gen, slow = FP64_OP_CLASSES[h.fd_order][name]
-        # shortest time of the FP64 form's instruction mix at the measured issue rates: the production
-        # kernels sum in integers and are not bound by it
+        # shortest time of the all-FP64 form's instruction mix at the measured issue rates
         t_mix = cells * (gen / pk["dfma_g_per_s"] + slow / pk["dadd_g_per_s"]) / 1e9 * 1e3
-        r = {"ms_per_launch": t, "cells_per_launch": cells, "flops_per_cell": fpc,
-             "fp64_form": {"instr_per_cell": ipc, "general_fma_per_cell": gen, "dadd_rate_ops_per_cell": slow,
-                           "mix_ceiling_ms": t_mix, "speedup_over_mix_ceiling": t_mix / t}}
+        rate = cells / (t * 1e-3)
+        issue = INSTR_PER_CELL[h.fd_order][name] * rate / 1e9
+        issue_peak = pk["sms"] * pk["sm_clock_mhz"] * 128 / 1e3
+        fp64 = FP64_PIPE_PER_CELL[h.fd_order][name] * rate / 1e9
+        fp64_peak = nominal_tflops * 1e3 / 2
+        on_fp64 = fp64 / fp64_peak > issue / issue_peak
+        dram = DRAM_BYTES_PER_CELL[h.fd_order][name]
+        r = {"ms_per_launch": t, "cells_per_launch": cells, "bound": "alu",
+             "pipe": "fp64" if on_fp64 else "issue", "achieved": fp64 if on_fp64 else issue,
+             "peak": fp64_peak if on_fp64 else issue_peak, "unit": "G thread instructions/s",
+             "frac": max(fp64 / fp64_peak, issue / issue_peak), "frac_of_fp64_issue": fp64 / fp64_peak,
+             "frac_of_issue": issue / issue_peak, "traffic": dram * cells,
+             "frac_of_hbm": dram * rate / 1e9 / HBM_GBS,
+             "fp64_form": {"instr_per_cell": FP64_INSTR_PER_CELL[h.fd_order][name], "general_fma_per_cell": gen,
+                           "dadd_rate_ops_per_cell": slow, "mix_ceiling_ms": t_mix,
+                           "speedup_over_mix_ceiling": t_mix / t}}
         if fpc is not None:
-            ach = cells * fpc / (t * 1e-3) / 1e12
-            r.update({"bound": "alu", "achieved": ach, "peak": nominal_tflops, "unit": "TFLOP/s",
-                      "frac": ach / nominal_tflops, "frac_of_measured_dfma": ach / dfma_tflops,
-                      "traffic": None})
+            r["method_flops"] = {"per_cell": fpc, "tflops": rate * fpc / 1e12,
+                                 "frac_of_fp64_peak": rate * fpc / 1e12 / nominal_tflops}
         roof[name] = r
     # Refinement-boundary ghost fill on the finest level: the tile-separable
     # prolongation (FP64: the FMAs its tiles execute, counted by the library)

@@ -4,9 +4,16 @@
  * "GPU-accelerated Subcycling Time Integration with the Einstein Toolkit"
  * (arXiv:2503.09629).
  *
- * Library: libsubcyc.so.  All arithmetic is FP64 and runs in CUDA kernels on
- * one GPU; there is no CPU fallback: every compute entry point fails with
- * SC_ECUDA when no device is usable.
+ * Library: libsubcyc.so.  Fields are FP64, and all arithmetic runs in CUDA
+ * kernels on one GPU; there is no CPU fallback: every compute entry point fails
+ * with SC_ECUDA when no device is usable.  Stencil sums, prolongation and the
+ * tensor sums of Z4c that reuse their operands are formed in integers aligned to the
+ * largest term (54 to 60 bits) and rounded once, with these errors at most:
+ * stencil sums 2^-49 (8th order: 2^-48) of the sum of their weighted values'
+ * magnitudes, tensor sums 2^-54 of their largest term for each product, prolonged
+ * ghost values 2^-54 of the largest of their 6 x 6 x 6 parent values.  Values that
+ * are not normal numbers, or near either end of the exponent range, are summed in
+ * FP64.
  *
  * Conventions shared by every call:
  *   - cell-centred grids; level l has spacing h_l = h0 / 2^l and cell index
@@ -341,12 +348,12 @@ sc_status sc_interpolate(sc_ctx* ctx, int npts, const double* xyz, int field, do
 /* Autotuner (no counterpart in the paper): on the context's largest level,
  * with CUDA events on its stream, time the Z4c derivative pass in its two-kernel
  * and (4th order) one-kernel forms and the Z4c stage kernel built for 2 and for
- * 3 warps per scheduler; keep the faster derivative form and stage build, rebuild
- * the tile lists and the coarse-step graphs.  (The wave stage and the two-kernel
- * derivative pass choose their tiles by box and level and have nothing to tune.)  The choice is cached for the process per
- * (system, box shapes of every level); a cached context skips the timing
- * (*ms_out = -1).  Overwrites only stage/scratch buffers that every coarse
- * step recomputes; call between sc_advance calls.  tile_out: 3 ints or NULL. */
+ * 3 warps per scheduler, over sample data; keep the faster derivative form and stage
+ * build, rebuild the tile lists and the coarse-step graphs.  (The wave stage and the
+ * two-kernel derivative pass choose their tiles by box and level and have nothing
+ * to tune.)  The choice is cached for the process per (system, order, box shapes of
+ * every level); a cached context skips the timing (*ms_out = -1).  Overwrites only
+ * stage/scratch buffers that every coarse step recomputes; call between sc_advance calls.  tile_out: 3 ints or NULL. */
 sc_status sc_autotune(sc_ctx* ctx, int* tile_out, double* ms_out);
 /* The tuning in effect (no counterpart in the paper): tile = 3 ints (tile
  * shape of the one-kernel derivative pass and the finiteness scan), deriv_form = 0 (Z4c derivative pass as two

@@ -15,8 +15,9 @@ namespace sc {
 // Prolongation sums.  Values are v * 2^e with |v| < 2^60.2 (59 bits at a node,
 // grown by less than 1.3 per axis: the weights' magnitudes sum to 10568 / 8192).
 // A position's six nodes are aligned to their largest exponent and the weights are
-// integers over 2^13, so a sum is exact to the last place of that alignment and
-// depends on the six values alone.  Nodes that hold an infinity, a NaN or a value
+// integers over 2^13, so a sum is exact to the last place of that alignment (2^-58
+// of the largest node, rounded down; three axes: 2^-54 of the largest of 216 nodes at
+// most) and depends on the six values alone.  Nodes that hold an infinity, a NaN or a value
 // near the ends of the exponent range carry kNodeFp64, which spreads to every
 // sum they enter; such a position is computed in FP64.
 constexpr int kNodeFp64 = 0x7fff;

@@ -14,7 +14,8 @@
 // its derivatives, all of the star for its Laplacian and the Kreiss-Oliger sum.  At
 // 4th order the weights multiply before the alignment cuts, or the weighted
 // values keep more bits, so that a sum's error is a few units of its smallest
-// weight: at most 2^-54 of its largest weighted term.  At 8th order the weights
+// weight: at most 2^-49 of the sum of its weighted values' magnitudes (8th order:
+// 2^-48; RMS errors are some 2^-53 of the largest value).  At 8th order the weights
 // are too far apart for that (1 to 8192), and sums whose lightly weighted outer
 // values are 2^3 to 2^5 times the inner ones are left to FP64, whose error
 // is relative to the weighted values (kExcess1 and so on; inside these limits the

@@ -15,9 +15,9 @@
 //      derivatives, evaluates the right-hand side, adds dissipation and
 //      performs the RK4 stage update.
 // FP64 is the scarce resource on this GPU (the FP64 pipe issues 1/64 of the
-// FP32 rate), so both passes work in integers (sc_fixed.cuh: the stencil sums;
-// sc_z4c_fixed.cuh: the tensor contractions), and the FP64 forms beside them
-// are for the cells whose values the integer forms do not take.
+// FP32 rate), so the stencil sums (sc_fixed.cuh) and the tensor sums that use
+// their operands many times (sc_z4c_point.cuh) are formed in integers; the FP64
+// forms beside them are for the cells whose values the integers do not take.
 #include "sc_device.cuh"
 #include "sc_z4c_point.cuh"
 
@@ -427,10 +427,10 @@ struct StageUpdate {
 // a row, 25% at 48), and the 152 SMs share the 125 runs of a 20^3 level.  BPS (a
 // choice of sc_autotune): 2 leaves 255 registers a thread, 3 has six blocks of 168
 // registers per SM.
-// Bound by the FP64 pipe, 70% of its rate with BPS 3 (of 11,800 instructions a cell
-// 567 are FP64, each 64 cycles of a scheduler's pipe), and by latency on small levels.  262,144
-// cells: 0.501 ms in FP64 throughout, 0.329 with BPS 3, 0.361 with 2; 110,592 cells:
-// 0.290, 0.150, 0.161; 8,000 cells: 0.041, 0.035, 0.035.  More of the sums in integers
+// Bound by the FP64 pipe, 72% of its rate with BPS 3 (of 11,793 instructions a cell
+// 564 are FP64, each 64 cycles of a scheduler's pipe), and by latency on small levels.
+// 262,144 cells: 0.501 ms in FP64 throughout, 0.329 with BPS 3, 0.361 with 2; 110,592
+// cells: 0.290, 0.150, 0.161; 8,000 cells: 0.041, 0.035, 0.035.  More of the sums in integers
 // (second derivatives contracted with gt^ij too: 512 FP64 instructions) ran in 0.349.
 template <int FORM, int BPS, class KT = FmaK>
 __global__ void __launch_bounds__(kRunCells, 2 * BPS)
