@@ -255,20 +255,37 @@ struct Z4cUnits {
   double pure, mh_pure;    // 48 or 560, and -1/2 of it
   double tp, tm;           // a third of the scales of second derivatives
 };
+// Every scale is formed in a pair of doubles and rounded once: their errors are the
+// same in every cell.  (Explicit FMAs, so that every host compiler gives the same values.)
+struct FxPair {
+  double h, l;
+};
+inline FxPair fx_pair_times(const FxPair& x, double k) {
+  const double h = x.h * k;
+  return FxPair{h, std::fma(x.l, k, std::fma(x.h, k, -h))};
+}
 inline Z4cUnits z4c_units(const DerivScales& ds, double h) {
   const double w = std::round(1.0 / (ds.s1 * h));  // 12 or 840
-  const long double u = 1.0L / (2.0L * w * h);     // (every scale is rounded once)
+  const FxPair d = fx_pair_times(FxPair{h, 0.0}, 2.0 * w);
+  FxPair u{1.0 / d.h, 0.0};
+  u.l = u.h * std::fma(-u.h, d.l, std::fma(-u.h, d.h, 1.0));
+  FxPair u2 = fx_pair_times(u, u.h);
+  u2.l = std::fma(u.h, u.l, u2.l);
+  auto third = [](const FxPair& x) {
+    const double q = x.h / 3.0;
+    return q + (std::fma(-q, 3.0, x.h) + x.l) / 3.0;
+  };
   Z4cUnits c;
-  c.u = (double)u;
-  c.iu = (double)(1.0L / u);
-  c.u2 = (double)(u * u);
+  c.u = u.h + u.l;
+  c.iu = d.h + d.l;
+  c.u2 = u2.h + u2.l;
   c.s1 = 2.0 * c.u;
   c.m2u = -2.0 * c.u;
   c.m2u2 = -2.0 * c.u2;
   c.pure = w == 12.0 ? 48.0 : 560.0;
   c.mh_pure = -0.5 * c.pure;
-  c.tp = (double)(u * u * c.pure / 3.0L);
-  c.tm = (double)(u * u * 4.0L / 3.0L);
+  c.tp = third(fx_pair_times(u2, c.pure));
+  c.tm = third(fx_pair_times(u2, 4.0));
   return c;
 }
 
