@@ -562,7 +562,7 @@ __device__ __forceinline__ void wave_stage_body(const StageArgs& a, const Tile* 
           else lap = fma(-43050.0, c[0], fma(8064.0, s[0], fma(-1008.0, s[1], fma(128.0, s[2], -9.0 * s[3]))));
         }
       }
-      const double kp = fmul(lap, a.ds.s2p, K);  // d_t Pi = Laplacian u, its sum over 12 h^2 or 5040 h^2
+      const double kp = fmul(lap, a.lap, K);  // d_t Pi = Laplacian u, its sum over 12 h^2 or 5040 h^2
       a.k[o] = ku;
       a.k[a.fs + o] = kp;
       if (a.form == kStageSingle) {

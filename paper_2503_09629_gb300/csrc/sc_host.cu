@@ -1195,7 +1195,8 @@ sc_status run_op(sc_ctx* c, const Op& o, cudaStream_t s) {
       a.sy = g.pitch;
       a.sz = g.pitch * g.ext[1];
       a.h = g.h;
-      a.ds = deriv_scales(c->order, g.h);
+      a.order = c->order;
+      a.lap = laplacian_scale(c->order, g.h);
       a.eta = L.eta;
       // graph form: one launch over the tiles of all boxes; per-box form: one per box
       const int nparts = c->exec_mode == SC_EXEC_PER_BOX ? (int)L.boxes.size() : 1;
@@ -1333,7 +1334,8 @@ void persistent_phases(sc_ctx* c, const std::vector<Op>& ops, std::vector<POp>& 
         p.a.sy = g.pitch;
         p.a.sz = g.pitch * g.ext[1];
         p.a.h = g.h;
-        p.a.ds = deriv_scales(c->order, g.h);
+        p.a.order = c->order;
+        p.a.lap = laplacian_scale(c->order, g.h);
         p.a.eta = L.eta;
         p.tiles = L.dtiles;
         p.ntiles = L.ndtiles;
@@ -1630,7 +1632,8 @@ StageArgs tuning_stage_args(const Level& L, int order) {
   a.sy = g.pitch;
   a.sz = g.pitch * g.ext[1];
   a.h = g.h;
-  a.ds = deriv_scales(order, g.h);
+  a.order = order;
+  a.lap = laplacian_scale(order, g.h);
   a.eta = L.eta;
   return a;
 }
@@ -2382,8 +2385,7 @@ sc_status sc_get_constraints(sc_ctx* c, int level, int box, double* dst) {
     CU(launch_z4c_derivs_split(Y, c->scratch, L.g.fs, sy, sz, L.dtiles + L.box_dtile_begin[box],
                                L.box_dtile_begin[box + 1] - L.box_dtile_begin[box], c->stream, c->order));
   }
-  CU(launch_z4c_constraints(Y, c->scratch, c->staging, L.g.fs, sy, sz, deriv_scales(c->order, L.g.h), L.g.h, ncell, blo,
-                            n, c->stream));
+  CU(launch_z4c_constraints(Y, c->scratch, c->staging, L.g.fs, sy, sz, c->order, L.g.h, ncell, blo, n, c->stream));
   CU(cudaMemcpyAsync(dst, c->staging, bytes, cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));
   if (dt) c->dfree(dt);  // the per-call tile list (the stream is idle)
@@ -2429,7 +2431,8 @@ sc_status sc_time_stage_kernels(sc_ctx* c, int level, int nrep, double* ms) {
   a.sy = g.pitch;
   a.sz = g.pitch * g.ext[1];
   a.h = g.h;
-  a.ds = deriv_scales(c->order, g.h);
+  a.order = c->order;
+  a.lap = laplacian_scale(c->order, g.h);
   a.eta = L.eta;
   cudaEvent_t e[3];
   for (auto& x : e) CU(cudaEventCreate(&x));

@@ -114,30 +114,9 @@ struct Weights {
   double restrict_w[kRN];
 };
 
-// Factors that turn the Z4c derivative pass's stored integer-weight stencil
-// sums into derivatives: first derivatives times s1, pure second derivatives
-// times s2p, mixed second derivatives times s2m (4th order: 1/(12h),
-// 1/(12h^2), 1/(144h^2); 8th order: 1/(840h), 1/(5040h^2), 1/(840h)^2).
-struct DerivScales {
-  double s1, s2p, s2m;  // first, pure second and mixed second derivative
-  double hs1, ts1, qs1;  // s1 / 2, s1 / 3 and s1 / 4
-  double hs2p, ts2m;    // s2p / 2 and 2 s2m
-};
-// The products are formed on the host so that the kernels take every factor
-// as a kernel-parameter operand (no register, no extra instruction).
-inline DerivScales deriv_scales(int order, double h) {
-  const double w1 = order == 8 ? 840.0 : 12.0, w2 = order == 8 ? 5040.0 : 12.0;
-  DerivScales d;
-  d.s1 = 1.0 / (w1 * h);
-  d.s2p = 1.0 / (w2 * h * h);
-  d.s2m = 1.0 / (w1 * h * w1 * h);
-  d.hs1 = 0.5 * d.s1;
-  d.ts1 = d.s1 / 3.0;
-  d.qs1 = 0.25 * d.s1;
-  d.hs2p = 0.5 * d.s2p;
-  d.ts2m = 2.0 * d.s2m;
-  return d;
-}
+// The factor that turns the wave's integer-weight Laplacian sum into the Laplacian:
+// 1/(12h^2) at 4th order, 1/(5040h^2) at 8th.
+inline double laplacian_scale(int order, double h) { return 1.0 / ((order == 8 ? 5040.0 : 12.0) * h * h); }
 
 // Arguments of one fused RK4 stage (right-hand side + stage update).
 struct StageArgs {
@@ -161,7 +140,8 @@ struct StageArgs {
   int sy, sz;        // strides of y and z in doubles
   double h;
   const double* eta; // Z4c: per-cell Gamma-driver damping eta(r), or null for the constant
-  DerivScales ds;    // scales of the derivative sums
+  int order;         // finite-difference order, 4 or 8
+  double lap;        // wave: laplacian_scale
 };
 
 // Additions, subtractions and scalings that do not fuse are written as fused
@@ -253,7 +233,7 @@ cudaError_t launch_z4c_stage(const StageArgs& a, const double* scratch, const Z4
 cudaError_t launch_radiative_stage(const StageArgs& a, const int32_t* cells, int ncells, int F,
                                    const Geom& g, int system, cudaStream_t s);
 cudaError_t launch_z4c_constraints(const double* Y, const double* scratch, double* out, long fs, int sy, int sz,
-                                   const DerivScales& ds, double h, long out_stride, const int* box_lo,
+                                   int order, double h, long out_stride, const int* box_lo,
                                    const int* box_n, cudaStream_t s);
 
 cudaError_t launch_periodic_copy(double* vec, long fs, int F, const int2* pairs, int npairs, cudaStream_t s);

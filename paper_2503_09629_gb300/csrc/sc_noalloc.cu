@@ -132,8 +132,7 @@ extern "C" sc_status sc_z4c_constraints_noalloc(const double* dev_state, double*
   e = sc::launch_z4c_derivs(dev_state, sym->scratch, fs, sy, sz, sym->tiles, (int)nt, s);
   if (e != cudaSuccess) return noalloc_fail(SC_ECUDA, "derivative kernel", e);
   const int lo[3] = {sc::kGhost, sc::kGhost, sc::kGhost};
-  e = sc::launch_z4c_constraints(dev_state, sym->scratch, dev_out, fs, sy, sz, sc::deriv_scales(4, h), h,
-                                 (long)n[0] * n[1] * n[2], lo, n, s);
+  e = sc::launch_z4c_constraints(dev_state, sym->scratch, dev_out, fs, sy, sz, 4, h, (long)n[0] * n[1] * n[2], lo, n, s);
   if (e != cudaSuccess) return noalloc_fail(SC_ECUDA, "constraint kernel", e);
   return SC_OK;
 }

@@ -8,7 +8,7 @@
 //      KO sum sum_d delta_d^6 u, and stores them in a scratch array indexed
 //      like the level array: scratch[q * fs + cell].  The stored values are
 //      the stencils' integer-weight sums, without their 1/h and 1/h^2
-//      factors (see DerivScales): a multiplication issues at the slower of
+//      factors (see Z4cUnits): a multiplication issues at the slower of
 //      the two FP64 rates, and the consumers fold the factors into FMA
 //      constants they evaluate anyway.
 //   2. z4c_stage_kernel: one thread per cell reads the 22 fields and their
@@ -564,7 +564,7 @@ namespace {
 template <int BPS>
 void launch_stage_bps(const StageArgs& a, const double* scratch, const Z4cParams& p, const CellRun* runs, int nruns,
                       int grid, cudaStream_t s, const FmaK& K, bool op_class) {
-  const Z4cUnits c = z4c_units(a.ds, a.h);
+  const Z4cUnits c = z4c_units(a.order, a.h);
   if (op_class)
     z4c_stage_kernel<kStageSingle, BPS, PlainK><<<grid, kRunCells, 0, s>>>(a, scratch, p, runs, nruns, c, PlainK{});
   else if (a.form == kStageRk4) z4c_stage_kernel<kStageRk4, BPS><<<grid, kRunCells, 0, s>>>(a, scratch, p, runs, nruns, c, K);
@@ -590,12 +590,13 @@ cudaError_t launch_z4c_stage(const StageArgs& a, const double* scratch, const Z4
 }
 
 cudaError_t launch_z4c_constraints(const double* Y, const double* scratch, double* out, long fs, int sy, int sz,
-                                   const DerivScales& ds, double h, long out_stride, const int* box_lo,
-                                   const int* box_n, cudaStream_t s) {
+                                   int order, double h, long out_stride, const int* box_lo, const int* box_n,
+                                   cudaStream_t s) {
   const long blocks = ((long)box_n[0] * box_n[1] * box_n[2] + kRunCells - 1) / kRunCells;
   const int grid = (int)(blocks < sm_count() * 16L ? blocks : sm_count() * 16L);
-  z4c_constraints_kernel<<<grid, kRunCells, 0, s>>>(Y, scratch, out, fs, sy, sz, z4c_units(ds, h), out_stride, box_lo[0], box_lo[1],
-                                                    box_lo[2], box_n[0], box_n[1], box_n[2], FmaK{1.0, -1.0, -0.0});
+  z4c_constraints_kernel<<<grid, kRunCells, 0, s>>>(Y, scratch, out, fs, sy, sz, z4c_units(order, h), out_stride,
+                                                    box_lo[0], box_lo[1], box_lo[2], box_n[0], box_n[1], box_n[2],
+                                                    FmaK{1.0, -1.0, -0.0});
   return cudaGetLastError();
 }
 

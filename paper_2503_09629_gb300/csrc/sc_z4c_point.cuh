@@ -264,8 +264,8 @@ inline FxPair fx_pair_times(const FxPair& x, double k) {
   const double h = x.h * k;
   return FxPair{h, std::fma(x.l, k, std::fma(x.h, k, -h))};
 }
-inline Z4cUnits z4c_units(const DerivScales& ds, double h) {
-  const double w = std::round(1.0 / (ds.s1 * h));  // 12 or 840
+inline Z4cUnits z4c_units(int order, double h) {
+  const double w = order == 8 ? 840.0 : 12.0;
   const FxPair d = fx_pair_times(FxPair{h, 0.0}, 2.0 * w);
   FxPair u{1.0 / d.h, 0.0};
   u.l = u.h * std::fma(-u.h, d.l, std::fma(-u.h, d.h, 1.0));
@@ -282,7 +282,7 @@ inline Z4cUnits z4c_units(const DerivScales& ds, double h) {
   c.s1 = 2.0 * c.u;
   c.m2u = -2.0 * c.u;
   c.m2u2 = -2.0 * c.u2;
-  c.pure = w == 12.0 ? 48.0 : 560.0;
+  c.pure = order == 8 ? 560.0 : 48.0;
   c.mh_pure = -0.5 * c.pure;
   c.tp = third(fx_pair_times(u2, c.pure));
   c.tm = third(fx_pair_times(u2, 4.0));
